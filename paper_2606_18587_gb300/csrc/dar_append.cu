@@ -47,33 +47,13 @@ struct BulkArgs {
     int ones_col[2];  // first of 16 padding columns set to 1 (-1: all padding is 0)
 };
 
-template <typename T, int DD>
-__global__ void __launch_bounds__(threads_bulk<T, DD>()) down_project_kernel(BulkArgs a)
+// The chains of RPT staged rows (threadIdx.x + k * NT) of a tile of 64-wide
+// rows whose 16-byte chunk c sits at chunk c ^ (r & 7); Ws = W[t][c].
+template <typename T, int DD, int RPT, int NT>
+__device__ __forceinline__ void project_rows(const unsigned char *rows, const float *Ws, float (&acc)[RPT][DD])
 {
-    constexpr int R = rows_bulk<T>();
-    constexpr int RPT = rows_per_thread<DD>();
-    constexpr int NT = threads_bulk<T, DD>();
     constexpr int E = Granule<T>::kElems;
-    constexpr int CPR = kHeadDim / E;  // 16-byte chunks per row (8 for bf16, 16 for fp32)
-    __shared__ __align__(16) unsigned char rows[kStageBytesBulk];
-    __shared__ __align__(16) float Ws[kHeadDim * DD];
-    const bool z = blockIdx.z != 0;  // (selects, not indexes: the arguments stay in parameter space)
-    const T *x = static_cast<const T *>(z ? a.x[1] : a.x[0]);
-    const int bg = blockIdx.y, g = bg % a.Hkv;
-    const int j0 = blockIdx.x * R;
-    const int nr = min(R, a.n - j0);
-    const float *W = (z ? a.W[1] : a.W[0]) + (size_t)g * kHeadDim * DD;
-    for (int i = threadIdx.x; i < kHeadDim * DD / 4; i += NT)
-        reinterpret_cast<float4 *>(Ws)[i] = __ldg(reinterpret_cast<const float4 *>(W) + i);
-    const uint4 *src = reinterpret_cast<const uint4 *>(x + ((size_t)bg * a.n + j0) * kHeadDim);
-    for (int i = threadIdx.x; i < nr * CPR; i += NT) {
-        const int r = i / CPR, c = i % CPR;
-        reinterpret_cast<uint4 *>(rows)[r * CPR + (c ^ (r & 7))] = ld_stream_v4(src + i);
-    }
-    __syncthreads();
-    // this thread's rows: threadIdx.x + k * NT, k < RPT (rows past nr compute on
-    // stale staging bytes and are not stored)
-    float acc[RPT][DD];
+    constexpr int CPR = kHeadDim / E;
 #pragma unroll
     for (int k = 0; k < RPT; ++k)
 #pragma unroll
@@ -102,6 +82,61 @@ __global__ void __launch_bounds__(threads_bulk<T, DD>()) down_project_kernel(Bul
             }
         }
     }
+}
+
+// DD fp32 values rounded once to T and stored as 16-byte words (the row is 16-byte aligned).
+template <typename T, int DD>
+__device__ __forceinline__ void store_row(T *o, const float (&x)[DD])
+{
+    constexpr int OE = 16 / sizeof(T);
+#pragma unroll
+    for (int c = 0; c < DD; c += OE) {
+        uint32_t u[4];
+        if constexpr (sizeof(T) == 2) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                __nv_bfloat162 v = __floats2bfloat162_rn(x[c + 2 * i], x[c + 2 * i + 1]);
+                u[i] = *reinterpret_cast<uint32_t *>(&v);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                u[i] = __float_as_uint(x[c + i]);
+        }
+        *reinterpret_cast<uint4 *>(o + c) = make_uint4(u[0], u[1], u[2], u[3]);
+    }
+}
+
+template <typename T, int DD>
+__global__ void __launch_bounds__(threads_bulk<T, DD>()) down_project_kernel(BulkArgs a)
+{
+    constexpr int R = rows_bulk<T>();
+    constexpr int RPT = rows_per_thread<DD>();
+    constexpr int NT = threads_bulk<T, DD>();
+    constexpr int E = Granule<T>::kElems;
+    constexpr int CPR = kHeadDim / E;  // 16-byte chunks per row (8 for bf16, 16 for fp32)
+    __shared__ __align__(16) unsigned char rows[kStageBytesBulk];
+    __shared__ __align__(16) float Ws[kHeadDim * DD];
+    const bool z = blockIdx.z != 0;  // (selects, not indexes: the arguments stay in parameter space)
+    const T *x = static_cast<const T *>(z ? a.x[1] : a.x[0]);
+    const int bg = blockIdx.y, g = bg % a.Hkv;
+    const int j0 = blockIdx.x * R;
+    const int nr = min(R, a.n - j0);
+    const float *W = (z ? a.W[1] : a.W[0]) + (size_t)g * kHeadDim * DD;
+    for (int i = threadIdx.x; i < kHeadDim * DD / 4; i += NT)
+        reinterpret_cast<float4 *>(Ws)[i] = __ldg(reinterpret_cast<const float4 *>(W) + i);
+    const uint4 *src = reinterpret_cast<const uint4 *>(x + ((size_t)bg * a.n + j0) * kHeadDim);
+    const uint32_t rows_s = sm100::smem_u32(rows);
+    for (int i = threadIdx.x; i < nr * CPR; i += NT) {
+        const int r = i / CPR, c = i % CPR;
+        sm100::cp_async16(rows_s + (r * CPR + (c ^ (r & 7))) * 16, src + i);
+    }
+    sm100::cp_async_wait_all();
+    __syncthreads();
+    // this thread's rows: threadIdx.x + k * NT, k < RPT (rows past nr compute on
+    // stale staging bytes and are not stored)
+    float acc[RPT][DD];
+    project_rows<T, DD, RPT, NT>(rows, Ws, acc);
     const int ostride = z ? a.ostride[1] : a.ostride[0];
     const int ones_col = z ? a.ones_col[1] : a.ones_col[0];
 #pragma unroll
@@ -111,23 +146,7 @@ __global__ void __launch_bounds__(threads_bulk<T, DD>()) down_project_kernel(Bul
             continue;
         T *o = static_cast<T *>(z ? a.out[1] : a.out[0]) + ((size_t)bg * a.n + j0 + r) * ostride;
         if (ostride == DD && (DD * sizeof(T)) % 16 == 0) {
-            constexpr int OE = 16 / sizeof(T);
-#pragma unroll
-            for (int c = 0; c < DD; c += OE) {
-                uint32_t u[4];
-                if constexpr (sizeof(T) == 2) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        __nv_bfloat162 v = __floats2bfloat162_rn(acc[k][c + 2 * i], acc[k][c + 2 * i + 1]);
-                        u[i] = *reinterpret_cast<uint32_t *>(&v);
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        u[i] = __float_as_uint(acc[k][c + i]);
-                }
-                *reinterpret_cast<uint4 *>(o + c) = make_uint4(u[0], u[1], u[2], u[3]);
-            }
+            store_row<T, DD>(o, acc[k]);
         } else if ((ostride * sizeof(T)) % 16 == 0 && ostride <= kHeadDim) {
             // padded rows (values, then zeros or a block of 16 ones), 16 bytes at a time
             constexpr int OE = 16 / sizeof(T);
@@ -191,6 +210,17 @@ __host__ __device__ inline int app_rows(int Hkv)
     return r < 1 ? 1 : r > kAppRows ? kAppRows : r;
 }
 
+// Whether sequence lengths L and L + nb are ones an append can take (DAR_OK, or the status to report).
+__device__ __forceinline__ int append_error(int L, int nb, const AppendArgs &a)
+{
+    const long long Lnew = (long long)L + nb;
+    if (L < 0 || nb < 0 || nb > a.n)
+        return DAR_ERR_INVALID_ARG;
+    if (Lnew - a.w > (long long)a.maxp * kPage || Lnew > 0x7fffffffLL)
+        return DAR_ERR_CAPACITY;
+    return DAR_OK;
+}
+
 template <typename T, int DD>
 __global__ void __launch_bounds__(kAppThreads) cache_append_kernel(AppendArgs a)
 {
@@ -244,17 +274,10 @@ __global__ void __launch_bounds__(kAppThreads) cache_append_kernel(AppendArgs a)
         pre = *reinterpret_cast<const uint4 *>(new_granule(tid, n - pre_rows));
     __syncthreads();
     if (tid == 0) {
-        const int L = s_L, nb = s_nb;
-        const long long Lnew = (long long)L + nb;
-        int ok = 1;
-        if (L < 0 || nb < 0 || nb > n) {
-            report(a.status, DAR_ERR_INVALID_ARG);
-            ok = 0;
-        } else if (Lnew - w > (long long)a.maxp * kPage || Lnew > 0x7fffffffLL) {
-            report(a.status, DAR_ERR_CAPACITY);
-            ok = 0;
-        }
-        s_ok = ok;
+        const int e = append_error(s_L, s_nb, a);
+        if (e != DAR_OK)
+            report(a.status, e);
+        s_ok = e == DAR_OK;
     }
     __syncthreads();
     if (!s_ok || s_nb == 0)
@@ -329,6 +352,101 @@ __global__ void __launch_bounds__(kAppThreads) cache_append_kernel(AppendArgs a)
         a.seq_lens[b] = Lnew;
 }
 
+// ------------------------------------------------------- cache append, bulk
+//
+// The same append for calls with many tokens per sequence (a prompt or a chunk
+// of one), spread over the chip: the kernel above runs one CTA per sequence,
+// eight rows at a time, and leaves most SMs idle (32 prompts of 1000 to 4096
+// tokens, 12 KV heads, d_down 16: 2740 us).  Here a CTA takes R consecutive new
+// tokens of one (sequence, KV head, keys or values).  New token j (position
+// L + j) pushes position m = L + j - w out of the window; the CTA that holds j
+// projects that row -- from ring slot m % w, or from the new rows when m >= L
+// -- into its page, and then overwrites ring slot (L + j) % w = m % w (j < w)
+// with the last new token that lands there.  A ring slot therefore has one
+// reader and one writer, in one CTA, and no order between CTAs is needed.  The
+// length is advanced by a second kernel once every CTA has read it.  The FMA
+// chains bound it: the same prompts take 146 us (2.0 G FMA, 50 us at the
+// chip's fp32 rate; 329 MB, 49 us at the copy rate).
+template <typename T, int DD, int RPT, int NT>
+__global__ void __launch_bounds__(NT) append_bulk_kernel(AppendArgs a, int tiles)
+{
+    constexpr int R = RPT * NT;
+    constexpr int E = Granule<T>::kElems;
+    constexpr int CPR = kHeadDim / E;
+    __shared__ __align__(16) unsigned char rows[R * kHeadDim * sizeof(T)];
+    __shared__ __align__(16) float Ws[kHeadDim * DD];
+    const int tid = threadIdx.x, kv = blockIdx.y;
+    const int bg = blockIdx.x / tiles, j0 = (blockIdx.x % tiles) * R;
+    const int b = bg / a.Hkv, g = bg % a.Hkv;
+    const int n = a.n, w = a.w;
+    const int L = a.seq_lens[b], nb = a.n_per_seq ? a.n_per_seq[b] : n;
+    if (append_error(L, nb, a) != DAR_OK || j0 >= nb)
+        return;
+    const T *xnew = static_cast<const T *>(kv ? a.v_new : a.k_new) + (size_t)bg * n * kHeadDim;
+    T *ring = static_cast<T *>(kv ? a.win_v : a.win_k) + (size_t)bg * w * kHeadDim;
+    const int nr = min(R, nb - j0);
+    const bool any = (long long)L + j0 + nr > w;  // the tile's last token pushes a position out
+    if (any) {
+        const uint32_t rows_s = sm100::smem_u32(rows);
+        for (int i = tid; i < nr * CPR; i += NT) {
+            const int r = i / CPR, c = i % CPR, m = L + j0 + r - w;
+            if (m >= 0) {
+                const T *src = m < L ? ring + (size_t)(m % w) * kHeadDim : xnew + (size_t)(m - L) * kHeadDim;
+                sm100::cp_async16(rows_s + (r * CPR + (c ^ (r & 7))) * 16, src + c * E);
+            }
+        }
+        const float *W = (kv ? a.Dv : a.Dk) + (size_t)g * kHeadDim * DD;
+        for (int i = tid; i < kHeadDim * DD / 4; i += NT)
+            reinterpret_cast<float4 *>(Ws)[i] = __ldg(reinterpret_cast<const float4 *>(W) + i);
+        int id[RPT];  // page of each of this thread's rows (-1: not a row that leaves, or no page)
+#pragma unroll
+        for (int k = 0; k < RPT; ++k) {
+            const int r = tid + k * NT, m = L + j0 + r - w;
+            id[k] = -1;
+            if (r < nr && m >= 0) {
+                const int e = a.block_table[(size_t)b * a.maxp + m / kPage];
+                if (e >= 0 && e < a.num_pages)
+                    id[k] = e;
+                else
+                    report(a.status, DAR_ERR_CAPACITY);
+            }
+        }
+        sm100::cp_async_wait_all();
+        __syncthreads();  // every ring row this CTA reads is in shared memory
+        float acc[RPT][DD];
+        project_rows<T, DD, RPT, NT>(rows, Ws, acc);
+        T *pool = static_cast<T *>(kv ? a.pool_vd : a.pool_kd);
+#pragma unroll
+        for (int k = 0; k < RPT; ++k) {
+            const int m = L + j0 + tid + k * NT - w;
+            if (id[k] >= 0)
+                store_row<T, DD>(pool + (((size_t)id[k] * a.Hkv + g) * kPage + m % kPage) * DD, acc[k]);
+        }
+    }
+    // ring slots (L + j) % w, j < min(nb, w): the last new token of each
+    const int slots = min(nb, w) - j0;
+    for (int i = tid; i < min(slots, R) * CPR; i += NT) {
+        const int c = i % CPR, j = j0 + i / CPR, last = j + (nb - 1 - j) / w * w;
+        *reinterpret_cast<uint4 *>(ring + (size_t)((L + j) % w) * kHeadDim + c * E) =
+            *reinterpret_cast<const uint4 *>(xnew + (size_t)last * kHeadDim + c * E);
+    }
+}
+
+// Advances the lengths (and reports refused sequences) after append_bulk_kernel.
+__global__ void append_lens_kernel(AppendArgs a)
+{
+    sm100::grid_dep_wait();  // every CTA of the append has read the lengths
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= a.B)
+        return;
+    const int L = a.seq_lens[b], nb = a.n_per_seq ? a.n_per_seq[b] : a.n;
+    const int e = append_error(L, nb, a);
+    if (e != DAR_OK)
+        report(a.status, e);
+    else
+        a.seq_lens[b] = L + nb;
+}
+
 // ----------------------------------------------------------------- launchers
 
 template <typename T>
@@ -394,10 +512,76 @@ static cudaError_t cache_append_t(int dd, const AppendArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
+template <typename T, int DD, int RPT, int NT>
+static cudaError_t append_bulk_launch(const AppendArgs &a, cudaStream_t s)
+{
+    const int tiles = (a.n + RPT * NT - 1) / (RPT * NT);
+    append_bulk_kernel<T, DD, RPT, NT><<<dim3((unsigned)(a.B * a.Hkv * tiles), 2), NT, 0, s>>>(a, tiles);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess)
+        return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((a.B + 127) / 128);
+    cfg.blockDim = dim3(128);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, append_lens_kernel, a);
+}
+
+// Big tiles (several rows per thread, so that one read of W feeds them all)
+// once they fill the chip a few times over; otherwise one row per thread.
+constexpr int kBulkSmallThreads = 64;
+constexpr long long kBulkBigCtas = 152 * 6 * 2;
+
+template <typename T, int DD>
+static cudaError_t append_bulk(const AppendArgs &a, cudaStream_t s)
+{
+    constexpr int RPT = rows_per_thread<DD>(), NT = threads_bulk<T, DD>();
+    const long long big = ((long long)a.n + RPT * NT - 1) / (RPT * NT) * a.B * a.Hkv * 2;
+    if (big >= kBulkBigCtas)
+        return append_bulk_launch<T, DD, RPT, NT>(a, s);
+    return append_bulk_launch<T, DD, 1, kBulkSmallThreads>(a, s);
+}
+
+template <typename T>
+static cudaError_t append_bulk_t(int dd, const AppendArgs &a, cudaStream_t s)
+{
+    switch (dd) {
+    case 8: return append_bulk<T, 8>(a, s);
+    case 16: return append_bulk<T, 16>(a, s);
+    case 32: return append_bulk<T, 32>(a, s);
+    case 64: return append_bulk<T, 64>(a, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+// More tokens than one round of the one-CTA-per-sequence kernel: the bulk
+// kernel.  Measured (d_down 16, w 128, context 500), one CTA per sequence / bulk:
+//   n = 8:  B 1, 8 heads 7.8 / 6.2 us; B 32, 12 heads 9.6 / 8.0; B 64, 8 heads 8.2 / 9.3
+//   n = 9:               9.2 / 6.6;                  11.3 / 8.4;                 9.4 / 9.7
+//   n = 64:             37.5 / 8.4;                  48.5 / 10.7;               37.7 / 11.9
+// and at n = 1 the bulk kernel's second launch costs 2 to 4 us.  (A cache with so many heads that not one row of them fits the
+// staging area stays with the kernel that refuses it; so does a call whose CTAs
+// a grid cannot count.)
+constexpr int kBulkMinTokens = kAppRows + 1;
+
+static bool use_bulk(dar_dtype dt, const AppendArgs &a)
+{
+    const long long row = 2ll * a.Hkv * kHeadDim * (dt == DAR_F32 ? 4 : 2);
+    const long long tiles = ((long long)a.n + kBulkSmallThreads - 1) / kBulkSmallThreads;
+    return a.n >= kBulkMinTokens && row <= kAppStageBytes && tiles * a.B * a.Hkv <= 0x7fffffffLL;
+}
+
 cudaError_t launch_cache_append(dar_dtype dt, int dd, const AppendArgs &a, cudaStream_t s)
 {
     if (a.B == 0)
         return cudaSuccess;
+    if (use_bulk(dt, a))
+        return dt == DAR_F32 ? append_bulk_t<float>(dd, a, s) : append_bulk_t<bf16>(dd, a, s);
     return dt == DAR_F32 ? cache_append_t<float>(dd, a, s) : cache_append_t<bf16>(dd, a, s);
 }
 

@@ -899,12 +899,16 @@ static cudaError_t launch_dp(const PrefillArgs &a, cudaStream_t s)
 //    global to some chunk query (< L0 + n - w): copied from its page when it
 //    migrated before this call (< L0 - w), else Eq. 1 of its full-d row with
 //    the same fp32 chain as the cache append; zero otherwise.
-// grid (B, Hkv), 256 threads.  Block (b, 0) records L0 in pos0[b].
+// grid (B, Hkv, slices), 256 threads: the rows of a (sequence, KV head) are
+// dealt out over the slices (one block per pair left 120 of the 152 SMs idle
+// on a 4-sequence, 8-head chunk of 512 tokens).  Block (b, 0, 0) records L0 in
+// pos0[b].
 template <int DD>
 __global__ void __launch_bounds__(256) chunk_gather_kernel(ChunkArgs c)
 {
     const AppendArgs &ap = c.app;
-    const int b = blockIdx.x, g = blockIdx.y, tid = threadIdx.x;
+    const int b = blockIdx.x, g = blockIdx.y;
+    const int tid = blockIdx.z * 256 + threadIdx.x, step = gridDim.z * 256;
     const int w = ap.w, n = ap.n, Hkv = ap.Hkv;
     const int NW = c.pf.NW, NT = c.pf.NT;
     int L0 = __ldcg(ap.seq_lens + b);
@@ -933,7 +937,7 @@ __global__ void __launch_bounds__(256) chunk_gather_kernel(ChunkArgs c)
     // ---- window rows, 16 bytes at a time
     uint4 *kw = reinterpret_cast<uint4 *>(static_cast<bf16 *>(c.kw) + bg * NW * 64);
     uint4 *vw = reinterpret_cast<uint4 *>(static_cast<bf16 *>(c.vw) + bg * NW * 64);
-    for (int i = tid; i < NW * 8; i += blockDim.x) {
+    for (int i = tid; i < NW * 8; i += step) {
         const int p = kb0 + i / 8, ch = i % 8;
         uint4 k4 = make_uint4(0u, 0u, 0u, 0u), v4 = k4;
         if (p >= loc_lo && p < L0 + n) {
@@ -948,7 +952,7 @@ __global__ void __launch_bounds__(256) chunk_gather_kernel(ChunkArgs c)
     bf16 *vdt = static_cast<bf16 *>(c.vdt) + bg * NT * DD;
     const bf16 *pk = static_cast<const bf16 *>(ap.pool_kd);
     const bf16 *pv = static_cast<const bf16 *>(ap.pool_vd);
-    for (int i = tid; i < NT * DD; i += blockDim.x) {
+    for (int i = tid; i < NT * DD; i += step) {
         const int r = i / DD, col = i % DD, p = kt0 + r;
         bf16 kx = __float2bfloat16_rn(0.f), vx = kx;
         if (p < L0 - w) {  // migrated before this call: its page
@@ -980,7 +984,8 @@ template <int DP>
 static cudaError_t launch_chunk_dp(const ChunkArgs &c, cudaStream_t s)
 {
     const PrefillArgs &a = c.pf;
-    chunk_gather_kernel<DP><<<dim3(a.B, a.Hkv), 256, 0, s>>>(c);
+    const int slices = min(64, (max(a.NT * DP, a.NW * 8) + 255) / 256);
+    chunk_gather_kernel<DP><<<dim3(a.B, a.Hkv, slices), 256, 0, s>>>(c);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return e;

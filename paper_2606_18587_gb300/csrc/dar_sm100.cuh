@@ -104,6 +104,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity, volati
     return false;
 }
 
+// ------------------------------------------------------------------ cp.async
+
+// One asynchronous 16-byte copy to shared memory (both addresses 16-byte aligned).
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+// Every cp.async of this thread has landed.
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // ------------------------------------------------------------------ TMA
 
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned bytes, uint64_t *bar)
