@@ -6,36 +6,21 @@
 // token's cached vector is bit-identical whichever kernel produced it.
 #include "dar_common.cuh"
 #include "dar_launch.h"
+#include "dar_project.cuh"
 #include "dar_sm100.cuh"
 
 namespace dar {
 
 // ---------------------------------------------------------------- bulk Eq. 1
 //
-// A block stages kStageBytesBulk of contiguous token rows in shared memory
-// with coalesced 16-byte loads (chunk c of row r stored at chunk c ^ (r & 7),
-// so a warp reading one chunk of 32 different rows touches every bank group
-// once); then each thread runs the chains of RPT rows at once, so that every
-// W[t][c] read from shared memory feeds RPT rows.  Two chains advance per
-// instruction (fma.rn.f32x2: outputs c and c + 1 share x_t); each element is
-// still the exact fp32 chain acc = fma(x_t, W[t][c], acc), t = 0..63.
+// A block takes a tile of contiguous token rows (dar_project.cuh); two chains
+// advance per instruction (fma.rn.f32x2: outputs c and c + 1 share x_t) and
+// each element is still the exact fp32 chain acc = fma(x_t, W[t][c], acc).
 // blockIdx.z selects the tensor: 0 = (x0, W0, out0), 1 = (x1, W1, out1).
-constexpr int kStageBytesBulk = 32 << 10;
-
-template <typename T>
-__host__ __device__ constexpr int rows_bulk()
-{
-    return kStageBytesBulk / (kHeadDim * (int)sizeof(T));
-}
-template <int DD>
-__host__ __device__ constexpr int rows_per_thread()
-{
-    return DD <= 16 ? 4 : DD == 32 ? 2 : 1;
-}
 template <typename T, int DD>
 __host__ __device__ constexpr int threads_bulk()
 {
-    return rows_bulk<T>() / rows_per_thread<DD>();
+    return rows_bulk<T>() / rows_per_thread<DD>() * slices<DD>();
 }
 
 struct BulkArgs {
@@ -47,74 +32,11 @@ struct BulkArgs {
     int ones_col[2];  // first of 16 padding columns set to 1 (-1: all padding is 0)
 };
 
-// The chains of RPT staged rows (threadIdx.x + k * NT) of a tile of 64-wide
-// rows whose 16-byte chunk c sits at chunk c ^ (r & 7); Ws = W[t][c].
-template <typename T, int DD, int RPT, int NT>
-__device__ __forceinline__ void project_rows(const unsigned char *rows, const float *Ws, float (&acc)[RPT][DD])
-{
-    constexpr int E = Granule<T>::kElems;
-    constexpr int CPR = kHeadDim / E;
-#pragma unroll
-    for (int k = 0; k < RPT; ++k)
-#pragma unroll
-        for (int c = 0; c < DD; ++c)
-            acc[k][c] = 0.0f;
-#pragma unroll 1
-    for (int q = 0; q < CPR; ++q) {
-        float xf[RPT][E];
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-            const int r = threadIdx.x + k * NT;
-            unpack(reinterpret_cast<const uint4 *>(rows)[r * CPR + (q ^ (r & 7))], xf[k], T());
-        }
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int t = q * E + e;
-#pragma unroll
-            for (int c = 0; c < DD; c += 4) {
-                const float4 w4 = *reinterpret_cast<const float4 *>(Ws + t * DD + c);
-#pragma unroll
-                for (int k = 0; k < RPT; ++k) {
-                    sm100::ffma2(acc[k][c], acc[k][c + 1], xf[k][e], xf[k][e], w4.x, w4.y, acc[k][c], acc[k][c + 1]);
-                    sm100::ffma2(acc[k][c + 2], acc[k][c + 3], xf[k][e], xf[k][e], w4.z, w4.w, acc[k][c + 2],
-                                 acc[k][c + 3]);
-                }
-            }
-        }
-    }
-}
-
-// DD fp32 values rounded once to T and stored as 16-byte words (the row is 16-byte aligned).
-template <typename T, int DD>
-__device__ __forceinline__ void store_row(T *o, const float (&x)[DD])
-{
-    constexpr int OE = 16 / sizeof(T);
-#pragma unroll
-    for (int c = 0; c < DD; c += OE) {
-        uint32_t u[4];
-        if constexpr (sizeof(T) == 2) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                __nv_bfloat162 v = __floats2bfloat162_rn(x[c + 2 * i], x[c + 2 * i + 1]);
-                u[i] = *reinterpret_cast<uint32_t *>(&v);
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                u[i] = __float_as_uint(x[c + i]);
-        }
-        *reinterpret_cast<uint4 *>(o + c) = make_uint4(u[0], u[1], u[2], u[3]);
-    }
-}
-
 template <typename T, int DD>
 __global__ void __launch_bounds__(threads_bulk<T, DD>()) down_project_kernel(BulkArgs a)
 {
-    constexpr int R = rows_bulk<T>();
-    constexpr int RPT = rows_per_thread<DD>();
-    constexpr int NT = threads_bulk<T, DD>();
-    constexpr int E = Granule<T>::kElems;
-    constexpr int CPR = kHeadDim / E;  // 16-byte chunks per row (8 for bf16, 16 for fp32)
+    constexpr int R = rows_bulk<T>(), RPT = rows_per_thread<DD>(), NT = threads_bulk<T, DD>(), NR = R / RPT;
+    constexpr int CW = cols_per_thread<DD>();
     __shared__ __align__(16) unsigned char rows[kStageBytesBulk];
     __shared__ __align__(16) float Ws[kHeadDim * DD];
     const bool z = blockIdx.z != 0;  // (selects, not indexes: the arguments stay in parameter space)
@@ -122,65 +44,35 @@ __global__ void __launch_bounds__(threads_bulk<T, DD>()) down_project_kernel(Bul
     const int bg = blockIdx.y, g = bg % a.Hkv;
     const int j0 = blockIdx.x * R;
     const int nr = min(R, a.n - j0);
+    stage_tile(rows, x + ((size_t)bg * a.n + j0) * kHeadDim, nr, threadIdx.x, NT);
     const float *W = (z ? a.W[1] : a.W[0]) + (size_t)g * kHeadDim * DD;
     for (int i = threadIdx.x; i < kHeadDim * DD / 4; i += NT)
         reinterpret_cast<float4 *>(Ws)[i] = __ldg(reinterpret_cast<const float4 *>(W) + i);
-    const uint4 *src = reinterpret_cast<const uint4 *>(x + ((size_t)bg * a.n + j0) * kHeadDim);
-    const uint32_t rows_s = sm100::smem_u32(rows);
-    for (int i = threadIdx.x; i < nr * CPR; i += NT) {
-        const int r = i / CPR, c = i % CPR;
-        sm100::cp_async16(rows_s + (r * CPR + (c ^ (r & 7))) * 16, src + i);
-    }
     sm100::cp_async_wait_all();
     __syncthreads();
-    // this thread's rows: threadIdx.x + k * NT, k < RPT (rows past nr compute on
-    // stale staging bytes and are not stored)
-    float acc[RPT][DD];
-    project_rows<T, DD, RPT, NT>(rows, Ws, acc);
+    // this thread's rows: r0 + k * NR, columns c0 .. c0 + CW - 1 (rows past nr
+    // compute on stale staging bytes and are not stored)
+    const int r0 = threadIdx.x % NR, c0 = slices<DD>() > 1 ? (int)threadIdx.x / NR * CW : 0;
+    float acc[rows_per_thread<DD>()][CW];
+    project_rows<T, DD, CW, rows_per_thread<DD>()>(rows, Ws + c0, r0, NR, acc);
     const int ostride = z ? a.ostride[1] : a.ostride[0];
     const int ones_col = z ? a.ones_col[1] : a.ones_col[0];
 #pragma unroll
-    for (int k = 0; k < RPT; ++k) {
-        const int r = threadIdx.x + k * NT;
+    for (int k = 0; k < rows_per_thread<DD>(); ++k) {
+        const int r = r0 + k * NR;
         if (r >= nr)
             continue;
         T *o = static_cast<T *>(z ? a.out[1] : a.out[0]) + ((size_t)bg * a.n + j0 + r) * ostride;
-        if (ostride == DD && (DD * sizeof(T)) % 16 == 0) {
-            store_row<T, DD>(o, acc[k]);
-        } else if ((ostride * sizeof(T)) % 16 == 0 && ostride <= kHeadDim) {
-            // padded rows (values, then zeros or a block of 16 ones), 16 bytes at a time
+        store_row<T, CW>(o + c0, acc[k]);
+        if (ostride > DD && c0 == 0) {  // padding after the values: zeros, or a block of 16 ones
             constexpr int OE = 16 / sizeof(T);
-#pragma unroll
-            for (int c0 = 0; c0 < kHeadDim; c0 += OE) {
-                if (c0 >= ostride)
-                    break;
+            for (int c = DD; c < ostride; c += OE) {
                 float v[OE];
 #pragma unroll
-                for (int e = 0; e < OE; ++e) {
-                    const int c = c0 + e;
-                    v[e] = c < DD ? acc[k][c < DD ? c : 0]
-                                  : (ones_col >= 0 && c >= ones_col && c < ones_col + 16 ? 1.f : 0.f);
-                }
-                uint32_t u[4];
-                if constexpr (sizeof(T) == 2) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        __nv_bfloat162 b2 = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-                        u[i] = *reinterpret_cast<uint32_t *>(&b2);
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        u[i] = __float_as_uint(v[i]);
-                }
-                *reinterpret_cast<uint4 *>(o + c0) = make_uint4(u[0], u[1], u[2], u[3]);
+                for (int e = 0; e < OE; ++e)
+                    v[e] = ones_col >= 0 && c + e >= ones_col && c + e < ones_col + 16 ? 1.f : 0.f;
+                store_row<T, OE>(o + c, v);
             }
-        } else {
-#pragma unroll
-            for (int c = 0; c < DD; ++c)
-                o[c] = from_f32<T>(acc[k][c]);
-            for (int c = DD; c < ostride; ++c)
-                o[c] = from_f32<T>(c >= ones_col && c < ones_col + 16 && ones_col >= 0 ? 1.f : 0.f);
         }
     }
 }
@@ -367,10 +259,11 @@ __global__ void __launch_bounds__(kAppThreads) cache_append_kernel(AppendArgs a)
 // length is advanced by a second kernel once every CTA has read it.  The FMA
 // chains bound it: the same prompts take 146 us (2.0 G FMA, 50 us at the
 // chip's fp32 rate; 329 MB, 49 us at the copy rate).
-template <typename T, int DD, int RPT, int NT>
-__global__ void __launch_bounds__(NT) append_bulk_kernel(AppendArgs a, int tiles)
+template <typename T, int DD, int RPT, int NR>
+__global__ void __launch_bounds__(NR *slices<DD>()) append_bulk_kernel(AppendArgs a, int tiles)
 {
-    constexpr int R = RPT * NT;
+    constexpr int R = RPT * NR, NT = NR * slices<DD>();
+    constexpr int CW = cols_per_thread<DD>();
     constexpr int E = Granule<T>::kElems;
     constexpr int CPR = kHeadDim / E;
     __shared__ __align__(16) unsigned char rows[R * kHeadDim * sizeof(T)];
@@ -398,10 +291,11 @@ __global__ void __launch_bounds__(NT) append_bulk_kernel(AppendArgs a, int tiles
         const float *W = (kv ? a.Dv : a.Dk) + (size_t)g * kHeadDim * DD;
         for (int i = tid; i < kHeadDim * DD / 4; i += NT)
             reinterpret_cast<float4 *>(Ws)[i] = __ldg(reinterpret_cast<const float4 *>(W) + i);
+        const int r0 = tid % NR, c0 = slices<DD>() > 1 ? tid / NR * CW : 0;  // this thread's rows r0 + k * NR and columns
         int id[RPT];  // page of each of this thread's rows (-1: not a row that leaves, or no page)
 #pragma unroll
         for (int k = 0; k < RPT; ++k) {
-            const int r = tid + k * NT, m = L + j0 + r - w;
+            const int r = r0 + k * NR, m = L + j0 + r - w;
             id[k] = -1;
             if (r < nr && m >= 0) {
                 const int e = a.block_table[(size_t)b * a.maxp + m / kPage];
@@ -413,14 +307,14 @@ __global__ void __launch_bounds__(NT) append_bulk_kernel(AppendArgs a, int tiles
         }
         sm100::cp_async_wait_all();
         __syncthreads();  // every ring row this CTA reads is in shared memory
-        float acc[RPT][DD];
-        project_rows<T, DD, RPT, NT>(rows, Ws, acc);
+        float acc[RPT][CW];
+        project_rows<T, DD, CW, RPT>(rows, Ws + c0, r0, NR, acc);
         T *pool = static_cast<T *>(kv ? a.pool_vd : a.pool_kd);
 #pragma unroll
         for (int k = 0; k < RPT; ++k) {
-            const int m = L + j0 + tid + k * NT - w;
+            const int m = L + j0 + r0 + k * NR - w;
             if (id[k] >= 0)
-                store_row<T, DD>(pool + (((size_t)id[k] * a.Hkv + g) * kPage + m % kPage) * DD, acc[k]);
+                store_row<T, CW>(pool + (((size_t)id[k] * a.Hkv + g) * kPage + m % kPage) * DD + c0, acc[k]);
         }
     }
     // ring slots (L + j) % w, j < min(nb, w): the last new token of each
@@ -512,11 +406,12 @@ static cudaError_t cache_append_t(int dd, const AppendArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-template <typename T, int DD, int RPT, int NT>
+template <typename T, int DD, int RPT, int NR>
 static cudaError_t append_bulk_launch(const AppendArgs &a, cudaStream_t s)
 {
-    const int tiles = (a.n + RPT * NT - 1) / (RPT * NT);
-    append_bulk_kernel<T, DD, RPT, NT><<<dim3((unsigned)(a.B * a.Hkv * tiles), 2), NT, 0, s>>>(a, tiles);
+    const int tiles = (a.n + RPT * NR - 1) / (RPT * NR);
+    append_bulk_kernel<T, DD, RPT, NR>
+        <<<dim3((unsigned)(a.B * a.Hkv * tiles), 2), NR * slices<DD>(), 0, s>>>(a, tiles);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return e;
@@ -534,17 +429,17 @@ static cudaError_t append_bulk_launch(const AppendArgs &a, cudaStream_t s)
 
 // Big tiles (several rows per thread, so that one read of W feeds them all)
 // once they fill the chip a few times over; otherwise one row per thread.
-constexpr int kBulkSmallThreads = 64;
+constexpr int kBulkSmallRows = 64;
 constexpr long long kBulkBigCtas = 152 * 6 * 2;
 
 template <typename T, int DD>
 static cudaError_t append_bulk(const AppendArgs &a, cudaStream_t s)
 {
-    constexpr int RPT = rows_per_thread<DD>(), NT = threads_bulk<T, DD>();
-    const long long big = ((long long)a.n + RPT * NT - 1) / (RPT * NT) * a.B * a.Hkv * 2;
+    constexpr int R = rows_bulk<T>();
+    const long long big = ((long long)a.n + R - 1) / R * a.B * a.Hkv * 2;
     if (big >= kBulkBigCtas)
-        return append_bulk_launch<T, DD, RPT, NT>(a, s);
-    return append_bulk_launch<T, DD, 1, kBulkSmallThreads>(a, s);
+        return append_bulk_launch<T, DD, rows_per_thread<DD>(), R / rows_per_thread<DD>()>(a, s);
+    return append_bulk_launch<T, DD, 1, kBulkSmallRows>(a, s);
 }
 
 template <typename T>
@@ -572,7 +467,7 @@ constexpr int kBulkMinTokens = kAppRows + 1;
 static bool use_bulk(dar_dtype dt, const AppendArgs &a)
 {
     const long long row = 2ll * a.Hkv * kHeadDim * (dt == DAR_F32 ? 4 : 2);
-    const long long tiles = ((long long)a.n + kBulkSmallThreads - 1) / kBulkSmallThreads;
+    const long long tiles = ((long long)a.n + kBulkSmallRows - 1) / kBulkSmallRows;
     return a.n >= kBulkMinTokens && row <= kAppStageBytes && tiles * a.B * a.Hkv <= 0x7fffffffLL;
 }
 
