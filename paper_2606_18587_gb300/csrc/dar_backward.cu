@@ -57,9 +57,15 @@ cudaError_t launch_backward(dar_dtype dt, const BackwardArgs &x, void *workspace
     a.dvd = reinterpret_cast<float *>(take(krows * x.dd * 4));
     a.part = reinterpret_cast<float *>(take((size_t)bwd::kChunks * 4 * x.Hkv * 64 * x.dd * 4));
     a.qtb = a.dotb = nullptr;
-    if (dt == DAR_BF16) {  // bf16 copies of q~ and dO~ for the tensor-core kernels
+    a.gm = a.gl = a.fac = nullptr;
+    if (dt == DAR_BF16 && x.dd >= 16) {
+        // the tensor-core kernels take q~ and dO~ in bf16; the room of their
+        // fp32 form (dd >= 16 words per row) holds three words per row instead
         a.qtb = reinterpret_cast<bf16 *>(take(qrows * x.dd * 2));
         a.dotb = reinterpret_cast<bf16 *>(take(qrows * x.dd * 2));
+        a.gm = a.qt;
+        a.gl = a.gm + qrows;
+        a.fac = a.gl + qrows;
     }
     a.B = x.B;
     a.Hq = x.Hq;

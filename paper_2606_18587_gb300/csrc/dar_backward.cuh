@@ -34,6 +34,7 @@
 
 #include "dar_common.cuh"
 #include "dar_launch.h"
+#include "dar_sm100.cuh"
 
 namespace dar {
 namespace bwd {
@@ -52,7 +53,13 @@ struct Args {
     float *drow, *lse;                   // [B][Hq][N]: D, log2-sum-exp2 of the scaled scores
     float *dqt, *od;                     // [B][Hq][N][DD]: dq~ (scaled), O^D
     float *dkd, *dvd;                    // [B][Hkv][N][DD]: dk^D (scaled), dv^D
-    bf16 *qtb, *dotb;                    // [B][Hq][N][DD]: q~, dO~ rounded to bf16 (tensor-core operands)
+    // tensor-core kernels only (nullptr otherwise): q~ and dO~ rounded to bf16
+    // [B][Hq][N][DD], and per row the global part's running maximum and sum
+    // and the factor that normalises its dq~ and O^D [B][Hq][N].  There drow
+    // and lse hold -D and minus the log-sum-exp, and dqt (scaled) and od are
+    // left unnormalised; qt and dot are not used.
+    bf16 *qtb, *dotb;
+    float *gm, *gl, *fac;
     float *part;                         // [kChunks][4][Hkv][64 * DD]
     int B, Hq, Hkv, G, N, w;
     float scale, c2;                     // scale, scale * log2(e)
@@ -106,10 +113,6 @@ __global__ void __launch_bounds__(256) bwd_rows_kernel(Args a)
             }
             a.qt[row * DD + c] = sq;
             a.dot[row * DD + c] = sd;
-            if (a.qtb) {
-                a.qtb[row * DD + c] = __float2bfloat16_rn(sq);
-                a.dotb[row * DD + c] = __float2bfloat16_rn(sd);
-            }
         }
         __syncwarp();
     }
@@ -501,55 +504,129 @@ __global__ void __launch_bounds__(kThreads) bwd_dkv_kernel(Args a)
 //         1: X = q, Y = dq~  (rows of (b, h in g)) -> dUk (transposed at the end)
 //         2: X = v, Y = dv^D                       -> dDv
 //         3: X = dO, Y = O^D                       -> dUv (transposed)
+// (with a.fac, Y of 1 and 3 times the row's factor).
+//
+// A thread holds a 4 x 4 block of outputs, so two 16-byte shared-memory reads
+// feed 16 products; 64 / DD groups of threads share out the rows of a stage and
+// are added up in group order at the end.  Stages of 32 rows arrive by cp.async,
+// several deep: the sums then run near the rate at which X and Y (0.8 GB for
+// B8 H16 N8192, d_down 16) come from memory.  With one output per thread and
+// row (two reads per product) and unbuffered stages that shape took 1743 us.
+constexpr int kWRows = 32;
+
+template <typename T, int DD>
+struct WpartSmem {
+    static constexpr int X = kWRows * kHeadDim * (int)sizeof(T), Y = X + kWRows * DD * 4, STAGE = Y + kWRows * 4;
+    static constexpr int NS = STAGE * 4 <= 48 << 10 ? 4 : 2;
+    static constexpr int RED = kThreads * 16 * 4;
+    static constexpr int TOTAL = NS * STAGE > RED ? NS * STAGE : RED;
+    static_assert(TOTAL <= 48 << 10, "static shared memory");
+};
+
 template <typename T, int DD>
 __global__ void __launch_bounds__(kThreads) bwd_wpart_kernel(Args a)
 {
-    constexpr int PER = 64 * DD / kThreads;  // outputs per thread
-    constexpr int RS = 32;                   // rows staged at a time
-    __shared__ float Xs[RS][kHeadDim + 1];
-    __shared__ float Ys[RS][DD + 1];
-    const int chunk = blockIdx.x, g = blockIdx.y, which = blockIdx.z;
+    using Sm = WpartSmem<T, DD>;
+    constexpr int NG = 64 / DD, TPG = kThreads / NG, NS = Sm::NS;
+    constexpr int XC = kHeadDim * (int)sizeof(T) / 16, YC = DD / 4;  // 16-byte chunks per row
+    __shared__ __align__(16) unsigned char sm[Sm::TOTAL];
+    const uint32_t sb = sm100::smem_u32(sm);
+    const int tid = threadIdx.x, chunk = blockIdx.x, g = blockIdx.y, which = blockIdx.z;
     const bool per_kv = which == 0 || which == 2;
-    const long nrows = per_kv ? (long)a.B * a.N : (long)a.B * a.G * a.N;
+    const bool scaled = !per_kv && a.fac != nullptr;
+    const int heads = per_kv ? 1 : a.G;  // of KV head g, per batch element
+    const long nrows = (long)a.B * heads * a.N;
     const long r0 = nrows * chunk / kChunks, r1 = nrows * (chunk + 1) / kChunks;
     const T *X = static_cast<const T *>(which == 0 ? a.k : which == 1 ? a.q : which == 2 ? a.v : a.dout);
     const float *Y = which == 0 ? a.dkd : which == 1 ? a.dqt : which == 2 ? a.dvd : a.od;
-    float acc[PER];
-#pragma unroll
-    for (int e = 0; e < PER; ++e)
-        acc[e] = 0.f;
-    for (long rb = r0; rb < r1; rb += RS) {
-        const int n = (int)min((long)RS, r1 - rb);
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < RS * kHeadDim; idx += kThreads) {
-            const int rr = idx / kHeadDim, t = idx % kHeadDim;
-            float xv = 0.f;
-            if (rr < n) {
-                const long u = rb + rr;  // per_kv: b * N + j; else (b * G + hh) * N + i
-                long row;
-                if (per_kv)
-                    row = ((u / a.N) * a.Hkv + g) * a.N + u % a.N;
-                else
-                    row = (((u / a.N) / a.G) * a.Hq + g * a.G + (u / a.N) % a.G) * a.N + u % a.N;
-                xv = to_f32(X[row * kHeadDim + t]);
-                if (t < DD)
-                    Ys[rr][t] = Y[row * DD + t];
-            }
-            Xs[rr][t] = xv;
+    // first row, in memory, of sequence-and-head u of the rows this block sums
+    auto base_of = [&](long u) -> long {
+        return (per_kv ? u * a.Hkv + g : u / a.G * a.Hq + g * a.G + u % a.G) * a.N;
+    };
+    const int ntiles = (int)((r1 - r0 + kWRows - 1) / kWRows);
+    auto stage = [&](int t) {
+        if (t < ntiles) {
+            const long rb = r0 + (long)t * kWRows, u0 = rb / a.N;
+            const int i0 = (int)(rb % a.N), n = (int)min((long)kWRows, r1 - rb);
+            const long first = base_of(u0);
+            const uint32_t d = sb + (t % NS) * Sm::STAGE;
+            auto row_of = [&](int r) -> long {  // row r of the tile (it may run into the next sequences)
+                int i = i0 + r;
+                if (i < a.N)
+                    return first + i;
+                long u = u0;
+                while (i >= a.N) {
+                    i -= a.N;
+                    ++u;
+                }
+                return base_of(u) + i;
+            };
+            for (int e = tid; e < n * XC; e += kThreads)
+                sm100::cp_async16(d + e * 16, X + row_of(e / XC) * kHeadDim + e % XC * (16 / (int)sizeof(T)));
+            for (int e = tid; e < n * YC; e += kThreads)
+                sm100::cp_async16(d + Sm::X + e * 16, Y + row_of(e / YC) * DD + e % YC * 4);
+            if (scaled && tid < n)
+                sm100::cp_async4(d + Sm::Y + tid * 4, a.fac + row_of(tid));
         }
-        __syncthreads();
-        for (int rr = 0; rr < n; ++rr) {
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    const int grp = tid / TPG, c0 = tid % TPG % YC * 4, t0 = tid % TPG / YC * 4;
+    float acc[4][4];
 #pragma unroll
-            for (int e = 0; e < PER; ++e) {
-                const int o = threadIdx.x + kThreads * e, t = o / DD, c = o % DD;
-                acc[e] = fmaf(Xs[rr][t], Ys[rr][c], acc[e]);
+    for (int e = 0; e < 4; ++e)
+        acc[e][0] = acc[e][1] = acc[e][2] = acc[e][3] = 0.f;
+    for (int t = 0; t < NS - 1; ++t)
+        stage(t);
+    for (int t = 0; t < ntiles; ++t) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(NS - 2) : "memory");
+        __syncthreads();
+        stage(t + NS - 1);
+        const unsigned char *st = sm + (t % NS) * Sm::STAGE;
+        const float *fac = reinterpret_cast<const float *>(st + Sm::Y);
+        const int n = (int)min((long)kWRows, r1 - r0 - (long)t * kWRows);
+#pragma unroll 4
+        for (int r = grp; r < n; r += NG) {
+            float x[4];
+            if constexpr (sizeof(T) == 2) {
+                const uint2 v = *reinterpret_cast<const uint2 *>(st + (r * kHeadDim + t0) * 2);
+                x[0] = bf16lo(v.x);
+                x[1] = bf16hi(v.x);
+                x[2] = bf16lo(v.y);
+                x[3] = bf16hi(v.y);
+            } else {
+                const float4 v = *reinterpret_cast<const float4 *>(st + (r * kHeadDim + t0) * 4);
+                x[0] = v.x;
+                x[1] = v.y;
+                x[2] = v.z;
+                x[3] = v.w;
+            }
+            float4 y = *reinterpret_cast<const float4 *>(st + Sm::X + (r * DD + c0) * 4);
+            if (scaled) {
+                const float f = fac[r];
+                y = make_float4(y.x * f, y.y * f, y.z * f, y.w * f);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                sm100::ffma2(acc[e][0], acc[e][1], x[e], x[e], y.x, y.y, acc[e][0], acc[e][1]);
+                sm100::ffma2(acc[e][2], acc[e][3], x[e], x[e], y.z, y.w, acc[e][2], acc[e][3]);
             }
         }
     }
-    float *dst = a.part + (((size_t)chunk * 4 + which) * a.Hkv + g) * 64 * DD;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    float *red = reinterpret_cast<float *>(sm);  // [NG][64 * DD]
 #pragma unroll
-    for (int e = 0; e < PER; ++e)
-        dst[threadIdx.x + kThreads * e] = acc[e];
+    for (int e = 0; e < 4; ++e)
+        *reinterpret_cast<float4 *>(red + grp * 64 * DD + (t0 + e) * DD + c0) =
+            make_float4(acc[e][0], acc[e][1], acc[e][2], acc[e][3]);
+    __syncthreads();
+    float *dst = a.part + (((size_t)chunk * 4 + which) * a.Hkv + g) * 64 * DD;
+    for (int o = tid; o < 64 * DD; o += kThreads) {
+        float s = red[o];
+        for (int k = 1; k < NG; ++k)
+            s += red[k * 64 * DD + o];
+        dst[o] = s;
+    }
 }
 
 template <int DD>

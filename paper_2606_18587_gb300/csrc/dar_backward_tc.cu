@@ -1,50 +1,58 @@
 // dar_backward_tc.cu -- the backward pass for bf16 storage on the tensor
 // cores (mma.sync m16n8k16: bf16 operands, fp32 accumulators), with the
-// row kernel and the projection-gradient kernels of dar_backward.cuh.
+// projection-gradient kernels of dar_backward.cuh.
 //
-// The same gradients as the CUDA-core kernels (dar_backward.cuh), arranged
-// as FlashAttention-style recomputation in 16-key (or 16-query) steps held in
-// registers:
-//  - dq kernel, one CTA per 64 query rows of a head (four warps of 16 rows):
-//    a first pass over the key tiles for the row log-sum-exp, a second for
-//      P = 2^(s c2 - lse),  dP = dO v | dO~ v^D,  dS = P (dP - D),
-//      dq += dS_loc K,  dq~ += dS_glob K^D,  O^D += P_glob V^D,
-//    the score and dP fragments turned into A operands in registers;
-//  - dkv kernel, one CTA per 64 keys of a KV head (four warps of 16 keys):
-//    over the group's query heads and the query tiles that see the keys,
-//    S^T and dP^T per 16-query step, then
-//      dv += P_loc dO,  dk += dS_loc Q,  dv^D += P_glob dO~,  dk^D += dS_glob q~.
-// Key / query tiles are staged with 16-byte cp.async copies into padded
-// shared-memory rows (row stride a multiple of 16 bytes plus 16, so the eight
-// rows of an ldmatrix fall in distinct banks), two stages deep; a tile whose
-// pairs are all global skips the full-d rows and vice versa.
+// The gradients of dar_backward.cuh as FlashAttention-style recomputation with
+// the local (full-width) and the global (d_down-wide) pairs in kernels of
+// their own, so that each holds only its own accumulators and operands:
+//  - rows: q~ = q Uk^T, dO~ = dO Uv^T (bf16) and -D = -dO . o.
+//  - dq, per tile of query rows, ONE pass over the keys.  D does not depend on
+//    the softmax, so every sum is linear in the weights and can be taken with
+//    the running maximum m of an online softmax instead of the log-sum-exp:
+//      dS' = 2^(s c2 - m) (dP - D),  dq' += dS' K,  l += 2^(s c2 - m),
+//    and the row is divided by l at its end.  The global kernel leaves its
+//    unnormalised dq~ and O^D with (m, l); the local kernel, run after it,
+//    merges both parts into the row's log-sum-exp, lifts dq~ and writes dq and
+//    the factor that normalises the global part's sums.
+//  - dk/dv, per tile of keys over the query heads of the group and the query
+//    rows that see them, from the log-sum-exp:
+//      dv += P dO, dk += dS Q (local) | dv^D += P dO~, dk^D += dS q~ (global);
+//    the local kernel, run after the global one, lifts dk^D and dv^D into its
+//    own dk and dv.
+// Both kinds of kernel hold the scores of a 16-key (16-query) step in registers
+// and turn them into A operands of the next products.  -D enters as the
+// accumulator input of dP, so dP - D costs no instruction; scores, weights and
+// sums advance two per instruction (f32x2).  A warp takes 32 rows where the
+// accumulators allow it, so an operand read from shared memory feeds two
+// products: with 16 rows the reads alone would take longer than the products.
+// Tiles arrive by 16-byte cp.async copies in padded rows (stride a multiple of
+// 16 bytes plus 16: the eight rows of an ldmatrix fall in distinct banks),
+// three stages deep.
 #include "dar_backward.cuh"
+#include "dar_project.cuh"
 #include "dar_sm100.cuh"
 
 namespace dar {
 namespace bwd {
 
+using sm100::add2;
 using sm100::cvt_bf16x2;
+using sm100::ex2_approx;
+using sm100::ffma2;
 using sm100::ldsm_x4;
 using sm100::ldsm_x4_t;
-using sm100::mma_bf16_16816;
+using sm100::mma_bf16_c;
+using sm100::mul2;
 using sm100::smem_u32;
 
-constexpr int kTc = 128;           // threads: four warps
-constexpr int kLdW = 64 * 2 + 16;  // bytes per padded row of a 64-wide bf16 tile
-template <int DD>
-constexpr int ld_dd()
-{
-    return DD * 2 + 16;
-}
+constexpr int kTc = 128;  // threads: four warps
+constexpr float kRaise = 8.0f;  // log2 units: a weight stays below 2^8 between raises of a running maximum
 
-__device__ __forceinline__ void cp16(uint32_t dst, const void *src)
+// 16-byte copy, or 16 zero bytes when !valid (src must still be an address in the tensor).
+__device__ __forceinline__ void cp16z(uint32_t dst, const void *src, bool valid)
 {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp4(uint32_t dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+    const int n = valid ? 16 : 0;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -53,29 +61,24 @@ __device__ __forceinline__ void cp_wait()
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Rows [0, n) of a row-major [*][W] bf16 matrix into a padded tile of 64 rows
-// (row stride LD bytes); rows n..63 are zero-filled.
-template <int W, int LD>
-__device__ __forceinline__ void stage_rows(uint32_t dst, unsigned char *dstp, const bf16 *src, int n, int tid)
+// Bytes per padded row of a W-wide bf16 tile.
+template <int W>
+__host__ __device__ constexpr int ld_of()
 {
-    constexpr int CH = W / 8;
-    for (int i = tid; i < 64 * CH; i += kTc) {
-        const int r = i / CH, c = i % CH;
-        if (r < n)
-            cp16(dst + r * LD + c * 16, src + (size_t)r * W + c * 8);
-        else
-            *reinterpret_cast<uint4 *>(dstp + r * LD + c * 16) = make_uint4(0u, 0u, 0u, 0u);
-    }
+    return W * 2 + 16;
 }
 
-// 64 fp32 values (n valid, the rest zero).
-__device__ __forceinline__ void stage_vec(uint32_t dst, float *dstp, const float *src, int n, int tid)
+// Rows [0, n) of a row-major [*][W] bf16 matrix into a padded tile of ROWS rows; the others are zero.
+template <int W, int ROWS>
+__device__ __forceinline__ void stage_rows(uint32_t dst, const bf16 *src, int n, int tid)
 {
-    if (tid < 64) {
-        if (tid < n)
-            cp4(dst + tid * 4, src + tid);
-        else
-            dstp[tid] = 0.f;
+    constexpr int CH = W / 8;
+    static_assert(ROWS * CH % kTc == 0, "every thread copies the same number of chunks");
+#pragma unroll
+    for (int e = 0; e < ROWS * CH / kTc; ++e) {
+        const int i = tid + e * kTc, r = i / CH, c = i % CH;
+        const bool ok = r < n;
+        cp16z(dst + r * ld_of<W>() + c * 16, src + (ok ? (size_t)r * W + c * 8 : 0), ok);
     }
 }
 
@@ -88,636 +91,651 @@ __device__ __forceinline__ void frag_a(uint32_t (&a)[4], const float (&c0)[4], c
     a[3] = cvt_bf16x2(c1[2], c1[3]);
 }
 
-// Row address for ldmatrix (non-transposed, B operand of two n-tiles): the
-// 16 rows r0.. of a tile with row stride LD, 16-element k-step kk.
+// Lane offset for ldmatrix (non-transposed, B operand of two n-tiles): 16 rows
+// of a tile with row stride LD, first 16 columns.
 template <int LD>
-__device__ __forceinline__ uint32_t b_addr(uint32_t base, int r0, int kk, int lane)
+__device__ __forceinline__ uint32_t b_lane(int lane)
 {
-    return base + (r0 + (lane & 7) + ((lane >> 4) << 3)) * LD + (2 * kk + ((lane >> 3) & 1)) * 16;
+    return ((lane & 7) + ((lane >> 4) << 3)) * LD + ((lane >> 3) & 1) * 16;
 }
-// Row address for ldmatrix.trans (B operand [k][n] of two n-tiles at column n0):
-// k rows k0..k0+15.
+// Lane offset for ldmatrix.trans (B operand [k][n] of two n-tiles): 16 rows k, first 16 columns n.
 template <int LD>
-__device__ __forceinline__ uint32_t bt_addr(uint32_t base, int k0, int n0, int lane)
+__device__ __forceinline__ uint32_t bt_lane(int lane)
 {
-    return base + (k0 + (lane & 7) + (((lane >> 3) & 1) << 3)) * LD + ((n0 + ((lane >> 4) << 3)) / 8) * 16;
+    return ((lane & 7) + (((lane >> 3) & 1) << 3)) * LD + (lane >> 4) * 16;
 }
-// Row address for ldmatrix of an A operand (16 rows r0.., k-step kk).
-template <int LD>
-__device__ __forceinline__ uint32_t a_addr(uint32_t base, int r0, int kk, int lane)
+
+// A fragments of 16 rows (row0 + lane group, + 8) of a row-major [*][W] bf16
+// matrix, straight from global memory; rows at or past n are zero.
+template <int W>
+__device__ __forceinline__ void load_a(uint32_t (&f)[W / 16][4], const bf16 *src, int row0, int n, int lane)
 {
-    return base + (r0 + (lane & 15)) * LD + (2 * kk + (lane >> 4)) * 16;
+    const int grp = lane >> 2, tig = lane & 3;
+#pragma unroll
+    for (int kk = 0; kk < W / 16; ++kk)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int r = row0 + grp + 8 * (e & 1);
+            f[kk][e] = r < n ? __ldg(reinterpret_cast<const uint32_t *>(src + (size_t)r * W + 16 * kk + 8 * (e >> 1) + 2 * tig))
+                             : 0u;
+        }
 }
+
+// C (+)= A B^T over W columns: A fragments of MT row tiles, B the 16 rows whose
+// ldmatrix lane address is `b`; c0 holds the accumulator input of each tile.
+template <int W, int MT>
+__device__ __forceinline__ void scores(float (&s)[MT][2][4], const uint32_t (&a)[MT][W / 16][4], uint32_t b,
+                                       const float (&c0)[MT][2][4])
+{
+#pragma unroll
+    for (int kk = 0; kk < W / 16; ++kk) {
+        uint32_t f[4];
+        ldsm_x4(b + kk * 32, f);
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+            if (kk == 0) {
+                mma_bf16_c(s[mt][0], a[mt][kk], f[0], f[1], c0[mt][0]);
+                mma_bf16_c(s[mt][1], a[mt][kk], f[2], f[3], c0[mt][1]);
+            } else {
+                mma_bf16_c(s[mt][0], a[mt][kk], f[0], f[1], s[mt][0]);
+                mma_bf16_c(s[mt][1], a[mt][kk], f[2], f[3], s[mt][1]);
+            }
+        }
+    }
+}
+
+// acc += A B over 16 rows: B [16 rows][W] read transposed at lane address `b`.
+template <int W, int MT>
+__device__ __forceinline__ void accumulate(float (&acc)[MT][W / 8][4], const uint32_t (&a)[MT][4], uint32_t b)
+{
+#pragma unroll
+    for (int n = 0; n < W / 8; n += 2) {
+        uint32_t f[4];
+        ldsm_x4_t(b + n * 16, f);
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+            mma_bf16_c(acc[mt][n], a[mt], f[0], f[1], acc[mt][n]);
+            mma_bf16_c(acc[mt][n + 1], a[mt], f[2], f[3], acc[mt][n + 1]);
+        }
+    }
+}
+
+// out[2] (columns t, t + 1 of a row) += sum_c x[c] M[c][t], M fp32 rows of 64 in shared memory.
+template <int DD>
+__device__ __forceinline__ void lift16(float (&o)[8][2], const float *x, const float *M, int tig)
+{
+#pragma unroll 4
+    for (int c = 0; c < DD; ++c) {
+        const float xv = x[c];
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            const float2 m = *reinterpret_cast<const float2 *>(M + c * 64 + 8 * n + 2 * tig);
+            ffma2(o[n][0], o[n][1], xv, xv, m.x, m.y, o[n][0], o[n][1]);
+        }
+    }
+}
+
+// Row tiles per warp and rows of the streamed tile per stage.
+template <int W, bool LOCAL>
+struct Shape {
+    static constexpr int MT = !LOCAL && W <= 32 ? 2 : 1;
+    static constexpr int ROWS = 64 * MT;                   // rows of a CTA's tile
+    static constexpr int BK = !LOCAL && W <= 32 ? 128 : 64;  // streamed rows per stage
+    static constexpr int NS = 3;
+    static constexpr int MINB = W == 16 ? 3 : W == 32 ? 2 : LOCAL ? 3 : 2;
+};
 
 // ---------------------------------------------------------------- dq
 
-template <int DD>
-struct DqLayout {
-    static constexpr int LD = ld_dd<DD>();
-    static constexpr uint32_t Q = 0;                      // [64][kLdW] q rows
-    static constexpr uint32_t DO = Q + 64 * kLdW;         // dO rows
-    static constexpr uint32_t QT = DO + 64 * kLdW;        // [64][LD] q~ rows (bf16)
-    static constexpr uint32_t DOT = QT + 64 * LD;         // dO~ rows (bf16)
-    static constexpr uint32_t STG = DOT + 64 * LD;        // two stages of key-side tiles
-    static constexpr uint32_t K_OFF = 0, V_OFF = 64 * kLdW, KD_OFF = 2 * 64 * kLdW, VD_OFF = KD_OFF + 64 * LD;
-    static constexpr uint32_t STAGE = VD_OFF + 64 * LD;
-    static constexpr uint32_t TOTAL = STG + 2 * STAGE;
-    static_assert(64 * (DD + 1) * 4 <= 2 * STAGE, "the epilogue's lift rows fit in the stage area");
+template <int W, bool LOCAL, int DD>
+struct DqSmem {
+    using Sh = Shape<W, LOCAL>;
+    static constexpr uint32_t V = Sh::BK * ld_of<W>(), STAGE = 2 * V;
+    static constexpr uint32_t TOTAL = Sh::NS * STAGE;
+    // the epilogue's lift: [64][DD + 1] dq~ rows and Uk
+    static_assert(!LOCAL || 64 * (DD + 1) * 4 + DD * 64 * 4 <= TOTAL, "the lift fits in the stage area");
 };
 
-template <int DD>
-__global__ void __launch_bounds__(kTc, DD <= 32 ? 3 : 1) bwd_dq_tc_kernel(Args a)
+template <int W, bool LOCAL, int DD>
+__global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(Args a)
 {
-    using Ly = DqLayout<DD>;
-    constexpr int LD = Ly::LD, KSD = DD / 16, NTD = DD / 8;
+    using Sh = Shape<W, LOCAL>;
+    using Sm = DqSmem<W, LOCAL, DD>;
+    constexpr int MT = Sh::MT, ROWS = Sh::ROWS, BK = Sh::BK, NS = Sh::NS, LD = ld_of<W>(), NT = W / 8;
     extern __shared__ __align__(128) unsigned char tsm[];
-    unsigned char *sm = tsm;
-    const uint32_t sb = smem_u32(sm);
-    const int N = a.N, w = a.w;
-    const int bh = blockIdx.y, b = bh / a.Hq, h = bh % a.Hq, g = h / a.G;
-    const int i0 = blockIdx.x * 64;
+    const uint32_t sb = smem_u32(tsm);
+    const int N = a.N, w = min(a.w, N);  // (a window past the sequence's length makes every pair local too)
+    const int heads = a.B * a.Hq, bh = blockIdx.x % heads, b = bh / a.Hq, h = bh % a.Hq, g = h / a.G;
+    const int i0 = ((int)(gridDim.x / heads) - 1 - (int)(blockIdx.x / heads)) * ROWS;  // longest rows first
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, grp = lane >> 2, tig = lane & 3;
-    const int nv = min(64, N - i0);
-    const size_t rowbase = ((size_t)b * a.Hq + h) * N + i0;
+    const size_t headrow = (size_t)bh * N;
     const size_t kvbase = ((size_t)b * a.Hkv + g) * N;
-    const bf16 *kp = static_cast<const bf16 *>(a.k) + kvbase * 64;
-    const bf16 *vp = static_cast<const bf16 *>(a.v) + kvbase * 64;
-    const bf16 *kdp = static_cast<const bf16 *>(a.kd) + kvbase * DD;
-    const bf16 *vdp = static_cast<const bf16 *>(a.vd) + kvbase * DD;
-    const int imax = min(N, i0 + 64) - 1;
-    const int ntiles = imax / 64 + 1;
-    const int wr0 = 16 * warp;  // this warp's first row in the tile
-
-    stage_rows<64, kLdW>(sb + Ly::Q, sm + Ly::Q, static_cast<const bf16 *>(a.q) + rowbase * 64, nv, tid);
-    stage_rows<64, kLdW>(sb + Ly::DO, sm + Ly::DO, static_cast<const bf16 *>(a.dout) + rowbase * 64, nv, tid);
-    stage_rows<DD, LD>(sb + Ly::QT, sm + Ly::QT, a.qtb + rowbase * DD, nv, tid);
-    stage_rows<DD, LD>(sb + Ly::DOT, sm + Ly::DOT, a.dotb + rowbase * DD, nv, tid);
-    cp_commit();
-
-    // virtual step v: pass v / ntiles (0: log-sum-exp, 1: gradients), key tile v % ntiles
-    auto stage_keys = [&](int v, int st) {
-        const int pass = v / ntiles, j0 = (v % ntiles) * 64, nk = min(64, N - j0);
-        const bool all_global = (i0 - (j0 + 63)) >= w, all_local = (i0 + 63 - j0) < w;
-        const uint32_t base = sb + Ly::STG + st * Ly::STAGE;
-        unsigned char *bp = sm + Ly::STG + st * Ly::STAGE;
-        if (!all_global) {
-            stage_rows<64, kLdW>(base + Ly::K_OFF, bp + Ly::K_OFF, kp + (size_t)j0 * 64, nk, tid);
-            if (pass)
-                stage_rows<64, kLdW>(base + Ly::V_OFF, bp + Ly::V_OFF, vp + (size_t)j0 * 64, nk, tid);
-        }
-        if (!all_local) {
-            stage_rows<DD, LD>(base + Ly::KD_OFF, bp + Ly::KD_OFF, kdp + (size_t)j0 * DD, nk, tid);
-            if (pass)
-                stage_rows<DD, LD>(base + Ly::VD_OFF, bp + Ly::VD_OFF, vdp + (size_t)j0 * DD, nk, tid);
+    const bf16 *kp = static_cast<const bf16 *>(LOCAL ? a.k : a.kd) + kvbase * W;
+    const bf16 *vp = static_cast<const bf16 *>(LOCAL ? a.v : a.vd) + kvbase * W;
+    const int i_last = min(N, i0 + ROWS) - 1;
+    // keys [jlo, jhi): local i - w < j <= i, global j <= i - w
+    const int jlo = LOCAL ? max(0, i0 - w + 1) / 16 * 16 : 0;
+    const int jhi = LOCAL ? (w > 0 ? i_last + 1 : jlo) : max(0, i_last - w + 1);
+    const int ntiles = (jhi - jlo + BK - 1) / BK;
+    auto stage = [&](int t) {
+        if (t < ntiles) {
+            const int j = jlo + t * BK;
+            const uint32_t dst = sb + (t % NS) * Sm::STAGE;
+            stage_rows<W, BK>(dst, kp + (size_t)j * W, N - j, tid);
+            stage_rows<W, BK>(dst + Sm::V, vp + (size_t)j * W, N - j, tid);
         }
         cp_commit();
     };
-    const int nvs = 2 * ntiles;
-    stage_keys(0, 0);
-    cp_wait<1>();  // the query-side rows (the first key stage may still be in flight)
-    __syncthreads();
+    for (int t = 0; t < NS - 1; ++t)
+        stage(t);
 
-    // A fragments: the d_down-wide rows stay in registers (every global step
-    // uses them); the 64-wide q and dO rows are read from shared memory by the
-    // (rarer) steps with local pairs, which keeps registers for occupancy
-    uint32_t qta[KSD][4], dota[KSD][4];
+    const int r0 = i0 + 16 * MT * warp;  // this warp's rows r0 .. r0 + 16 MT - 1
+    uint32_t qa[MT][W / 16][4], da[MT][W / 16][4];
+    float nD[MT][2][4], zero[MT][2][4];
+    float m[MT][2], l[MT][2][2];
 #pragma unroll
-    for (int kk = 0; kk < KSD; ++kk) {
-        ldsm_x4(a_addr<LD>(sb + Ly::QT, wr0, kk, lane), qta[kk]);
-        ldsm_x4(a_addr<LD>(sb + Ly::DOT, wr0, kk, lane), dota[kk]);
+    for (int mt = 0; mt < MT; ++mt) {
+        load_a<W>(qa[mt], (LOCAL ? static_cast<const bf16 *>(a.q) : a.qtb) + headrow * W, r0 + 16 * mt, N, lane);
+        load_a<W>(da[mt], (LOCAL ? static_cast<const bf16 *>(a.dout) : a.dotb) + headrow * W, r0 + 16 * mt, N, lane);
+#pragma unroll
+        for (int hr = 0; hr < 2; ++hr) {
+            const int i = r0 + 16 * mt + grp + 8 * hr;
+            const float d = i < N ? a.drow[headrow + i] : 0.f;
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt) {
+                nD[mt][nt][2 * hr] = nD[mt][nt][2 * hr + 1] = d;
+                zero[mt][nt][2 * hr] = zero[mt][nt][2 * hr + 1] = 0.f;
+            }
+            m[mt][hr] = -INFINITY;
+            l[mt][hr][0] = l[mt][hr][1] = 0.f;
+        }
     }
-    const int ir0 = i0 + wr0 + grp;  // this thread's rows: ir0 and ir0 + 8
-    float Dr[2], m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f}, lse[2] = {0.f, 0.f};
+    // dq~ and O^D (global), dq (local)
+    float dq[MT][NT][4], od[LOCAL ? 1 : MT][LOCAL ? 1 : NT][4];
 #pragma unroll
-    for (int r = 0; r < 2; ++r)
-        Dr[r] = ir0 + 8 * r < N ? a.drow[rowbase + wr0 + grp + 8 * r] : 0.f;
-    float dq[8][4], dqt[NTD][4], od[NTD][4];
+    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-    for (int n = 0; n < 8; ++n)
-        dq[n][0] = dq[n][1] = dq[n][2] = dq[n][3] = 0.f;
+        for (int n = 0; n < NT; ++n)
 #pragma unroll
-    for (int n = 0; n < NTD; ++n)
-        dqt[n][0] = dqt[n][1] = dqt[n][2] = dqt[n][3] = od[n][0] = od[n][1] = od[n][2] = od[n][3] = 0.f;
+            for (int e = 0; e < 4; ++e) {
+                dq[mt][n][e] = 0.f;
+                if constexpr (!LOCAL)
+                    od[mt][n][e] = 0.f;
+            }
+    const float c2 = a.c2;
+    bool fresh = true;  // some row of the warp may still have m = -infinity
 
-    for (int v = 0; v < nvs; ++v) {
-        const int pass = v / ntiles, st = v & 1;
-        const int j0 = (v % ntiles) * 64;
-        if (v + 1 < nvs) {
-            stage_keys(v + 1, st ^ 1);
-            cp_wait<1>();
-        } else {
-            cp_wait<0>();
-        }
-        __syncthreads();
-        if (pass == 1 && v == ntiles) {
-            // the rows' log-sum-exp: combine the four threads of each row
+    // raise the running maxima to those of these scores
+    auto raise = [&](const float (&s)[MT][2][4]) {
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
+        for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-                for (int o = 1; o <= 2; o <<= 1) {
-                    const float mo = __shfl_xor_sync(0xffffffffu, m[r], o), lo = __shfl_xor_sync(0xffffffffu, l[r], o);
-                    const float mn = fmaxf(m[r], mo);
-                    l[r] = (m[r] == -INFINITY ? 0.f : l[r] * exp2f(m[r] - mn)) +
-                           (mo == -INFINITY ? 0.f : lo * exp2f(mo - mn));
-                    m[r] = mn;
-                }
-                lse[r] = m[r] + log2f(l[r]);
-                if (tig == 0 && ir0 + 8 * r < N)
-                    a.lse[rowbase + wr0 + grp + 8 * r] = lse[r];
-            }
-        }
-        const bool all_global = (i0 - (j0 + 63)) >= w, all_local = (i0 + 63 - j0) < w;
-        // all pairs global, every key before every row, every row inside the sequence
-        const bool interior = all_global && j0 + 63 <= i0 && i0 + 63 < N;
-        const uint32_t stg = sb + Ly::STG + st * Ly::STAGE;
-#pragma unroll 1
-        for (int kc = 0; kc < 4; ++kc) {
-            if (j0 + 16 * kc > i0 + wr0 + 15)
-                break;  // every key of the step is after every row of this warp (causal)
-            float sl[2][4] = {}, sg[2][4] = {};
-            if (!all_global) {
+            for (int hr = 0; hr < 2; ++hr) {
+                float x = fmaxf(fmaxf(s[mt][0][2 * hr], s[mt][0][2 * hr + 1]), fmaxf(s[mt][1][2 * hr], s[mt][1][2 * hr + 1]));
+                x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 1));
+                x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 2));
+                const float mn = fmaxf(m[mt][hr], x * c2);
+                const float f = m[mt][hr] == -INFINITY ? 0.f : ex2_approx(m[mt][hr] - mn);
+                m[mt][hr] = mn;
+                l[mt][hr][0] *= f;
+                l[mt][hr][1] *= f;
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    uint32_t bfr[4], afr[4];
-                    ldsm_x4(a_addr<kLdW>(sb + Ly::Q, wr0, kk, lane), afr);
-                    ldsm_x4(b_addr<kLdW>(stg + Ly::K_OFF, 16 * kc, kk, lane), bfr);
-                    mma_bf16_16816(sl[0], afr, bfr[0], bfr[1]);
-                    mma_bf16_16816(sl[1], afr, bfr[2], bfr[3]);
-                }
-            }
-            if (!all_local) {
-#pragma unroll
-                for (int kk = 0; kk < KSD; ++kk) {
-                    uint32_t bfr[4];
-                    ldsm_x4(b_addr<LD>(stg + Ly::KD_OFF, 16 * kc, kk, lane), bfr);
-                    mma_bf16_16816(sg[0], qta[kk], bfr[0], bfr[1]);
-                    mma_bf16_16816(sg[1], qta[kk], bfr[2], bfr[3]);
-                }
-            }
-            if (interior) {  // every pair of the step is valid and global: no masks, no local part
-                if (pass == 0) {
-#pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const float x0 = sg[0][2 * r] * a.c2, x1 = sg[0][2 * r + 1] * a.c2;
-                        const float x2 = sg[1][2 * r] * a.c2, x3 = sg[1][2 * r + 1] * a.c2;
-                        const float mn = fmaxf(m[r], fmaxf(fmaxf(x0, x1), fmaxf(x2, x3)));
-                        l[r] = l[r] * sm100::ex2_approx(m[r] - mn) + (sm100::ex2_approx(x0 - mn) + sm100::ex2_approx(x1 - mn)) +
-                               (sm100::ex2_approx(x2 - mn) + sm100::ex2_approx(x3 - mn));
-                        m[r] = mn;
+                for (int n = 0; n < NT; ++n) {
+                    dq[mt][n][2 * hr] *= f;
+                    dq[mt][n][2 * hr + 1] *= f;
+                    if constexpr (!LOCAL) {
+                        od[mt][n][2 * hr] *= f;
+                        od[mt][n][2 * hr + 1] *= f;
                     }
-                    continue;
                 }
-                float dpg[2][4] = {};
+            }
+    };
+    auto exponents = [&](const float (&s)[MT][2][4], float (&y)[MT][2][4]) {
 #pragma unroll
-                for (int kk = 0; kk < KSD; ++kk) {
-                    uint32_t bfr[4];
-                    ldsm_x4(b_addr<LD>(stg + Ly::VD_OFF, 16 * kc, kk, lane), bfr);
-                    mma_bf16_16816(dpg[0], dota[kk], bfr[0], bfr[1]);
-                    mma_bf16_16816(dpg[1], dota[kk], bfr[2], bfr[3]);
-                }
-                float pg[2][4], dsg[2][4];
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int hr = 0; hr < 2; ++hr) {
+                const float nm = m[mt][hr] == -INFINITY ? 0.f : -m[mt][hr];
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        pg[nt][e] = sm100::ex2_approx(fmaf(sg[nt][e], a.c2, -lse[e >> 1]));
-                        dsg[nt][e] = pg[nt][e] * (dpg[nt][e] - Dr[e >> 1]);
-                    }
-                uint32_t ag[4], ap[4];
-                frag_a(ag, dsg[0], dsg[1]);
-                frag_a(ap, pg[0], pg[1]);
-#pragma unroll
-                for (int n0 = 0; n0 < DD; n0 += 16) {
-                    uint32_t bfr[4];
-                    ldsm_x4_t(bt_addr<LD>(stg + Ly::KD_OFF, 16 * kc, n0, lane), bfr);
-                    mma_bf16_16816(dqt[n0 / 8], ag, bfr[0], bfr[1]);
-                    mma_bf16_16816(dqt[n0 / 8 + 1], ag, bfr[2], bfr[3]);
-                    ldsm_x4_t(bt_addr<LD>(stg + Ly::VD_OFF, 16 * kc, n0, lane), bfr);
-                    mma_bf16_16816(od[n0 / 8], ap, bfr[0], bfr[1]);
-                    mma_bf16_16816(od[n0 / 8 + 1], ap, bfr[2], bfr[3]);
-                }
-                continue;
+                    ffma2(y[mt][nt][2 * hr], y[mt][nt][2 * hr + 1], s[mt][nt][2 * hr], s[mt][nt][2 * hr + 1], c2, c2,
+                          nm, nm);
             }
-            float x[2][4];
-            bool loc[2][4];
+    };
+
+    for (int t = 0; t < ntiles; ++t) {
+        cp_wait<NS - 2>();
+        __syncthreads();  // tile t is in; every warp is done with tile t - 1
+        stage(t + NS - 1);
+        const uint32_t ks = sb + (t % NS) * Sm::STAGE;
+        const int jt = jlo + t * BK;
+#pragma unroll 1
+        for (int kc = 0; kc < BK / 16; ++kc) {
+            const int j = jt + 16 * kc;
+            // Eq. 3: no pair of the step / every pair of the step is of this kind
+            if (LOCAL ? j > r0 + 16 * MT - 1 : j > r0 + 16 * MT - 1 - w)
+                break;
+            if (LOCAL && j + 15 <= r0 - w)
+                continue;
+            // (a masked pair's weight is 0; its dP - D is set to 0 too, so that no
+            // 0 * infinity arises from a key the row does not see)
+            const bool all = LOCAL ? j + 15 <= r0 && j > r0 + 16 * MT - 1 - w : j + 15 <= r0 - w;
+            const uint32_t kst = ks + 16 * kc * LD, vst = kst + Sm::V;
+            float s[MT][2][4], dp[MT][2][4], y[MT][2][4];
+            scores<W, MT>(s, qa, kst + b_lane<LD>(lane), zero);
+            scores<W, MT>(dp, da, vst + b_lane<LD>(lane), nD);
+            if (!all) {
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int i = ir0 + 8 * (e >> 1), j = j0 + 16 * kc + 8 * nt + 2 * tig + (e & 1);
-                    loc[nt][e] = i - j < w;
-                    x[nt][e] = (i < N && j <= i) ? (loc[nt][e] ? sl[nt][e] : sg[nt][e]) * a.c2 : -INFINITY;
-                }
-            if (pass == 0) {
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    const float mx = fmaxf(fmaxf(x[0][2 * r], x[0][2 * r + 1]), fmaxf(x[1][2 * r], x[1][2 * r + 1]));
-                    const float mn = fmaxf(m[r], mx);
-                    if (mn == -INFINITY)
-                        continue;
-                    float ps = 0.f;
+                for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                     for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-                        for (int e = 0; e < 2; ++e)
-                            ps += x[nt][2 * r + e] == -INFINITY ? 0.f : sm100::ex2_approx(x[nt][2 * r + e] - mn);
-                    l[r] = (m[r] == -INFINITY ? 0.f : l[r] * sm100::ex2_approx(m[r] - mn)) + ps;
-                    m[r] = mn;
-                }
-                continue;
+                        for (int e = 0; e < 4; ++e) {
+                            const int i = r0 + 16 * mt + grp + 8 * (e >> 1), jj = j + 8 * nt + 2 * tig + (e & 1);
+                            const bool in = LOCAL ? jj <= i && jj > i - w : jj <= i - w;
+                            s[mt][nt][e] = in ? s[mt][nt][e] : -INFINITY;
+                            dp[mt][nt][e] = in ? dp[mt][nt][e] : 0.f;
+                        }
             }
-            float dpl[2][4] = {}, dpg[2][4] = {};
-            if (!all_global) {
+            exponents(s, y);
+            float top = -INFINITY;
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    uint32_t bfr[4], afr[4];
-                    ldsm_x4(a_addr<kLdW>(sb + Ly::DO, wr0, kk, lane), afr);
-                    ldsm_x4(b_addr<kLdW>(stg + Ly::V_OFF, 16 * kc, kk, lane), bfr);
-                    mma_bf16_16816(dpl[0], afr, bfr[0], bfr[1]);
-                    mma_bf16_16816(dpl[1], afr, bfr[2], bfr[3]);
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt) {
+                    top = sm100::max3(top, y[mt][nt][0], y[mt][nt][1]);
+                    top = sm100::max3(top, y[mt][nt][2], y[mt][nt][3]);
                 }
+            if (__any_sync(0xffffffffu, top > kRaise) || fresh) {
+                raise(s);
+                exponents(s, y);
+                bool none = false;  // every row has seen a key from here on, once no maximum is -infinity
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt)
+                    none = none || m[mt][0] == -INFINITY || m[mt][1] == -INFINITY;
+                fresh = __any_sync(0xffffffffu, none);
             }
-            if (!all_local) {
+            uint32_t ds[MT][4], pa[MT][4];
 #pragma unroll
-                for (int kk = 0; kk < KSD; ++kk) {
-                    uint32_t bfr[4];
-                    ldsm_x4(b_addr<LD>(stg + Ly::VD_OFF, 16 * kc, kk, lane), bfr);
-                    mma_bf16_16816(dpg[0], dota[kk], bfr[0], bfr[1]);
-                    mma_bf16_16816(dpg[1], dota[kk], bfr[2], bfr[3]);
-                }
+            for (int mt = 0; mt < MT; ++mt) {
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                    for (int hr = 0; hr < 2; ++hr) {
+                        float &p0 = y[mt][nt][2 * hr], &p1 = y[mt][nt][2 * hr + 1];
+                        p0 = ex2_approx(p0);
+                        p1 = ex2_approx(p1);
+                        add2(l[mt][hr][0], l[mt][hr][1], p0, p1, l[mt][hr][0], l[mt][hr][1]);
+                        mul2(dp[mt][nt][2 * hr], dp[mt][nt][2 * hr + 1], p0, p1, dp[mt][nt][2 * hr],
+                             dp[mt][nt][2 * hr + 1]);
+                    }
+                frag_a(ds[mt], dp[mt][0], dp[mt][1]);
+                if constexpr (!LOCAL)
+                    frag_a(pa[mt], y[mt][0], y[mt][1]);
             }
-            float dsl[2][4], dsg[2][4], pgl[2][4];
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float p = x[nt][e] == -INFINITY ? 0.f : sm100::ex2_approx(x[nt][e] - lse[e >> 1]);
-                    const float ds = p * ((loc[nt][e] ? dpl[nt][e] : dpg[nt][e]) - Dr[e >> 1]);
-                    dsl[nt][e] = loc[nt][e] ? ds : 0.f;
-                    dsg[nt][e] = loc[nt][e] ? 0.f : ds;
-                    pgl[nt][e] = loc[nt][e] ? 0.f : p;
-                }
-            if (!all_global) {
-                uint32_t af[4];
-                frag_a(af, dsl[0], dsl[1]);
-#pragma unroll
-                for (int n0 = 0; n0 < 64; n0 += 16) {
-                    uint32_t bfr[4];
-                    ldsm_x4_t(bt_addr<kLdW>(stg + Ly::K_OFF, 16 * kc, n0, lane), bfr);
-                    mma_bf16_16816(dq[n0 / 8], af, bfr[0], bfr[1]);
-                    mma_bf16_16816(dq[n0 / 8 + 1], af, bfr[2], bfr[3]);
-                }
-            }
-            if (!all_local) {
-                uint32_t ag[4], ap[4];
-                frag_a(ag, dsg[0], dsg[1]);
-                frag_a(ap, pgl[0], pgl[1]);
-#pragma unroll
-                for (int n0 = 0; n0 < DD; n0 += 16) {
-                    uint32_t bfr[4];
-                    ldsm_x4_t(bt_addr<LD>(stg + Ly::KD_OFF, 16 * kc, n0, lane), bfr);
-                    mma_bf16_16816(dqt[n0 / 8], ag, bfr[0], bfr[1]);
-                    mma_bf16_16816(dqt[n0 / 8 + 1], ag, bfr[2], bfr[3]);
-                    ldsm_x4_t(bt_addr<LD>(stg + Ly::VD_OFF, 16 * kc, n0, lane), bfr);
-                    mma_bf16_16816(od[n0 / 8], ap, bfr[0], bfr[1]);
-                    mma_bf16_16816(od[n0 / 8 + 1], ap, bfr[2], bfr[3]);
-                }
-            }
+            accumulate<W, MT>(dq, ds, kst + bt_lane<LD>(lane));
+            if constexpr (!LOCAL)
+                accumulate<W, MT>(od, pa, vst + bt_lane<LD>(lane));
         }
-        __syncthreads();  // stage st is free for the copy issued in the next step
     }
 
-    // epilogue: dq = scale (dq_loc + dq~ Uk), dq~ (scaled) and O^D for the projection gradients
-    float *lift = reinterpret_cast<float *>(sm + Ly::STG);  // [64][DD + 1], the idle stage area
+    float lsum[MT][2];
 #pragma unroll
-    for (int n = 0; n < NTD; ++n)
+    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            lift[(wr0 + grp + 8 * (e >> 1)) * (DD + 1) + 8 * n + 2 * tig + (e & 1)] = dqt[n][e] * a.scale;
-    __syncwarp();
-    const float *Uk = a.Uk + (size_t)g * DD * 64;
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const int rr = wr0 + grp + 8 * r;
-        if (i0 + rr >= N)
-            continue;
-        const size_t row = rowbase + rr;
-        bf16 *dqr = static_cast<bf16 *>(a.dq) + row * 64;
-#pragma unroll
-        for (int n = 0; n < 8; ++n) {
-            const int t = 8 * n + 2 * tig;
-            float o0 = dq[n][2 * r] * a.scale, o1 = dq[n][2 * r + 1] * a.scale;
-            for (int c = 0; c < DD; ++c) {
-                const float x2 = lift[rr * (DD + 1) + c];
-                o0 = fmaf(x2, __ldg(Uk + c * 64 + t), o0);
-                o1 = fmaf(x2, __ldg(Uk + c * 64 + t + 1), o1);
-            }
-            *reinterpret_cast<uint32_t *>(dqr + t) = cvt_bf16x2(o0, o1);
+        for (int hr = 0; hr < 2; ++hr) {
+            float x = l[mt][hr][0] + l[mt][hr][1];
+            x += __shfl_xor_sync(0xffffffffu, x, 1);
+            x += __shfl_xor_sync(0xffffffffu, x, 2);
+            lsum[mt][hr] = x;
         }
+    if constexpr (!LOCAL) {
+        // the global part's sums relative to 2^m: dq~ (times scale), O^D, m, l
 #pragma unroll
-        for (int n = 0; n < NTD; ++n) {
-            const int c = 8 * n + 2 * tig;
-            *reinterpret_cast<float2 *>(a.dqt + row * DD + c) =
-                make_float2(dqt[n][2 * r] * a.scale, dqt[n][2 * r + 1] * a.scale);
-            *reinterpret_cast<float2 *>(a.od + row * DD + c) = make_float2(od[n][2 * r], od[n][2 * r + 1]);
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int hr = 0; hr < 2; ++hr) {
+                const int i = r0 + 16 * mt + grp + 8 * hr;
+                if (i >= N)
+                    continue;
+                const size_t row = headrow + i;
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                    const int c = 8 * n + 2 * tig;
+                    *reinterpret_cast<float2 *>(a.dqt + row * W + c) =
+                        make_float2(dq[mt][n][2 * hr] * a.scale, dq[mt][n][2 * hr + 1] * a.scale);
+                    *reinterpret_cast<float2 *>(a.od + row * W + c) = make_float2(od[mt][n][2 * hr], od[mt][n][2 * hr + 1]);
+                }
+                if (tig == 0) {
+                    a.gm[row] = m[mt][hr];
+                    a.gl[row] = lsum[mt][hr];
+                }
+            }
+    } else {
+        static_assert(!LOCAL || MT == 1, "the lift stages 64 rows");
+        // merge with the global part; dq = scale dq_loc / l + (dq~ / l) Uk
+        cp_wait<0>();
+        __syncthreads();  // the stage area is idle
+        float *lift = reinterpret_cast<float *>(tsm);  // [64][DD + 1]
+        float *uk = lift + 64 * (DD + 1);              // [DD][64]; 16-byte words: 64 * (DD + 1) floats come before
+        for (int e = tid; e < DD * 16; e += kTc)
+            reinterpret_cast<float4 *>(uk)[e] = __ldg(reinterpret_cast<const float4 *>(a.Uk + (size_t)g * DD * 64) + e);
+        const int nv = min(ROWS, N - i0);
+        for (int e = tid; e < nv * DD; e += kTc)
+            lift[(e / DD) * (DD + 1) + e % DD] = a.dqt[(headrow + i0) * DD + e];
+        __syncthreads();
+#pragma unroll
+        for (int hr = 0; hr < 2; ++hr) {
+            const int i = r0 + grp + 8 * hr;
+            if (i >= N)
+                continue;
+            const size_t row = headrow + i;
+            const float mg = a.gm[row], lg = a.gl[row], ml = m[0][hr], M = fmaxf(mg, ml);
+            const float L = (mg == -INFINITY ? 0.f : lg * ex2_approx(mg - M)) +
+                            (ml == -INFINITY ? 0.f : lsum[0][hr] * ex2_approx(ml - M));
+            const float lse = M + log2f(L);
+            const float fl = ml == -INFINITY ? 0.f : exp2f(ml - lse) * a.scale;
+            const float fg = mg == -INFINITY ? 0.f : exp2f(mg - lse);
+            if (tig == 0) {
+                a.lse[row] = -lse;
+                a.fac[row] = fg;
+            }
+            float o[8][2];
+#pragma unroll
+            for (int n = 0; n < 8; ++n)
+                o[n][0] = o[n][1] = 0.f;
+            lift16<DD>(o, lift + (i - i0) * (DD + 1), uk, tig);
+            bf16 *dst = static_cast<bf16 *>(a.dq) + row * 64;
+#pragma unroll
+            for (int n = 0; n < 8; ++n)
+                *reinterpret_cast<uint32_t *>(dst + 8 * n + 2 * tig) =
+                    cvt_bf16x2(fmaf(dq[0][n][2 * hr], fl, o[n][0] * fg), fmaf(dq[0][n][2 * hr + 1], fl, o[n][1] * fg));
         }
     }
 }
 
 // ---------------------------------------------------------------- dk, dv
 
-template <int DD>
-struct DkvLayout {
-    static constexpr int LD = ld_dd<DD>();
-    static constexpr uint32_t K = 0;                      // [64][kLdW] this CTA's keys
-    static constexpr uint32_t V = K + 64 * kLdW;
-    static constexpr uint32_t KD = V + 64 * kLdW;         // [64][LD]
-    static constexpr uint32_t VD = KD + 64 * LD;
-    static constexpr uint32_t STG = VD + 64 * LD;         // two stages of query-side tiles
-    static constexpr uint32_t Q_OFF = 0, DO_OFF = 64 * kLdW, QT_OFF = 2 * 64 * kLdW, DOT_OFF = QT_OFF + 64 * LD;
-    static constexpr uint32_t LSE_OFF = DOT_OFF + 64 * LD, DR_OFF = LSE_OFF + 256;
-    static constexpr uint32_t STAGE = DR_OFF + 256;
-    static constexpr uint32_t TOTAL = STG + 2 * STAGE;
-    static_assert(2 * 64 * (DD + 1) * 4 <= 2 * STAGE, "the epilogue's lift rows fit in the stage area");
+template <int W, bool LOCAL, int DD>
+struct DkvSmem {
+    using Sh = Shape<W, LOCAL>;
+    static constexpr uint32_t DO = Sh::BK * ld_of<W>();
+    static constexpr uint32_t LSE = 2 * DO, DR = LSE + Sh::BK * 4, STAGE = DR + Sh::BK * 4;
+    static constexpr uint32_t TOTAL = Sh::NS * STAGE;
+    // the epilogue's lift: [64][DD + 1] rows and W_down^T
+    static_assert(!LOCAL || 64 * (DD + 1) * 4 + DD * 64 * 4 <= TOTAL, "the lift fits in the stage area");
 };
 
-template <int DD>
-__global__ void __launch_bounds__(kTc, DD <= 32 ? 3 : 1) bwd_dkv_tc_kernel(Args a)
+template <int W, bool LOCAL, int DD>
+__global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dkv_tc_kernel(Args a)
 {
-    using Ly = DkvLayout<DD>;
-    constexpr int LD = Ly::LD, KSD = DD / 16, NTD = DD / 8;
+    using Sh = Shape<W, LOCAL>;
+    using Sm = DkvSmem<W, LOCAL, DD>;
+    constexpr int MT = Sh::MT, ROWS = Sh::ROWS, BK = Sh::BK, NS = Sh::NS, LD = ld_of<W>(), NT = W / 8;
     extern __shared__ __align__(128) unsigned char tsm[];
-    unsigned char *sm = tsm;
-    const uint32_t sb = smem_u32(sm);
-    const int N = a.N, w = a.w;
-    const int bg = blockIdx.y, b = bg / a.Hkv, g = bg % a.Hkv;
-    const int j0 = blockIdx.x * 64;
+    const uint32_t sb = smem_u32(tsm);
+    const int N = a.N, w = min(a.w, N);
+    const int heads = a.B * a.Hkv, bg = blockIdx.x % heads, b = bg / a.Hkv, g = bg % a.Hkv;
+    const int j0 = blockIdx.x / heads * ROWS;  // keys with the most queries first
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, grp = lane >> 2, tig = lane & 3;
-    const int nk = min(64, N - j0);
-    const size_t kvbase = ((size_t)b * a.Hkv + g) * N + j0;
-    const int wk0 = 16 * warp;
-    const int jr0 = j0 + wk0 + grp;  // this thread's keys: jr0 and jr0 + 8
-
-    stage_rows<64, kLdW>(sb + Ly::K, sm + Ly::K, static_cast<const bf16 *>(a.k) + kvbase * 64, nk, tid);
-    stage_rows<64, kLdW>(sb + Ly::V, sm + Ly::V, static_cast<const bf16 *>(a.v) + kvbase * 64, nk, tid);
-    stage_rows<DD, LD>(sb + Ly::KD, sm + Ly::KD, static_cast<const bf16 *>(a.kd) + kvbase * DD, nk, tid);
-    stage_rows<DD, LD>(sb + Ly::VD, sm + Ly::VD, static_cast<const bf16 *>(a.vd) + kvbase * DD, nk, tid);
-    cp_commit();
-
-    const int it0 = j0 / 64, ntq = (N + 63) / 64, per_head = ntq - it0, nvs = a.G * per_head;
-    auto stage_q = [&](int v, int st) {
-        const int h = g * a.G + v / per_head, i0 = (it0 + v % per_head) * 64, nv = min(64, N - i0);
-        const bool all_global = (i0 - (j0 + 63)) >= w, all_local = (i0 + 63 - j0) < w;
-        const size_t rowbase = ((size_t)b * a.Hq + h) * N + i0;
-        const uint32_t base = sb + Ly::STG + st * Ly::STAGE;
-        unsigned char *bp = sm + Ly::STG + st * Ly::STAGE;
-        if (!all_global) {
-            stage_rows<64, kLdW>(base + Ly::Q_OFF, bp + Ly::Q_OFF, static_cast<const bf16 *>(a.q) + rowbase * 64, nv,
-                                 tid);
-            stage_rows<64, kLdW>(base + Ly::DO_OFF, bp + Ly::DO_OFF, static_cast<const bf16 *>(a.dout) + rowbase * 64,
-                                 nv, tid);
+    const size_t kvbase = (size_t)bg * N;
+    // queries [ilo, ihi): local j <= i < j + w, global i >= j + w
+    const int j_last = min(N, j0 + ROWS) - 1;
+    const int ilo = LOCAL ? j0 : (w < N - j0 ? j0 + w : N);
+    const int ihi = LOCAL ? (w > 0 ? (w < N - j_last ? j_last + w : N) : j0) : N;
+    const int per_head = (ihi - ilo + BK - 1) / BK, ntiles = a.G * per_head;
+    auto stage = [&](int t) {
+        if (t < ntiles) {
+            const int i = ilo + (t % per_head) * BK, n = N - i;
+            const size_t row = ((size_t)b * a.Hq + g * a.G + t / per_head) * N + i;
+            const uint32_t dst = sb + (t % NS) * Sm::STAGE;
+            stage_rows<W, BK>(dst, (LOCAL ? static_cast<const bf16 *>(a.q) : a.qtb) + row * W, n, tid);
+            stage_rows<W, BK>(dst + Sm::DO, (LOCAL ? static_cast<const bf16 *>(a.dout) : a.dotb) + row * W, n, tid);
+            if (tid < BK) {
+                if (tid < n) {
+                    sm100::cp_async4(dst + Sm::LSE + tid * 4, a.lse + row + tid);
+                    sm100::cp_async4(dst + Sm::DR + tid * 4, a.drow + row + tid);
+                } else {  // past the end: weights 2^(-infinity) = 0
+                    float *f = reinterpret_cast<float *>(tsm + (t % NS) * Sm::STAGE);
+                    f[Sm::LSE / 4 + tid] = -INFINITY;
+                    f[Sm::DR / 4 + tid] = 0.f;
+                }
+            }
         }
-        if (!all_local) {
-            stage_rows<DD, LD>(base + Ly::QT_OFF, bp + Ly::QT_OFF, a.qtb + rowbase * DD, nv, tid);
-            stage_rows<DD, LD>(base + Ly::DOT_OFF, bp + Ly::DOT_OFF, a.dotb + rowbase * DD, nv, tid);
-        }
-        stage_vec(base + Ly::LSE_OFF, reinterpret_cast<float *>(bp + Ly::LSE_OFF), a.lse + rowbase, nv, tid);
-        stage_vec(base + Ly::DR_OFF, reinterpret_cast<float *>(bp + Ly::DR_OFF), a.drow + rowbase, nv, tid);
         cp_commit();
     };
-    if (nvs > 0)
-        stage_q(0, 0);
-    cp_wait<1>();  // the key-side rows
-    __syncthreads();
+    for (int t = 0; t < NS - 1; ++t)
+        stage(t);
 
-    // A fragments: the d_down-wide key rows stay in registers; the 64-wide k
-    // and v rows are read from shared memory by the steps with local pairs
-    uint32_t kda[KSD][4], vda[KSD][4];
+    const int r0 = j0 + 16 * MT * warp;  // this warp's keys r0 .. r0 + 16 MT - 1
+    uint32_t ka[MT][W / 16][4], va[MT][W / 16][4];
+    float dk[MT][NT][4], dv[MT][NT][4], zero[MT][2][4];
 #pragma unroll
-    for (int kk = 0; kk < KSD; ++kk) {
-        ldsm_x4(a_addr<LD>(sb + Ly::KD, wk0, kk, lane), kda[kk]);
-        ldsm_x4(a_addr<LD>(sb + Ly::VD, wk0, kk, lane), vda[kk]);
+    for (int mt = 0; mt < MT; ++mt) {
+        load_a<W>(ka[mt], static_cast<const bf16 *>(LOCAL ? a.k : a.kd) + kvbase * W, r0 + 16 * mt, N, lane);
+        load_a<W>(va[mt], static_cast<const bf16 *>(LOCAL ? a.v : a.vd) + kvbase * W, r0 + 16 * mt, N, lane);
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                dk[mt][n][e] = dv[mt][n][e] = 0.f;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                zero[mt][nt][e] = 0.f;
     }
-    float dk[8][4], dv[8][4], dkd[NTD][4], dvd[NTD][4];
-#pragma unroll
-    for (int n = 0; n < 8; ++n)
-        dk[n][0] = dk[n][1] = dk[n][2] = dk[n][3] = dv[n][0] = dv[n][1] = dv[n][2] = dv[n][3] = 0.f;
-#pragma unroll
-    for (int n = 0; n < NTD; ++n)
-        dkd[n][0] = dkd[n][1] = dkd[n][2] = dkd[n][3] = dvd[n][0] = dvd[n][1] = dvd[n][2] = dvd[n][3] = 0.f;
+    const float c2 = a.c2;
 
-    for (int v = 0; v < nvs; ++v) {
-        const int st = v & 1;
-        const int i0 = (it0 + v % per_head) * 64;
-        if (v + 1 < nvs) {
-            stage_q(v + 1, st ^ 1);
-            cp_wait<1>();
-        } else {
-            cp_wait<0>();
-        }
+    for (int t = 0; t < ntiles; ++t) {
+        cp_wait<NS - 2>();
         __syncthreads();
-        const bool all_global = (i0 - (j0 + 63)) >= w, all_local = (i0 + 63 - j0) < w;
-        // all pairs global, every key before every query, every key and query inside the sequence
-        const bool interior = all_global && j0 + 63 <= i0 && i0 + 63 < N;
-        const uint32_t stg = sb + Ly::STG + st * Ly::STAGE;
-        const float *lse_s = reinterpret_cast<const float *>(sm + Ly::STG + st * Ly::STAGE + Ly::LSE_OFF);
-        const float *dr_s = reinterpret_cast<const float *>(sm + Ly::STG + st * Ly::STAGE + Ly::DR_OFF);
+        stage(t + NS - 1);
+        const uint32_t qs = sb + (t % NS) * Sm::STAGE;
+        const float *lse_s = reinterpret_cast<const float *>(tsm + (t % NS) * Sm::STAGE + Sm::LSE);
+        const float *dr_s = reinterpret_cast<const float *>(tsm + (t % NS) * Sm::STAGE + Sm::DR);
+        const int it = ilo + (t % per_head) * BK;
 #pragma unroll 1
-        for (int qc = 0; qc < 4; ++qc) {
-            if (i0 + 16 * qc + 15 < j0 + wk0)
-                continue;  // every query of the step is before every key of this warp (causal)
-            float sl[2][4] = {}, sg[2][4] = {};
-            if (!all_global) {
+        for (int qc = 0; qc < BK / 16; ++qc) {
+            const int i = it + 16 * qc;
+            if (i >= N || (LOCAL && i >= r0 + 16 * MT - 1 + w))
+                break;
+            if (LOCAL ? i + 15 < r0 : i + 15 < r0 + w)
+                continue;
+            const bool all = LOCAL ? i >= r0 + 16 * MT - 1 && i + 15 < r0 + w : i >= r0 + 16 * MT - 1 + w;
+            const uint32_t qst = qs + 16 * qc * LD, dst = qst + Sm::DO;
+            float s[MT][2][4], dp[MT][2][4], nD[MT][2][4];
+            float2 nl[2];
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    uint32_t bfr[4], afr[4];
-                    ldsm_x4(a_addr<kLdW>(sb + Ly::K, wk0, kk, lane), afr);
-                    ldsm_x4(b_addr<kLdW>(stg + Ly::Q_OFF, 16 * qc, kk, lane), bfr);
-                    mma_bf16_16816(sl[0], afr, bfr[0], bfr[1]);
-                    mma_bf16_16816(sl[1], afr, bfr[2], bfr[3]);
+            for (int nt = 0; nt < 2; ++nt) {
+                const float2 d = *reinterpret_cast<const float2 *>(dr_s + 16 * qc + 8 * nt + 2 * tig);
+                nl[nt] = *reinterpret_cast<const float2 *>(lse_s + 16 * qc + 8 * nt + 2 * tig);
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    nD[mt][nt][0] = nD[mt][nt][2] = d.x;
+                    nD[mt][nt][1] = nD[mt][nt][3] = d.y;
                 }
             }
-            if (!all_local) {
+            scores<W, MT>(s, ka, qst + b_lane<LD>(lane), zero);
+            scores<W, MT>(dp, va, dst + b_lane<LD>(lane), nD);
+            if (!all) {
 #pragma unroll
-                for (int kk = 0; kk < KSD; ++kk) {
-                    uint32_t bfr[4];
-                    ldsm_x4(b_addr<LD>(stg + Ly::QT_OFF, 16 * qc, kk, lane), bfr);
-                    mma_bf16_16816(sg[0], kda[kk], bfr[0], bfr[1]);
-                    mma_bf16_16816(sg[1], kda[kk], bfr[2], bfr[3]);
-                }
+                for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                    for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int jj = r0 + 16 * mt + grp + 8 * (e >> 1), ii = i + 8 * nt + 2 * tig + (e & 1);
+                            const bool in = LOCAL ? jj <= ii && jj > ii - w : jj <= ii - w;
+                            s[mt][nt][e] = in ? s[mt][nt][e] : -INFINITY;
+                            dp[mt][nt][e] = in ? dp[mt][nt][e] : 0.f;
+                        }
             }
-            if (interior) {  // every pair of the step is valid and global: no masks, no local part
-                float dpg[2][4] = {};
+            uint32_t pa[MT][4], ds[MT][4];
 #pragma unroll
-                for (int kk = 0; kk < KSD; ++kk) {
-                    uint32_t bfr[4];
-                    ldsm_x4(b_addr<LD>(stg + Ly::DOT_OFF, 16 * qc, kk, lane), bfr);
-                    mma_bf16_16816(dpg[0], vda[kk], bfr[0], bfr[1]);
-                    mma_bf16_16816(dpg[1], vda[kk], bfr[2], bfr[3]);
-                }
-                float pg[2][4], dsg[2][4];
+            for (int mt = 0; mt < MT; ++mt) {
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int il = 16 * qc + 8 * nt + 2 * tig + (e & 1);
-                        pg[nt][e] = sm100::ex2_approx(fmaf(sg[nt][e], a.c2, -lse_s[il]));
-                        dsg[nt][e] = pg[nt][e] * (dpg[nt][e] - dr_s[il]);
+                    for (int hr = 0; hr < 2; ++hr) {
+                        float &p0 = s[mt][nt][2 * hr], &p1 = s[mt][nt][2 * hr + 1];
+                        ffma2(p0, p1, p0, p1, c2, c2, nl[nt].x, nl[nt].y);
+                        p0 = ex2_approx(p0);
+                        p1 = ex2_approx(p1);
+                        mul2(dp[mt][nt][2 * hr], dp[mt][nt][2 * hr + 1], p0, p1, dp[mt][nt][2 * hr],
+                             dp[mt][nt][2 * hr + 1]);
                     }
-                uint32_t ap[4], ad[4];
-                frag_a(ap, pg[0], pg[1]);
-                frag_a(ad, dsg[0], dsg[1]);
-#pragma unroll
-                for (int n0 = 0; n0 < DD; n0 += 16) {
-                    uint32_t bfr[4];
-                    ldsm_x4_t(bt_addr<LD>(stg + Ly::DOT_OFF, 16 * qc, n0, lane), bfr);
-                    mma_bf16_16816(dvd[n0 / 8], ap, bfr[0], bfr[1]);
-                    mma_bf16_16816(dvd[n0 / 8 + 1], ap, bfr[2], bfr[3]);
-                    ldsm_x4_t(bt_addr<LD>(stg + Ly::QT_OFF, 16 * qc, n0, lane), bfr);
-                    mma_bf16_16816(dkd[n0 / 8], ad, bfr[0], bfr[1]);
-                    mma_bf16_16816(dkd[n0 / 8 + 1], ad, bfr[2], bfr[3]);
-                }
-                continue;
+                frag_a(pa[mt], s[mt][0], s[mt][1]);
+                frag_a(ds[mt], dp[mt][0], dp[mt][1]);
             }
-            float dpl[2][4] = {}, dpg[2][4] = {};
-            if (!all_global) {
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    uint32_t bfr[4], afr[4];
-                    ldsm_x4(a_addr<kLdW>(sb + Ly::V, wk0, kk, lane), afr);
-                    ldsm_x4(b_addr<kLdW>(stg + Ly::DO_OFF, 16 * qc, kk, lane), bfr);
-                    mma_bf16_16816(dpl[0], afr, bfr[0], bfr[1]);
-                    mma_bf16_16816(dpl[1], afr, bfr[2], bfr[3]);
-                }
-            }
-            if (!all_local) {
-#pragma unroll
-                for (int kk = 0; kk < KSD; ++kk) {
-                    uint32_t bfr[4];
-                    ldsm_x4(b_addr<LD>(stg + Ly::DOT_OFF, 16 * qc, kk, lane), bfr);
-                    mma_bf16_16816(dpg[0], vda[kk], bfr[0], bfr[1]);
-                    mma_bf16_16816(dpg[1], vda[kk], bfr[2], bfr[3]);
-                }
-            }
-            float pl[2][4], dsl[2][4], pg[2][4], dsg[2][4];
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int j = jr0 + 8 * (e >> 1), il = 16 * qc + 8 * nt + 2 * tig + (e & 1), i = i0 + il;
-                    const bool loc = i - j < w;
-                    float p = 0.f, ds = 0.f;
-                    if (j < N && i < N && j <= i) {
-                        p = sm100::ex2_approx((loc ? sl[nt][e] : sg[nt][e]) * a.c2 - lse_s[il]);
-                        ds = p * ((loc ? dpl[nt][e] : dpg[nt][e]) - dr_s[il]);
-                    }
-                    pl[nt][e] = loc ? p : 0.f;
-                    dsl[nt][e] = loc ? ds : 0.f;
-                    pg[nt][e] = loc ? 0.f : p;
-                    dsg[nt][e] = loc ? 0.f : ds;
-                }
-            if (!all_global) {
-                uint32_t ap[4], ad[4];
-                frag_a(ap, pl[0], pl[1]);
-                frag_a(ad, dsl[0], dsl[1]);
-#pragma unroll
-                for (int n0 = 0; n0 < 64; n0 += 16) {
-                    uint32_t bfr[4];
-                    ldsm_x4_t(bt_addr<kLdW>(stg + Ly::DO_OFF, 16 * qc, n0, lane), bfr);
-                    mma_bf16_16816(dv[n0 / 8], ap, bfr[0], bfr[1]);
-                    mma_bf16_16816(dv[n0 / 8 + 1], ap, bfr[2], bfr[3]);
-                    ldsm_x4_t(bt_addr<kLdW>(stg + Ly::Q_OFF, 16 * qc, n0, lane), bfr);
-                    mma_bf16_16816(dk[n0 / 8], ad, bfr[0], bfr[1]);
-                    mma_bf16_16816(dk[n0 / 8 + 1], ad, bfr[2], bfr[3]);
-                }
-            }
-            if (!all_local) {
-                uint32_t ap[4], ad[4];
-                frag_a(ap, pg[0], pg[1]);
-                frag_a(ad, dsg[0], dsg[1]);
-#pragma unroll
-                for (int n0 = 0; n0 < DD; n0 += 16) {
-                    uint32_t bfr[4];
-                    ldsm_x4_t(bt_addr<LD>(stg + Ly::DOT_OFF, 16 * qc, n0, lane), bfr);
-                    mma_bf16_16816(dvd[n0 / 8], ap, bfr[0], bfr[1]);
-                    mma_bf16_16816(dvd[n0 / 8 + 1], ap, bfr[2], bfr[3]);
-                    ldsm_x4_t(bt_addr<LD>(stg + Ly::QT_OFF, 16 * qc, n0, lane), bfr);
-                    mma_bf16_16816(dkd[n0 / 8], ad, bfr[0], bfr[1]);
-                    mma_bf16_16816(dkd[n0 / 8 + 1], ad, bfr[2], bfr[3]);
-                }
-            }
+            accumulate<W, MT>(dv, pa, dst + bt_lane<LD>(lane));
+            accumulate<W, MT>(dk, ds, qst + bt_lane<LD>(lane));
         }
-        __syncthreads();  // stage st is free for the copy issued in the next step
     }
-    cp_wait<0>();
-    __syncthreads();
 
-    // epilogue: dk = scale dk_loc + dk^D Dk^T (dk^D = scale sum dS q~), dv = dv_loc + dv^D Dv^T
-    float *lk = reinterpret_cast<float *>(sm + Ly::STG);  // [64][DD + 1] dk^D, then dv^D
-    float *lv = lk + 64 * (DD + 1);
+    if constexpr (!LOCAL) {
 #pragma unroll
-    for (int n = 0; n < NTD; ++n)
+        for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int idx = (wk0 + grp + 8 * (e >> 1)) * (DD + 1) + 8 * n + 2 * tig + (e & 1);
-            lk[idx] = dkd[n][e] * a.scale;
-            lv[idx] = dvd[n][e];
-        }
-    __syncwarp();
-    const float *Dk = a.Dk + (size_t)g * 64 * DD, *Dv = a.Dv + (size_t)g * 64 * DD;
+            for (int hr = 0; hr < 2; ++hr) {
+                const int j = r0 + 16 * mt + grp + 8 * hr;
+                if (j >= N)
+                    continue;
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const int kr = wk0 + grp + 8 * r;
-        if (j0 + kr >= N)
-            continue;
-        const size_t row = kvbase + kr;
-        bf16 *dkr = static_cast<bf16 *>(a.dk) + row * 64;
-        bf16 *dvr = static_cast<bf16 *>(a.dv) + row * 64;
-#pragma unroll
-        for (int n = 0; n < 8; ++n) {
-            const int t = 8 * n + 2 * tig;
-            float k0 = dk[n][2 * r] * a.scale, k1 = dk[n][2 * r + 1] * a.scale;
-            float v0 = dv[n][2 * r], v1 = dv[n][2 * r + 1];
-            for (int c = 0; c < DD; ++c) {
-                const float xk = lk[kr * (DD + 1) + c], xv = lv[kr * (DD + 1) + c];
-                k0 = fmaf(xk, __ldg(Dk + t * DD + c), k0);
-                k1 = fmaf(xk, __ldg(Dk + (t + 1) * DD + c), k1);
-                v0 = fmaf(xv, __ldg(Dv + t * DD + c), v0);
-                v1 = fmaf(xv, __ldg(Dv + (t + 1) * DD + c), v1);
+                for (int n = 0; n < NT; ++n) {
+                    const size_t at = (kvbase + j) * W + 8 * n + 2 * tig;
+                    *reinterpret_cast<float2 *>(a.dkd + at) =
+                        make_float2(dk[mt][n][2 * hr] * a.scale, dk[mt][n][2 * hr + 1] * a.scale);
+                    *reinterpret_cast<float2 *>(a.dvd + at) = make_float2(dv[mt][n][2 * hr], dv[mt][n][2 * hr + 1]);
+                }
             }
-            *reinterpret_cast<uint32_t *>(dkr + t) = cvt_bf16x2(k0, k1);
-            *reinterpret_cast<uint32_t *>(dvr + t) = cvt_bf16x2(v0, v1);
-        }
+    } else {
+        static_assert(!LOCAL || MT == 1, "the lift stages 64 rows");
+        // dk = scale dk_loc + dk^D Dk^T, dv = dv_loc + dv^D Dv^T, one after the other
+        float *lift = reinterpret_cast<float *>(tsm);  // [64][DD + 1]
+        float *wt = lift + 64 * (DD + 1);              // [DD][64] W_down^T
+        const int nv = min(ROWS, N - j0);
 #pragma unroll
-        for (int n = 0; n < NTD; ++n) {
-            const int c = 8 * n + 2 * tig;
-            *reinterpret_cast<float2 *>(a.dkd + row * DD + c) =
-                make_float2(dkd[n][2 * r] * a.scale, dkd[n][2 * r + 1] * a.scale);
-            *reinterpret_cast<float2 *>(a.dvd + row * DD + c) = make_float2(dvd[n][2 * r], dvd[n][2 * r + 1]);
+        for (int kv = 0; kv < 2; ++kv) {
+            cp_wait<0>();
+            __syncthreads();  // the stage area (or the other lift) is idle
+            const float *Wd = (kv ? a.Dv : a.Dk) + (size_t)g * 64 * DD;
+            const float *x = (kv ? a.dvd : a.dkd) + (kvbase + j0) * DD;
+            for (int e = tid; e < 64 * DD; e += kTc)
+                wt[(e % DD) * 64 + e / DD] = __ldg(Wd + e);
+            for (int e = tid; e < nv * DD; e += kTc)
+                lift[(e / DD) * (DD + 1) + e % DD] = x[e];
+            __syncthreads();
+#pragma unroll
+            for (int hr = 0; hr < 2; ++hr) {
+                const int j = r0 + grp + 8 * hr;
+                if (j >= N)
+                    continue;
+                float o[8][2];
+#pragma unroll
+                for (int n = 0; n < 8; ++n) {
+                    o[n][0] = kv ? dv[0][n][2 * hr] : dk[0][n][2 * hr] * a.scale;
+                    o[n][1] = kv ? dv[0][n][2 * hr + 1] : dk[0][n][2 * hr + 1] * a.scale;
+                }
+                lift16<DD>(o, lift + (j - j0) * (DD + 1), wt, tig);
+                bf16 *dst = static_cast<bf16 *>(kv ? a.dv : a.dk) + (kvbase + j) * 64;
+#pragma unroll
+                for (int n = 0; n < 8; ++n)
+                    *reinterpret_cast<uint32_t *>(dst + 8 * n + 2 * tig) = cvt_bf16x2(o[n][0], o[n][1]);
+            }
         }
     }
 }
 
+// ---------------------------------------------------------------- rows
+
+// Per query row, tile by tile as the Eq. 1 kernel: blockIdx.z = 0: q~ = q Uk^T;
+// 1: dO~ = dO Uv^T and -D = -dO . o.
+template <int DD>
+__global__ void __launch_bounds__(rows_bulk<bf16>() / rows_per_thread<DD>() *slices<DD>()) bwd_rows_tc_kernel(Args a)
+{
+    constexpr int R = rows_bulk<bf16>(), NR = R / rows_per_thread<DD>(), NTH = NR * slices<DD>(), CW = cols_per_thread<DD>();
+    __shared__ __align__(16) unsigned char rows[kStageBytesBulk];
+    __shared__ __align__(16) float Ws[64 * DD];
+    const bool z = blockIdx.z != 0;
+    const int tid = threadIdx.x, bh = blockIdx.y, g = bh % a.Hq / a.G, i0 = blockIdx.x * R;
+    const int nr = min(R, a.N - i0);
+    const size_t row0 = (size_t)bh * a.N + i0;
+    stage_tile(rows, static_cast<const bf16 *>(z ? a.dout : a.q) + row0 * 64, nr, tid, NTH);
+    const float *U = (z ? a.Uv : a.Uk) + (size_t)g * DD * 64;
+    for (int e = tid; e < 64 * DD; e += NTH)
+        Ws[(e % 64) * DD + e / 64] = __ldg(U + e);
+    sm100::cp_async_wait_all();
+    __syncthreads();
+    if (z) {  // eight lanes per row
+        const uint4 *o = reinterpret_cast<const uint4 *>(static_cast<const bf16 *>(a.out) + row0 * 64);
+#pragma unroll 4
+        for (int e = tid; e < R * 8; e += NTH) {
+            const int r = e / 8, c = e % 8;
+            float x[8], y[8], s = 0.f;
+            unpack(reinterpret_cast<const uint4 *>(rows)[r * 8 + (c ^ (r & 7))], x, bf16());
+            unpack(r < nr ? __ldg(o + e) : make_uint4(0u, 0u, 0u, 0u), y, bf16());
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                s = fmaf(x[k], y[k], s);
+#pragma unroll
+            for (int k = 1; k < 8; k <<= 1)
+                s += __shfl_xor_sync(0xffffffffu, s, k);
+            if (c == 0 && r < nr)
+                a.drow[row0 + r] = -s;
+        }
+    }
+    const int r0 = tid % NR, c0 = slices<DD>() > 1 ? tid / NR * CW : 0;
+    float acc[rows_per_thread<DD>()][CW];
+    project_rows<bf16, DD, CW, rows_per_thread<DD>()>(rows, Ws + c0, r0, NR, acc);
+    bf16 *dst = (z ? a.dotb : a.qtb) + row0 * DD + c0;
+#pragma unroll
+    for (int k = 0; k < rows_per_thread<DD>(); ++k)
+        if (r0 + k * NR < nr)
+            store_row<bf16, CW>(dst + (size_t)(r0 + k * NR) * DD, acc[k]);
+}
+
 // ---------------------------------------------------------------- host side
+
+template <typename K>
+static cudaError_t opt_in(K kern, size_t smem)
+{
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)  // several CTAs per SM need the largest shared-memory carve-out
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+    return e;
+}
 
 template <int DD>
 static cudaError_t run_tc(const Args &a, cudaStream_t s)
 {
-    const size_t smq = DqLayout<DD>::TOTAL, smk = DkvLayout<DD>::TOTAL;
+    auto dq_g = bwd_dq_tc_kernel<DD, false, DD>;
+    auto dq_l = bwd_dq_tc_kernel<64, true, DD>;
+    auto dkv_g = bwd_dkv_tc_kernel<DD, false, DD>;
+    auto dkv_l = bwd_dkv_tc_kernel<64, true, DD>;
+    constexpr size_t sq_g = DqSmem<DD, false, DD>::TOTAL, sq_l = DqSmem<64, true, DD>::TOTAL;
+    constexpr size_t sk_g = DkvSmem<DD, false, DD>::TOTAL, sk_l = DkvSmem<64, true, DD>::TOTAL;
     static PerDeviceOnce once;
     cudaError_t e = per_device_once(once, [&](int) {
-        cudaError_t e2 = cudaFuncSetAttribute(bwd_dq_tc_kernel<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)smq);
+        cudaError_t e2 = opt_in(dq_g, sq_g);
         if (e2 == cudaSuccess)
-            e2 = cudaFuncSetAttribute(bwd_dkv_tc_kernel<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smk);
+            e2 = opt_in(dq_l, sq_l);
+        if (e2 == cudaSuccess)
+            e2 = opt_in(dkv_g, sk_g);
+        if (e2 == cudaSuccess)
+            e2 = opt_in(dkv_l, sk_l);
         return e2;
     });
     if (e != cudaSuccess)
         return e;
-    bwd_rows_kernel<bf16, DD><<<rows_grid(a), 256, 0, s>>>(a);
-    const int tiles = (a.N + 63) / 64;
-    bwd_dq_tc_kernel<DD><<<dim3(tiles, a.B * a.Hq), kTc, smq, s>>>(a);
-    bwd_dkv_tc_kernel<DD><<<dim3(tiles, a.B * a.Hkv), kTc, smk, s>>>(a);
+    constexpr int R = rows_bulk<bf16>();
+    bwd_rows_tc_kernel<DD><<<dim3((a.N + R - 1) / R, a.B * a.Hq, 2), R / rows_per_thread<DD>() * slices<DD>(), 0, s>>>(a);
+    constexpr int RG = Shape<DD, false>::ROWS, RL = Shape<64, true>::ROWS;
+    const unsigned tg = (a.N + RG - 1) / RG, tl = (a.N + RL - 1) / RL;
+    dq_g<<<a.B * a.Hq * tg, kTc, sq_g, s>>>(a);
+    dq_l<<<a.B * a.Hq * tl, kTc, sq_l, s>>>(a);
+    dkv_g<<<a.B * a.Hkv * tg, kTc, sk_g, s>>>(a);
+    dkv_l<<<a.B * a.Hkv * tl, kTc, sk_l, s>>>(a);
     return run_weights<bf16, DD>(a, s);
 }
 

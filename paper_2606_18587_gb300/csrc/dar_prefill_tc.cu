@@ -127,13 +127,6 @@ struct Layout {
     static_assert(VD_OFF + BN * vd_row<DP>() * 2 <= STAGE, "a stage holds either part");
 };
 
-__device__ __forceinline__ float max3(float a, float b, float c)
-{
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
