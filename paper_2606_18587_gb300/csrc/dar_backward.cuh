@@ -504,19 +504,16 @@ __global__ void __launch_bounds__(kThreads) bwd_dkv_kernel(Args a)
 //         1: X = q, Y = dq~  (rows of (b, h in g)) -> dUk (transposed at the end)
 //         2: X = v, Y = dv^D                       -> dDv
 //         3: X = dO, Y = O^D                       -> dUv (transposed)
-// (with a.fac, Y of 1 and 3 times the row's factor).
 //
 // A thread holds a 4 x 4 block of outputs, so two 16-byte shared-memory reads
 // feed 16 products; 64 / DD groups of threads share out the rows of a stage and
-// are added up in group order at the end.  Stages of 32 rows arrive by cp.async,
-// several deep: the sums then run near the rate at which X and Y (0.8 GB for
-// B8 H16 N8192, d_down 16) come from memory.  With one output per thread and
-// row (two reads per product) and unbuffered stages that shape took 1743 us.
+// are added up in group order at the end; stages of 32 rows arrive by cp.async,
+// several deep.
 constexpr int kWRows = 32;
 
 template <typename T, int DD>
 struct WpartSmem {
-    static constexpr int X = kWRows * kHeadDim * (int)sizeof(T), Y = X + kWRows * DD * 4, STAGE = Y + kWRows * 4;
+    static constexpr int X = kWRows * kHeadDim * (int)sizeof(T), STAGE = X + kWRows * DD * 4;
     static constexpr int NS = STAGE * 4 <= 48 << 10 ? 4 : 2;
     static constexpr int RED = kThreads * 16 * 4;
     static constexpr int TOTAL = NS * STAGE > RED ? NS * STAGE : RED;
@@ -533,7 +530,6 @@ __global__ void __launch_bounds__(kThreads) bwd_wpart_kernel(Args a)
     const uint32_t sb = sm100::smem_u32(sm);
     const int tid = threadIdx.x, chunk = blockIdx.x, g = blockIdx.y, which = blockIdx.z;
     const bool per_kv = which == 0 || which == 2;
-    const bool scaled = !per_kv && a.fac != nullptr;
     const int heads = per_kv ? 1 : a.G;  // of KV head g, per batch element
     const long nrows = (long)a.B * heads * a.N;
     const long r0 = nrows * chunk / kChunks, r1 = nrows * (chunk + 1) / kChunks;
@@ -565,8 +561,6 @@ __global__ void __launch_bounds__(kThreads) bwd_wpart_kernel(Args a)
                 sm100::cp_async16(d + e * 16, X + row_of(e / XC) * kHeadDim + e % XC * (16 / (int)sizeof(T)));
             for (int e = tid; e < n * YC; e += kThreads)
                 sm100::cp_async16(d + Sm::X + e * 16, Y + row_of(e / YC) * DD + e % YC * 4);
-            if (scaled && tid < n)
-                sm100::cp_async4(d + Sm::Y + tid * 4, a.fac + row_of(tid));
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -582,7 +576,6 @@ __global__ void __launch_bounds__(kThreads) bwd_wpart_kernel(Args a)
         __syncthreads();
         stage(t + NS - 1);
         const unsigned char *st = sm + (t % NS) * Sm::STAGE;
-        const float *fac = reinterpret_cast<const float *>(st + Sm::Y);
         const int n = (int)min((long)kWRows, r1 - r0 - (long)t * kWRows);
 #pragma unroll 4
         for (int r = grp; r < n; r += NG) {
@@ -600,11 +593,7 @@ __global__ void __launch_bounds__(kThreads) bwd_wpart_kernel(Args a)
                 x[2] = v.z;
                 x[3] = v.w;
             }
-            float4 y = *reinterpret_cast<const float4 *>(st + Sm::X + (r * DD + c0) * 4);
-            if (scaled) {
-                const float f = fac[r];
-                y = make_float4(y.x * f, y.y * f, y.z * f, y.w * f);
-            }
+            const float4 y = *reinterpret_cast<const float4 *>(st + Sm::X + (r * DD + c0) * 4);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 sm100::ffma2(acc[e][0], acc[e][1], x[e], x[e], y.x, y.y, acc[e][0], acc[e][1]);

@@ -1,6 +1,5 @@
 // dar_backward_tc.cu -- the backward pass for bf16 storage on the tensor
-// cores (mma.sync m16n8k16: bf16 operands, fp32 accumulators), with the
-// projection-gradient kernels of dar_backward.cuh.
+// cores (mma.sync m16n8k16: bf16 operands, fp32 accumulators).
 //
 // The gradients of dar_backward.cuh as FlashAttention-style recomputation with
 // the local (full-width) and the global (d_down-wide) pairs in kernels of
@@ -105,20 +104,19 @@ __device__ __forceinline__ uint32_t bt_lane(int lane)
     return ((lane & 7) + (((lane >> 3) & 1) << 3)) * LD + (lane >> 4) * 16;
 }
 
-// A fragments of 16 rows (row0 + lane group, + 8) of a row-major [*][W] bf16
-// matrix, straight from global memory; rows at or past n are zero.
-template <int W>
-__device__ __forceinline__ void load_a(uint32_t (&f)[W / 16][4], const bf16 *src, int row0, int n, int lane)
+// Lane offset for ldmatrix of an A operand: 16 rows, first 16 columns.
+template <int LD>
+__device__ __forceinline__ uint32_t a_lane(int lane)
 {
-    const int grp = lane >> 2, tig = lane & 3;
+    return (lane & 15) * LD + (lane >> 4) * 16;
+}
+// A fragments of 16 rows of a padded W-wide tile.
+template <int W>
+__device__ __forceinline__ void load_a(uint32_t (&f)[W / 16][4], uint32_t rows, int lane)
+{
 #pragma unroll
     for (int kk = 0; kk < W / 16; ++kk)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int r = row0 + grp + 8 * (e & 1);
-            f[kk][e] = r < n ? __ldg(reinterpret_cast<const uint32_t *>(src + (size_t)r * W + 16 * kk + 8 * (e >> 1) + 2 * tig))
-                             : 0u;
-        }
+        ldsm_x4(rows + a_lane<ld_of<W>()>(lane) + kk * 32, f[kk]);
 }
 
 // C (+)= A B^T over W columns: A fragments of MT row tiles, B the 16 rows whose
@@ -160,20 +158,23 @@ __device__ __forceinline__ void accumulate(float (&acc)[MT][W / 8][4], const uin
     }
 }
 
-// out[2] (columns t, t + 1 of a row) += sum_c x[c] M[c][t], M fp32 rows of 64 in shared memory.
-template <int DD>
-__device__ __forceinline__ void lift16(float (&o)[8][2], const float *x, const float *M, int tig)
+// o[r][n] (columns 8n + 2 tig, + 1 of two rows) += sum_c x_r[c] M[c][t], fp32:
+// M in shared memory with row stride LS floats.
+template <int DD, int LS>
+__device__ __forceinline__ void lift_rows(float (&o)[2][8][2], const float *x0, const float *x1, const float *M, int tig)
 {
-#pragma unroll 4
+#pragma unroll 2
     for (int c = 0; c < DD; ++c) {
-        const float xv = x[c];
+        const float a0 = x0[c], a1 = x1[c];
 #pragma unroll
         for (int n = 0; n < 8; ++n) {
-            const float2 m = *reinterpret_cast<const float2 *>(M + c * 64 + 8 * n + 2 * tig);
-            ffma2(o[n][0], o[n][1], xv, xv, m.x, m.y, o[n][0], o[n][1]);
+            const float2 m = *reinterpret_cast<const float2 *>(M + c * LS + 8 * n + 2 * tig);
+            ffma2(o[0][n][0], o[0][n][1], a0, a0, m.x, m.y, o[0][n][0], o[0][n][1]);
+            ffma2(o[1][n][0], o[1][n][1], a1, a1, m.x, m.y, o[1][n][0], o[1][n][1]);
         }
     }
 }
+constexpr int kLiftLd = 66;  // row stride of a transposed W_down: its column-wise stores fall in distinct banks
 
 // Row tiles per warp and rows of the streamed tile per stage.
 template <int W, bool LOCAL>
@@ -182,7 +183,9 @@ struct Shape {
     static constexpr int ROWS = 64 * MT;                   // rows of a CTA's tile
     static constexpr int BK = !LOCAL && W <= 32 ? 128 : 64;  // streamed rows per stage
     static constexpr int NS = 3;
-    static constexpr int MINB = W == 16 ? 3 : W == 32 ? 2 : LOCAL ? 3 : 2;
+    static constexpr int MINB = W == 16 ? 4 : W == 32 ? 2 : LOCAL ? 3 : 2;
+    // a stage also takes the CTA's own rows, whose A fragments are read before it is needed
+    static_assert(ROWS <= BK, "the CTA's tile fits in a stage");
 };
 
 // ---------------------------------------------------------------- dq
@@ -226,21 +229,36 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
         }
         cp_commit();
     };
+    // this CTA's rows into the last stage, then the first tiles
+    stage_rows<W, ROWS>(sb + (NS - 1) * Sm::STAGE,
+                        (LOCAL ? static_cast<const bf16 *>(a.q) : a.qtb) + (headrow + i0) * W, N - i0, tid);
+    stage_rows<W, ROWS>(sb + (NS - 1) * Sm::STAGE + Sm::V,
+                        (LOCAL ? static_cast<const bf16 *>(a.dout) : a.dotb) + (headrow + i0) * W, N - i0, tid);
+    cp_commit();
     for (int t = 0; t < NS - 1; ++t)
         stage(t);
 
     const int r0 = i0 + 16 * MT * warp;  // this warp's rows r0 .. r0 + 16 MT - 1
     uint32_t qa[MT][W / 16][4], da[MT][W / 16][4];
     float nD[MT][2][4], zero[MT][2][4];
-    float m[MT][2], l[MT][2][2];
+    float m[MT][2], l[MT][2][2], drow[MT][2];
 #pragma unroll
-    for (int mt = 0; mt < MT; ++mt) {
-        load_a<W>(qa[mt], (LOCAL ? static_cast<const bf16 *>(a.q) : a.qtb) + headrow * W, r0 + 16 * mt, N, lane);
-        load_a<W>(da[mt], (LOCAL ? static_cast<const bf16 *>(a.dout) : a.dotb) + headrow * W, r0 + 16 * mt, N, lane);
+    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
         for (int hr = 0; hr < 2; ++hr) {
             const int i = r0 + 16 * mt + grp + 8 * hr;
-            const float d = i < N ? a.drow[headrow + i] : 0.f;
+            drow[mt][hr] = i < N ? a.drow[headrow + i] : 0.f;
+        }
+    cp_wait<NS - 1>();
+    __syncthreads();
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) {
+        const uint32_t own = sb + (NS - 1) * Sm::STAGE + 16 * (MT * warp + mt) * LD;
+        load_a<W>(qa[mt], own, lane);
+        load_a<W>(da[mt], own + Sm::V, lane);
+#pragma unroll
+        for (int hr = 0; hr < 2; ++hr) {
+            const float d = drow[mt][hr];
 #pragma unroll
             for (int nt = 0; nt < 2; ++nt) {
                 nD[mt][nt][2 * hr] = nD[mt][nt][2 * hr + 1] = d;
@@ -290,7 +308,7 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
                 }
             }
     };
-    auto exponents = [&](const float (&s)[MT][2][4], float (&y)[MT][2][4]) {
+    auto exponents = [&](float (&s)[MT][2][4]) {
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
@@ -298,7 +316,7 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
                 const float nm = m[mt][hr] == -INFINITY ? 0.f : -m[mt][hr];
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt)
-                    ffma2(y[mt][nt][2 * hr], y[mt][nt][2 * hr + 1], s[mt][nt][2 * hr], s[mt][nt][2 * hr + 1], c2, c2,
+                    ffma2(s[mt][nt][2 * hr], s[mt][nt][2 * hr + 1], s[mt][nt][2 * hr], s[mt][nt][2 * hr + 1], c2, c2,
                           nm, nm);
             }
     };
@@ -321,8 +339,44 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
             // 0 * infinity arises from a key the row does not see)
             const bool all = LOCAL ? j + 15 <= r0 && j > r0 + 16 * MT - 1 - w : j + 15 <= r0 - w;
             const uint32_t kst = ks + 16 * kc * LD, vst = kst + Sm::V;
-            float s[MT][2][4], dp[MT][2][4], y[MT][2][4];
-            scores<W, MT>(s, qa, kst + b_lane<LD>(lane), zero);
+            float s[MT][2][4], dp[MT][2][4];
+            auto in_kind = [&](int mt, int nt, int e) {
+                const int i = r0 + 16 * mt + grp + 8 * (e >> 1), jj = j + 8 * nt + 2 * tig + (e & 1);
+                return LOCAL ? jj <= i && jj > i - w : jj <= i - w;
+            };
+            auto masked_scores = [&]() {
+                scores<W, MT>(s, qa, kst + b_lane<LD>(lane), zero);
+                if (!all) {
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                s[mt][nt][e] = in_kind(mt, nt, e) ? s[mt][nt][e] : -INFINITY;
+                }
+            };
+            masked_scores();
+            exponents(s);
+            float top = -INFINITY;
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt) {
+                    top = sm100::max3(top, s[mt][nt][0], s[mt][nt][1]);
+                    top = sm100::max3(top, s[mt][nt][2], s[mt][nt][3]);
+                }
+            if (__builtin_expect(__any_sync(0xffffffffu, top > kRaise) || fresh, 0)) {
+                // rare: the scores again (they were overwritten), then larger maxima
+                masked_scores();
+                raise(s);
+                exponents(s);
+                bool none = false;  // once no maximum is -infinity, every row has seen a key
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt)
+                    none = none || m[mt][0] == -INFINITY || m[mt][1] == -INFINITY;
+                fresh = __any_sync(0xffffffffu, none);
+            }
             scores<W, MT>(dp, da, vst + b_lane<LD>(lane), nD);
             if (!all) {
 #pragma unroll
@@ -330,30 +384,8 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
 #pragma unroll
                     for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int i = r0 + 16 * mt + grp + 8 * (e >> 1), jj = j + 8 * nt + 2 * tig + (e & 1);
-                            const bool in = LOCAL ? jj <= i && jj > i - w : jj <= i - w;
-                            s[mt][nt][e] = in ? s[mt][nt][e] : -INFINITY;
-                            dp[mt][nt][e] = in ? dp[mt][nt][e] : 0.f;
-                        }
-            }
-            exponents(s, y);
-            float top = -INFINITY;
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt) {
-                    top = sm100::max3(top, y[mt][nt][0], y[mt][nt][1]);
-                    top = sm100::max3(top, y[mt][nt][2], y[mt][nt][3]);
-                }
-            if (__any_sync(0xffffffffu, top > kRaise) || fresh) {
-                raise(s);
-                exponents(s, y);
-                bool none = false;  // every row has seen a key from here on, once no maximum is -infinity
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt)
-                    none = none || m[mt][0] == -INFINITY || m[mt][1] == -INFINITY;
-                fresh = __any_sync(0xffffffffu, none);
+                        for (int e = 0; e < 4; ++e)
+                            dp[mt][nt][e] = in_kind(mt, nt, e) ? dp[mt][nt][e] : 0.f;
             }
             uint32_t ds[MT][4], pa[MT][4];
 #pragma unroll
@@ -362,7 +394,7 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
                 for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
                     for (int hr = 0; hr < 2; ++hr) {
-                        float &p0 = y[mt][nt][2 * hr], &p1 = y[mt][nt][2 * hr + 1];
+                        float &p0 = s[mt][nt][2 * hr], &p1 = s[mt][nt][2 * hr + 1];
                         p0 = ex2_approx(p0);
                         p1 = ex2_approx(p1);
                         add2(l[mt][hr][0], l[mt][hr][1], p0, p1, l[mt][hr][0], l[mt][hr][1]);
@@ -371,7 +403,7 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
                     }
                 frag_a(ds[mt], dp[mt][0], dp[mt][1]);
                 if constexpr (!LOCAL)
-                    frag_a(pa[mt], y[mt][0], y[mt][1]);
+                    frag_a(pa[mt], s[mt][0], s[mt][1]);
             }
             accumulate<W, MT>(dq, ds, kst + bt_lane<LD>(lane));
             if constexpr (!LOCAL)
@@ -424,6 +456,12 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
         for (int e = tid; e < nv * DD; e += kTc)
             lift[(e / DD) * (DD + 1) + e % DD] = a.dqt[(headrow + i0) * DD + e];
         __syncthreads();
+        float o[2][8][2];
+#pragma unroll
+        for (int n = 0; n < 8; ++n)
+            o[0][n][0] = o[0][n][1] = o[1][n][0] = o[1][n][1] = 0.f;
+        const float *x = lift + (16 * warp + grp) * (DD + 1);  // (rows past the end lift stale bytes and are not stored)
+        lift_rows<DD, 64>(o, x, x + 8 * (DD + 1), uk, tig);
 #pragma unroll
         for (int hr = 0; hr < 2; ++hr) {
             const int i = r0 + grp + 8 * hr;
@@ -440,16 +478,11 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
                 a.lse[row] = -lse;
                 a.fac[row] = fg;
             }
-            float o[8][2];
-#pragma unroll
-            for (int n = 0; n < 8; ++n)
-                o[n][0] = o[n][1] = 0.f;
-            lift16<DD>(o, lift + (i - i0) * (DD + 1), uk, tig);
             bf16 *dst = static_cast<bf16 *>(a.dq) + row * 64;
 #pragma unroll
             for (int n = 0; n < 8; ++n)
-                *reinterpret_cast<uint32_t *>(dst + 8 * n + 2 * tig) =
-                    cvt_bf16x2(fmaf(dq[0][n][2 * hr], fl, o[n][0] * fg), fmaf(dq[0][n][2 * hr + 1], fl, o[n][1] * fg));
+                *reinterpret_cast<uint32_t *>(dst + 8 * n + 2 * tig) = cvt_bf16x2(
+                    fmaf(dq[0][n][2 * hr], fl, o[hr][n][0] * fg), fmaf(dq[0][n][2 * hr + 1], fl, o[hr][n][1] * fg));
         }
     }
 }
@@ -463,7 +496,7 @@ struct DkvSmem {
     static constexpr uint32_t LSE = 2 * DO, DR = LSE + Sh::BK * 4, STAGE = DR + Sh::BK * 4;
     static constexpr uint32_t TOTAL = Sh::NS * STAGE;
     // the epilogue's lift: [64][DD + 1] rows and W_down^T
-    static_assert(!LOCAL || 64 * (DD + 1) * 4 + DD * 64 * 4 <= TOTAL, "the lift fits in the stage area");
+    static_assert(!LOCAL || 64 * (DD + 1) * 4 + DD * kLiftLd * 4 <= TOTAL, "the lift fits in the stage area");
 };
 
 template <int W, bool LOCAL, int DD>
@@ -504,16 +537,25 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dkv_tc_kernel(
         }
         cp_commit();
     };
+    // this CTA's keys and values into the last stage, then the first tiles
+    stage_rows<W, ROWS>(sb + (NS - 1) * Sm::STAGE, static_cast<const bf16 *>(LOCAL ? a.k : a.kd) + (kvbase + j0) * W,
+                        N - j0, tid);
+    stage_rows<W, ROWS>(sb + (NS - 1) * Sm::STAGE + Sm::DO,
+                        static_cast<const bf16 *>(LOCAL ? a.v : a.vd) + (kvbase + j0) * W, N - j0, tid);
+    cp_commit();
     for (int t = 0; t < NS - 1; ++t)
         stage(t);
+    cp_wait<NS - 1>();
+    __syncthreads();
 
     const int r0 = j0 + 16 * MT * warp;  // this warp's keys r0 .. r0 + 16 MT - 1
     uint32_t ka[MT][W / 16][4], va[MT][W / 16][4];
     float dk[MT][NT][4], dv[MT][NT][4], zero[MT][2][4];
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt) {
-        load_a<W>(ka[mt], static_cast<const bf16 *>(LOCAL ? a.k : a.kd) + kvbase * W, r0 + 16 * mt, N, lane);
-        load_a<W>(va[mt], static_cast<const bf16 *>(LOCAL ? a.v : a.vd) + kvbase * W, r0 + 16 * mt, N, lane);
+        const uint32_t own = sb + (NS - 1) * Sm::STAGE + 16 * (MT * warp + mt) * LD;
+        load_a<W>(ka[mt], own, lane);
+        load_a<W>(va[mt], own + Sm::DO, lane);
 #pragma unroll
         for (int n = 0; n < NT; ++n)
 #pragma unroll
@@ -613,7 +655,7 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dkv_tc_kernel(
         static_assert(!LOCAL || MT == 1, "the lift stages 64 rows");
         // dk = scale dk_loc + dk^D Dk^T, dv = dv_loc + dv^D Dv^T, one after the other
         float *lift = reinterpret_cast<float *>(tsm);  // [64][DD + 1]
-        float *wt = lift + 64 * (DD + 1);              // [DD][64] W_down^T
+        float *wt = lift + 64 * (DD + 1);              // [DD][kLiftLd] W_down^T
         const int nv = min(ROWS, N - j0);
 #pragma unroll
         for (int kv = 0; kv < 2; ++kv) {
@@ -622,26 +664,29 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dkv_tc_kernel(
             const float *Wd = (kv ? a.Dv : a.Dk) + (size_t)g * 64 * DD;
             const float *x = (kv ? a.dvd : a.dkd) + (kvbase + j0) * DD;
             for (int e = tid; e < 64 * DD; e += kTc)
-                wt[(e % DD) * 64 + e / DD] = __ldg(Wd + e);
+                wt[(e % DD) * kLiftLd + e / DD] = __ldg(Wd + e);
             for (int e = tid; e < nv * DD; e += kTc)
                 lift[(e / DD) * (DD + 1) + e % DD] = x[e];
             __syncthreads();
+            float o[2][8][2];
+#pragma unroll
+            for (int hr = 0; hr < 2; ++hr)
+#pragma unroll
+                for (int n = 0; n < 8; ++n) {
+                    o[hr][n][0] = kv ? dv[0][n][2 * hr] : dk[0][n][2 * hr] * a.scale;
+                    o[hr][n][1] = kv ? dv[0][n][2 * hr + 1] : dk[0][n][2 * hr + 1] * a.scale;
+                }
+            const float *xr = lift + (16 * warp + grp) * (DD + 1);
+            lift_rows<DD, kLiftLd>(o, xr, xr + 8 * (DD + 1), wt, tig);
 #pragma unroll
             for (int hr = 0; hr < 2; ++hr) {
                 const int j = r0 + grp + 8 * hr;
                 if (j >= N)
                     continue;
-                float o[8][2];
-#pragma unroll
-                for (int n = 0; n < 8; ++n) {
-                    o[n][0] = kv ? dv[0][n][2 * hr] : dk[0][n][2 * hr] * a.scale;
-                    o[n][1] = kv ? dv[0][n][2 * hr + 1] : dk[0][n][2 * hr + 1] * a.scale;
-                }
-                lift16<DD>(o, lift + (j - j0) * (DD + 1), wt, tig);
                 bf16 *dst = static_cast<bf16 *>(kv ? a.dv : a.dk) + (kvbase + j) * 64;
 #pragma unroll
                 for (int n = 0; n < 8; ++n)
-                    *reinterpret_cast<uint32_t *>(dst + 8 * n + 2 * tig) = cvt_bf16x2(o[n][0], o[n][1]);
+                    *reinterpret_cast<uint32_t *>(dst + 8 * n + 2 * tig) = cvt_bf16x2(o[hr][n][0], o[hr][n][1]);
             }
         }
     }
@@ -669,7 +714,7 @@ __global__ void __launch_bounds__(rows_bulk<bf16>() / rows_per_thread<DD>() *sli
     __syncthreads();
     if (z) {  // eight lanes per row
         const uint4 *o = reinterpret_cast<const uint4 *>(static_cast<const bf16 *>(a.out) + row0 * 64);
-#pragma unroll 4
+#pragma unroll 8
         for (int e = tid; e < R * 8; e += NTH) {
             const int r = e / 8, c = e % 8;
             float x[8], y[8], s = 0.f;
@@ -693,6 +738,164 @@ __global__ void __launch_bounds__(rows_bulk<bf16>() / rows_per_thread<DD>() *sli
     for (int k = 0; k < rows_per_thread<DD>(); ++k)
         if (r0 + k * NR < nr)
             store_row<bf16, CW>(dst + (size_t)(r0 + k * NR) * DD, acc[k]);
+}
+
+// ---------------------------------------------------------------- projection gradients
+
+// bwd_wpart on the tensor cores: X is bf16, and Y (fp32) enters as the sum of
+// three bf16 terms, hi + mid + lo, each the rounded rest of the one before
+// (24 bits together, so a product is off by no more than an fp32 one's
+// rounding), accumulated in fp32.  X^T is the A operand (ldmatrix.trans from
+// rows of 64), Y the B operand, split in registers.  Eight warps share out the
+// columns (32 at most each) and the 16-row steps of a stage of 128 rows and are
+// added up in warp order.  The CUDA-core kernel spent 344 us on B8 H16 N8192,
+// d_down 16, on instructions: 19 per 16 products.
+constexpr int kWtRows = 128;
+
+template <int DD>
+struct WpartTc {
+    static constexpr int NC = DD < 32 ? DD : 32;       // columns per warp
+    static constexpr int CG = DD / NC, RW = 8 / CG;    // column groups, warps that share out the rows
+    static constexpr int XLD = 64 * 2 + 16, YLD = DD + 4;  // bytes / floats per padded row
+    static constexpr uint32_t Y = kWtRows * XLD, FAC = Y + kWtRows * YLD * 4, STAGE = FAC + kWtRows * 4;
+    static constexpr uint32_t TOTAL = 2 * STAGE;
+    static_assert(RW * 64 * DD * 4 <= (int)TOTAL, "the warps' sums fit in the stage area");
+};
+
+template <int DD>
+__global__ void __launch_bounds__(256) bwd_wpart_tc_kernel(Args a)
+{
+    using L = WpartTc<DD>;
+    constexpr int NC = L::NC, RW = L::RW;
+    extern __shared__ __align__(128) unsigned char tsm[];
+    const uint32_t sb = smem_u32(tsm);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, grp = lane >> 2, tig = lane & 3;
+    const int chunk = blockIdx.x, g = blockIdx.y, which = blockIdx.z;
+    const bool per_kv = which == 0 || which == 2;
+    const int heads = per_kv ? 1 : a.G;
+    const long nrows = (long)a.B * heads * a.N;
+    const long r0 = nrows * chunk / kChunks, r1 = nrows * (chunk + 1) / kChunks;
+    const bf16 *X = static_cast<const bf16 *>(which == 0 ? a.k : which == 1 ? a.q : which == 2 ? a.v : a.dout);
+    const float *Yp = which == 0 ? a.dkd : which == 1 ? a.dqt : which == 2 ? a.dvd : a.od;
+    const int ntiles = (int)((r1 - r0 + kWtRows - 1) / kWtRows);
+    // the next tile to stage starts at row i of sequence-and-head u
+    long u = r0 / a.N;
+    int i = (int)(r0 % a.N);
+    auto base_of = [&](long v) -> long {
+        return (per_kv ? v * a.Hkv + g : v / a.G * a.Hq + g * a.G + v % a.G) * a.N;
+    };
+    long base = base_of(u);
+    auto stage = [&](int t) {
+        const uint32_t d = sb + (t & 1) * L::STAGE;
+        const int n = (int)min((long)kWtRows, r1 - r0 - (long)t * kWtRows);
+        auto row_of = [&](int r) -> long {
+            int k = i + r;
+            if (k < a.N)
+                return base + k;
+            long v = u;
+            for (; k >= a.N; k -= a.N)
+                ++v;
+            return base_of(v) + k;
+        };
+#pragma unroll
+        for (int e = 0; e < kWtRows * 8 / 256; ++e) {
+            const int r = tid / 8 + 32 * e, c = tid % 8;
+            const bool ok = r < n;
+            cp16z(d + r * L::XLD + c * 16, X + (ok ? row_of(r) * 64 + c * 8 : 0), ok);
+        }
+#pragma unroll
+        for (int e = 0; e < kWtRows * (DD / 4) / 256; ++e) {
+            const int r = tid / (DD / 4) + 256 / (DD / 4) * e, c = tid % (DD / 4);
+            const bool ok = r < n;
+            cp16z(d + L::Y + r * (L::YLD * 4) + c * 16, Yp + (ok ? row_of(r) * DD + c * 4 : 0), ok);
+        }
+        if (!per_kv && tid < kWtRows) {
+            if (tid < n)
+                sm100::cp_async4(d + L::FAC + tid * 4, a.fac + row_of(tid));
+            else
+                reinterpret_cast<float *>(tsm + (t & 1) * L::STAGE + L::FAC)[tid] = 0.f;
+        }
+        cp_commit();
+        for (i += kWtRows; i >= a.N; i -= a.N)
+            base = base_of(++u);
+    };
+    float acc[4][NC / 8][4];
+#pragma unroll
+    for (int mt = 0; mt < 4; ++mt)
+#pragma unroll
+        for (int n = 0; n < NC / 8; ++n)
+            acc[mt][n][0] = acc[mt][n][1] = acc[mt][n][2] = acc[mt][n][3] = 0.f;
+    const int c0 = warp / RW * NC, k0 = warp % RW;
+    if (ntiles > 0)
+        stage(0);
+    for (int t = 0; t < ntiles; ++t) {
+        cp_wait<0>();
+        __syncthreads();  // tile t is in; every warp is done with tile t - 1
+        if (t + 1 < ntiles)
+            stage(t + 1);
+        const uint32_t xs = sb + (t & 1) * L::STAGE;
+        const float *ys = reinterpret_cast<const float *>(tsm + (t & 1) * L::STAGE + L::Y);
+        const float *fs = reinterpret_cast<const float *>(tsm + (t & 1) * L::STAGE + L::FAC);
+#pragma unroll
+        for (int ks = 0; ks < kWtRows / 16 / RW; ++ks) {
+            const int row = 16 * (k0 + RW * ks);
+            uint32_t xa[4][4];
+#pragma unroll
+            for (int mt = 0; mt < 4; ++mt)
+                ldsm_x4_t(xs + (row + (lane & 7) + ((lane >> 4) << 3)) * L::XLD + (16 * mt + ((lane >> 3) & 1) * 8) * 2,
+                          xa[mt]);
+            float f[4] = {1.f, 1.f, 1.f, 1.f};
+            if (!per_kv)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    f[e] = fs[row + 2 * tig + (e & 1) + 8 * (e >> 1)];
+#pragma unroll
+            for (int n = 0; n < NC / 8; ++n) {
+                uint32_t b[3][2];  // hi, mid, lo of rows 2 tig, + 1 (and + 8) of column grp
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float *y = ys + (row + 2 * tig + 8 * e) * L::YLD + c0 + 8 * n + grp;
+                    float y0 = y[0], y1 = y[L::YLD];
+                    if (!per_kv) {
+                        y0 *= f[2 * e];
+                        y1 *= f[2 * e + 1];
+                    }
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        b[k][e] = cvt_bf16x2(y0, y1);
+                        // (an infinity has no rest: it stays one, and is not turned into inf - inf)
+                        const float h0 = bf16lo(b[k][e]), h1 = bf16hi(b[k][e]);
+                        y0 = k == 0 && fabsf(h0) == INFINITY ? 0.f : y0 - h0;
+                        y1 = k == 0 && fabsf(h1) == INFINITY ? 0.f : y1 - h1;
+                    }
+                }
+#pragma unroll
+                for (int mt = 0; mt < 4; ++mt)
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        mma_bf16_c(acc[mt][n], xa[mt], b[k][0], b[k][1], acc[mt][n]);
+            }
+        }
+    }
+    __syncthreads();
+    float *red = reinterpret_cast<float *>(tsm);  // [RW][64][DD]
+#pragma unroll
+    for (int mt = 0; mt < 4; ++mt)
+#pragma unroll
+        for (int n = 0; n < NC / 8; ++n)
+#pragma unroll
+            for (int hr = 0; hr < 2; ++hr)
+                *reinterpret_cast<float2 *>(red + (size_t)k0 * 64 * DD + (16 * mt + grp + 8 * hr) * DD + c0 + 8 * n + 2 * tig) =
+                    make_float2(acc[mt][n][2 * hr], acc[mt][n][2 * hr + 1]);
+    __syncthreads();
+    float *dst = a.part + (((size_t)chunk * 4 + which) * a.Hkv + g) * 64 * DD;
+    for (int o = tid; o < 64 * DD; o += 256) {
+        float s = red[o];
+#pragma unroll
+        for (int k = 1; k < RW; ++k)
+            s += red[k * 64 * DD + o];
+        dst[o] = s;
+    }
 }
 
 // ---------------------------------------------------------------- host side
@@ -724,6 +927,8 @@ static cudaError_t run_tc(const Args &a, cudaStream_t s)
             e2 = opt_in(dkv_g, sk_g);
         if (e2 == cudaSuccess)
             e2 = opt_in(dkv_l, sk_l);
+        if (e2 == cudaSuccess)
+            e2 = opt_in(bwd_wpart_tc_kernel<DD>, WpartTc<DD>::TOTAL);
         return e2;
     });
     if (e != cudaSuccess)
@@ -736,7 +941,9 @@ static cudaError_t run_tc(const Args &a, cudaStream_t s)
     dq_l<<<a.B * a.Hq * tl, kTc, sq_l, s>>>(a);
     dkv_g<<<a.B * a.Hkv * tg, kTc, sk_g, s>>>(a);
     dkv_l<<<a.B * a.Hkv * tl, kTc, sk_l, s>>>(a);
-    return run_weights<bf16, DD>(a, s);
+    bwd_wpart_tc_kernel<DD><<<dim3(kChunks, a.Hkv, 4), 256, WpartTc<DD>::TOTAL, s>>>(a);
+    bwd_wsum_kernel<DD><<<(4 * a.Hkv * 64 * DD + kThreads - 1) / kThreads, kThreads, 0, s>>>(a);
+    return cudaGetLastError();
 }
 
 // bf16 storage: the tensor-core kernels for d_down >= 16 (whole 16-wide
