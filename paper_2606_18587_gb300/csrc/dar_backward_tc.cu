@@ -40,6 +40,7 @@ using sm100::ex2_approx;
 using sm100::ffma2;
 using sm100::ldsm_x4;
 using sm100::ldsm_x4_t;
+using sm100::mma_bf16_acc;
 using sm100::mma_bf16_c;
 using sm100::mul2;
 using sm100::smem_u32;
@@ -135,8 +136,8 @@ __device__ __forceinline__ void scores(float (&s)[MT][2][4], const uint32_t (&a)
                 mma_bf16_c(s[mt][0], a[mt][kk], f[0], f[1], c0[mt][0]);
                 mma_bf16_c(s[mt][1], a[mt][kk], f[2], f[3], c0[mt][1]);
             } else {
-                mma_bf16_c(s[mt][0], a[mt][kk], f[0], f[1], s[mt][0]);
-                mma_bf16_c(s[mt][1], a[mt][kk], f[2], f[3], s[mt][1]);
+                mma_bf16_acc(s[mt][0], a[mt][kk], f[0], f[1]);
+                mma_bf16_acc(s[mt][1], a[mt][kk], f[2], f[3]);
             }
         }
     }
@@ -152,8 +153,8 @@ __device__ __forceinline__ void accumulate(float (&acc)[MT][W / 8][4], const uin
         ldsm_x4_t(b + n * 16, f);
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
-            mma_bf16_c(acc[mt][n], a[mt], f[0], f[1], acc[mt][n]);
-            mma_bf16_c(acc[mt][n + 1], a[mt], f[2], f[3], acc[mt][n + 1]);
+            mma_bf16_acc(acc[mt][n], a[mt], f[0], f[1]);
+            mma_bf16_acc(acc[mt][n + 1], a[mt], f[2], f[3]);
         }
     }
 }
@@ -176,6 +177,11 @@ __device__ __forceinline__ void lift_rows(float (&o)[2][8][2], const float *x0, 
 }
 constexpr int kLiftLd = 66;  // row stride of a transposed W_down: its column-wise stores fall in distinct banks
 
+template <int V>
+struct Int {
+    static constexpr int value = V;
+};
+
 // Row tiles per warp and rows of the streamed tile per stage.
 template <int W, bool LOCAL>
 struct Shape {
@@ -183,7 +189,13 @@ struct Shape {
     static constexpr int ROWS = 64 * MT;                   // rows of a CTA's tile
     static constexpr int BK = !LOCAL && W <= 32 ? 128 : 64;  // streamed rows per stage
     static constexpr int NS = 3;
-    static constexpr int MINB = W == 16 ? 4 : W == 32 ? 2 : LOCAL ? 3 : 2;
+    static constexpr int MINB = LOCAL ? 3 : 2;
+    // 16-key blocks a dq step takes, 16-query steps in flight of dk/dv.  The
+    // 16-wide global kernels do best with few warps and long independent runs
+    // (B8 H16 N8192 w512, us, dq / dk, dv: 1431 / 1345 at 4, 8 and two CTAs per
+    // SM; 1461 / 1349 at 2, 2 and four; 1536 / 1378 at 1, 1 and four; at B8 H8
+    // N2047 w128 59 / 51, 69 / 57 and 65 / 58)
+    static constexpr int KSQ = W == 16 ? 4 : 2, UNKV = W == 16 ? 8 : 2;
     // a stage also takes the CTA's own rows, whose A fragments are read before it is needed
     static_assert(ROWS <= BK, "the CTA's tile fits in a stage");
 };
@@ -321,71 +333,74 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
             }
     };
 
-    for (int t = 0; t < ntiles; ++t) {
-        cp_wait<NS - 2>();
-        __syncthreads();  // tile t is in; every warp is done with tile t - 1
-        stage(t + NS - 1);
-        const uint32_t ks = sb + (t % NS) * Sm::STAGE;
-        const int jt = jlo + t * BK;
-#pragma unroll 1
-        for (int kc = 0; kc < BK / 16; ++kc) {
-            const int j = jt + 16 * kc;
-            // Eq. 3: no pair of the step / every pair of the step is of this kind
-            if (LOCAL ? j > r0 + 16 * MT - 1 : j > r0 + 16 * MT - 1 - w)
-                break;
-            if (LOCAL && j + 15 <= r0 - w)
-                continue;
-            // (a masked pair's weight is 0; its dP - D is set to 0 too, so that no
-            // 0 * infinity arises from a key the row does not see)
-            const bool all = LOCAL ? j + 15 <= r0 && j > r0 + 16 * MT - 1 - w : j + 15 <= r0 - w;
-            const uint32_t kst = ks + 16 * kc * LD, vst = kst + Sm::V;
-            float s[MT][2][4], dp[MT][2][4];
-            auto in_kind = [&](int mt, int nt, int e) {
-                const int i = r0 + 16 * mt + grp + 8 * (e >> 1), jj = j + 8 * nt + 2 * tig + (e & 1);
-                return LOCAL ? jj <= i && jj > i - w : jj <= i - w;
-            };
-            auto masked_scores = [&]() {
-                scores<W, MT>(s, qa, kst + b_lane<LD>(lane), zero);
-                if (!all) {
+    // KS 16-key blocks at once, the first at shared-memory row address kst and
+    // position j; ALL: every pair is of this kernel's kind, else the others are
+    // masked: their weight is 0, and their dP - D is set to 0 too, so that no
+    // 0 * infinity arises from a key the row does not see.
+    auto step = [&](auto all_c, auto ks_c, uint32_t kst, int j) {
+        constexpr bool ALL = decltype(all_c)::value != 0;
+        constexpr int KS = decltype(ks_c)::value;
+        float s[KS][MT][2][4];
+        auto in_kind = [&](int k, int mt, int nt, int e) {
+            const int i = r0 + 16 * mt + grp + 8 * (e >> 1), jj = j + 16 * k + 8 * nt + 2 * tig + (e & 1);
+            return LOCAL ? jj <= i && jj > i - w : jj <= i - w;
+        };
+        auto masked_scores = [&]() {
+#pragma unroll
+            for (int k = 0; k < KS; ++k) {
+                scores<W, MT>(s[k], qa, kst + 16 * k * LD + b_lane<LD>(lane), zero);
+                if constexpr (!ALL) {
 #pragma unroll
                     for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                         for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
                             for (int e = 0; e < 4; ++e)
-                                s[mt][nt][e] = in_kind(mt, nt, e) ? s[mt][nt][e] : -INFINITY;
+                                s[k][mt][nt][e] = in_kind(k, mt, nt, e) ? s[k][mt][nt][e] : -INFINITY;
                 }
-            };
-            masked_scores();
-            exponents(s);
-            float top = -INFINITY;
+            }
+        };
+        masked_scores();
+        float top = -INFINITY;
+#pragma unroll
+        for (int k = 0; k < KS; ++k) {
+            exponents(s[k]);
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt) {
-                    top = sm100::max3(top, s[mt][nt][0], s[mt][nt][1]);
-                    top = sm100::max3(top, s[mt][nt][2], s[mt][nt][3]);
+                    top = sm100::max3(top, s[k][mt][nt][0], s[k][mt][nt][1]);
+                    top = sm100::max3(top, s[k][mt][nt][2], s[k][mt][nt][3]);
                 }
-            if (__builtin_expect(__any_sync(0xffffffffu, top > kRaise) || fresh, 0)) {
-                // rare: the scores again (they were overwritten), then larger maxima
-                masked_scores();
-                raise(s);
-                exponents(s);
-                bool none = false;  // once no maximum is -infinity, every row has seen a key
+        }
+        if (__builtin_expect(__any_sync(0xffffffffu, top > kRaise) || fresh, 0)) {
+            // rare: the scores again (they were overwritten), then larger maxima
+            masked_scores();
 #pragma unroll
-                for (int mt = 0; mt < MT; ++mt)
-                    none = none || m[mt][0] == -INFINITY || m[mt][1] == -INFINITY;
-                fresh = __any_sync(0xffffffffu, none);
-            }
-            scores<W, MT>(dp, da, vst + b_lane<LD>(lane), nD);
-            if (!all) {
+            for (int k = 0; k < KS; ++k)
+                raise(s[k]);
+#pragma unroll
+            for (int k = 0; k < KS; ++k)
+                exponents(s[k]);
+            bool none = false;  // once no maximum is -infinity, every row has seen a key
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+                none = none || m[mt][0] == -INFINITY || m[mt][1] == -INFINITY;
+            fresh = __any_sync(0xffffffffu, none);
+        }
+#pragma unroll
+        for (int k = 0; k < KS; ++k) {
+            const uint32_t kr = kst + 16 * k * LD, vr = kr + Sm::V;
+            float dp[MT][2][4];
+            scores<W, MT>(dp, da, vr + b_lane<LD>(lane), nD);
+            if constexpr (!ALL) {
 #pragma unroll
                 for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                     for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
                         for (int e = 0; e < 4; ++e)
-                            dp[mt][nt][e] = in_kind(mt, nt, e) ? dp[mt][nt][e] : 0.f;
+                            dp[mt][nt][e] = in_kind(k, mt, nt, e) ? dp[mt][nt][e] : 0.f;
             }
             uint32_t ds[MT][4], pa[MT][4];
 #pragma unroll
@@ -394,7 +409,7 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
                 for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
                     for (int hr = 0; hr < 2; ++hr) {
-                        float &p0 = s[mt][nt][2 * hr], &p1 = s[mt][nt][2 * hr + 1];
+                        float &p0 = s[k][mt][nt][2 * hr], &p1 = s[k][mt][nt][2 * hr + 1];
                         p0 = ex2_approx(p0);
                         p1 = ex2_approx(p1);
                         add2(l[mt][hr][0], l[mt][hr][1], p0, p1, l[mt][hr][0], l[mt][hr][1]);
@@ -403,11 +418,41 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
                     }
                 frag_a(ds[mt], dp[mt][0], dp[mt][1]);
                 if constexpr (!LOCAL)
-                    frag_a(pa[mt], s[mt][0], s[mt][1]);
+                    frag_a(pa[mt], s[k][mt][0], s[k][mt][1]);
             }
-            accumulate<W, MT>(dq, ds, kst + bt_lane<LD>(lane));
+            accumulate<W, MT>(dq, ds, kr + bt_lane<LD>(lane));
             if constexpr (!LOCAL)
-                accumulate<W, MT>(od, pa, vst + bt_lane<LD>(lane));
+                accumulate<W, MT>(od, pa, vr + bt_lane<LD>(lane));
+        }
+    };
+
+    for (int t = 0; t < ntiles; ++t) {
+        cp_wait<NS - 2>();
+        __syncthreads();  // tile t is in; every warp is done with tile t - 1
+        stage(t + NS - 1);
+        const uint32_t ks = sb + (t % NS) * Sm::STAGE;
+        const int jt = jlo + t * BK;
+        // Eq. 3 over the warp's rows: a tile, or a 16-key block, all of whose pairs are of this kind
+        auto whole = [&](int j, int n) {
+            return LOCAL ? j + n - 1 <= r0 && j > r0 + 16 * MT - 1 - w : j + n - 1 <= r0 - w;
+        };
+        if (whole(jt, BK)) {
+#pragma unroll 1
+            for (int kc = 0; kc < BK / 16; kc += Sh::KSQ)
+                step(Int<1>(), Int<Sh::KSQ>(), ks + 16 * kc * LD, 0);
+            continue;
+        }
+#pragma unroll 1
+        for (int kc = 0; kc < BK / 16; ++kc) {
+            const int j = jt + 16 * kc;
+            if (LOCAL ? j > r0 + 16 * MT - 1 : j > r0 + 16 * MT - 1 - w)
+                break;  // no pair of this block or a later one
+            if (LOCAL && j + 15 <= r0 - w)
+                continue;
+            if (whole(j, 16))
+                step(Int<1>(), Int<1>(), ks + 16 * kc * LD, 0);
+            else
+                step(Int<0>(), Int<1>(), ks + 16 * kc * LD, j);
         }
     }
 
@@ -569,14 +614,75 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dkv_tc_kernel(
     }
     const float c2 = a.c2;
 
+    // the 16 queries at shared-memory row address qst (log-sum-exp and D at
+    // `rows`) and position i; ALL as in the dq kernel
+    auto step = [&](auto all_c, uint32_t qst, const float *rows, int i) {
+        constexpr bool ALL = decltype(all_c)::value != 0;
+        const uint32_t dst = qst + Sm::DO;
+        float s[MT][2][4], dp[MT][2][4], nD[MT][2][4];
+        float2 nl[2];
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+            const float2 d = *reinterpret_cast<const float2 *>(rows + (Sm::DR - Sm::LSE) / 4 + 8 * nt + 2 * tig);
+            nl[nt] = *reinterpret_cast<const float2 *>(rows + 8 * nt + 2 * tig);
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+                nD[mt][nt][0] = nD[mt][nt][2] = d.x;
+                nD[mt][nt][1] = nD[mt][nt][3] = d.y;
+            }
+        }
+        scores<W, MT>(s, ka, qst + b_lane<LD>(lane), zero);
+        scores<W, MT>(dp, va, dst + b_lane<LD>(lane), nD);
+        if constexpr (!ALL) {
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int jj = r0 + 16 * mt + grp + 8 * (e >> 1), ii = i + 8 * nt + 2 * tig + (e & 1);
+                        const bool in = LOCAL ? jj <= ii && jj > ii - w : jj <= ii - w;
+                        s[mt][nt][e] = in ? s[mt][nt][e] : -INFINITY;
+                        dp[mt][nt][e] = in ? dp[mt][nt][e] : 0.f;
+                    }
+        }
+        uint32_t pa[MT][4], ds[MT][4];
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                for (int hr = 0; hr < 2; ++hr) {
+                    float &p0 = s[mt][nt][2 * hr], &p1 = s[mt][nt][2 * hr + 1];
+                    ffma2(p0, p1, p0, p1, c2, c2, nl[nt].x, nl[nt].y);
+                    p0 = ex2_approx(p0);
+                    p1 = ex2_approx(p1);
+                    mul2(dp[mt][nt][2 * hr], dp[mt][nt][2 * hr + 1], p0, p1, dp[mt][nt][2 * hr],
+                         dp[mt][nt][2 * hr + 1]);
+                }
+            frag_a(pa[mt], s[mt][0], s[mt][1]);
+            frag_a(ds[mt], dp[mt][0], dp[mt][1]);
+        }
+        accumulate<W, MT>(dv, pa, dst + bt_lane<LD>(lane));
+        accumulate<W, MT>(dk, ds, qst + bt_lane<LD>(lane));
+    };
+
     for (int t = 0; t < ntiles; ++t) {
         cp_wait<NS - 2>();
         __syncthreads();
         stage(t + NS - 1);
         const uint32_t qs = sb + (t % NS) * Sm::STAGE;
-        const float *lse_s = reinterpret_cast<const float *>(tsm + (t % NS) * Sm::STAGE + Sm::LSE);
-        const float *dr_s = reinterpret_cast<const float *>(tsm + (t % NS) * Sm::STAGE + Sm::DR);
+        const float *rows = reinterpret_cast<const float *>(tsm + (t % NS) * Sm::STAGE + Sm::LSE);
         const int it = ilo + (t % per_head) * BK;
+        auto whole = [&](int i, int n) {  // (rows past the sequence's end have weight 0)
+            return LOCAL ? i >= r0 + 16 * MT - 1 && i + n - 1 < r0 + w : i >= r0 + 16 * MT - 1 + w;
+        };
+        if (whole(it, BK)) {
+#pragma unroll Sh::UNKV
+            for (int qc = 0; qc < BK / 16; ++qc)
+                step(Int<1>(), qs + 16 * qc * LD, rows + 16 * qc, 0);
+            continue;
+        }
 #pragma unroll 1
         for (int qc = 0; qc < BK / 16; ++qc) {
             const int i = it + 16 * qc;
@@ -584,54 +690,10 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dkv_tc_kernel(
                 break;
             if (LOCAL ? i + 15 < r0 : i + 15 < r0 + w)
                 continue;
-            const bool all = LOCAL ? i >= r0 + 16 * MT - 1 && i + 15 < r0 + w : i >= r0 + 16 * MT - 1 + w;
-            const uint32_t qst = qs + 16 * qc * LD, dst = qst + Sm::DO;
-            float s[MT][2][4], dp[MT][2][4], nD[MT][2][4];
-            float2 nl[2];
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt) {
-                const float2 d = *reinterpret_cast<const float2 *>(dr_s + 16 * qc + 8 * nt + 2 * tig);
-                nl[nt] = *reinterpret_cast<const float2 *>(lse_s + 16 * qc + 8 * nt + 2 * tig);
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt) {
-                    nD[mt][nt][0] = nD[mt][nt][2] = d.x;
-                    nD[mt][nt][1] = nD[mt][nt][3] = d.y;
-                }
-            }
-            scores<W, MT>(s, ka, qst + b_lane<LD>(lane), zero);
-            scores<W, MT>(dp, va, dst + b_lane<LD>(lane), nD);
-            if (!all) {
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-                    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int jj = r0 + 16 * mt + grp + 8 * (e >> 1), ii = i + 8 * nt + 2 * tig + (e & 1);
-                            const bool in = LOCAL ? jj <= ii && jj > ii - w : jj <= ii - w;
-                            s[mt][nt][e] = in ? s[mt][nt][e] : -INFINITY;
-                            dp[mt][nt][e] = in ? dp[mt][nt][e] : 0.f;
-                        }
-            }
-            uint32_t pa[MT][4], ds[MT][4];
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt) {
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                    for (int hr = 0; hr < 2; ++hr) {
-                        float &p0 = s[mt][nt][2 * hr], &p1 = s[mt][nt][2 * hr + 1];
-                        ffma2(p0, p1, p0, p1, c2, c2, nl[nt].x, nl[nt].y);
-                        p0 = ex2_approx(p0);
-                        p1 = ex2_approx(p1);
-                        mul2(dp[mt][nt][2 * hr], dp[mt][nt][2 * hr + 1], p0, p1, dp[mt][nt][2 * hr],
-                             dp[mt][nt][2 * hr + 1]);
-                    }
-                frag_a(pa[mt], s[mt][0], s[mt][1]);
-                frag_a(ds[mt], dp[mt][0], dp[mt][1]);
-            }
-            accumulate<W, MT>(dv, pa, dst + bt_lane<LD>(lane));
-            accumulate<W, MT>(dk, ds, qst + bt_lane<LD>(lane));
+            if (whole(i, 16))
+                step(Int<1>(), qs + 16 * qc * LD, rows + 16 * qc, 0);
+            else
+                step(Int<0>(), qs + 16 * qc * LD, rows + 16 * qc, i);
         }
     }
 
@@ -873,7 +935,7 @@ __global__ void __launch_bounds__(256) bwd_wpart_tc_kernel(Args a)
                 for (int mt = 0; mt < 4; ++mt)
 #pragma unroll
                     for (int k = 0; k < 3; ++k)
-                        mma_bf16_c(acc[mt][n], xa[mt], b[k][0], b[k][1], acc[mt][n]);
+                        mma_bf16_acc(acc[mt][n], xa[mt], b[k][0], b[k][1]);
             }
         }
     }
