@@ -20,11 +20,11 @@
 // the global part the ones ride in the v^D rows of the workspace (16 columns
 // after the d_down values), so one product of N = d_down + 16 gives both.
 //
-// Softmax arithmetic per score (the kernel is bound by the exponentials: one
-// per causal pair, 32 per clock per SM on the multi-function unit): a 3-input
-// max for the tile maximum, then per pair of scores one fp32x2 FMA
-// (x = s * scale * log2(e) - m), one conversion of the pair to bf16x2 and one
-// bf16x2 exp2, whose result is the packed bf16 P the PV product reads.
+// Softmax arithmetic per pair of scores (the kernel is bound by its issue slots
+// and the exponentials: one per causal pair, 32 per clock per SM on the
+// multi-function unit): one fp32x2 FMA (x = s * scale * log2(e) - m), one
+// 3-input max for the vote on raising m, one conversion of the pair to bf16x2
+// and one bf16x2 exp2, whose result is the packed bf16 P the PV product reads.
 //
 // Warp roles (352 threads): warp 0 issues TMA loads, warp 10 the S products
 // (and q~), warp 1 allocates TMEM and issues the PV products (each issuing
@@ -561,6 +561,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 
         const float c2 = a.qscale;  // softmax scale * log2(e)
         float mA = -INFINITY, mB = -INFINITY;  // running maxima (log2 units) of rows ra, ra + 8
+        bool fresh = true;  // some row of the warp has no running maximum yet
         // last tile whose PV this thread has seen complete, per S buffer
         int pv_seen0 = -1, pv_seen1 = -1;
         // wait until PV(v) (its own products) has completed
@@ -660,35 +661,64 @@ __global__ void __launch_bounds__(kThreads, 2)
                     }
                 }
             }
-            // row maxima: this thread's 16 columns, then across the row's four threads
-            float xA = max3(max3(sa[0], sa[1], sa[2]), max3(sa[3], sa[4], sa[5]), max3(sa[6], sa[7], sa[8]));
-            float xB = max3(max3(sv[0], sv[1], sv[2]), max3(sv[3], sv[4], sv[5]), max3(sv[6], sv[7], sv[8]));
-            xA = max3(xA, max3(sa[9], sa[10], sa[11]), max3(sa[12], sa[13], fmaxf(sa[14], sa[15])));
-            xB = max3(xB, max3(sv[9], sv[10], sv[11]), max3(sv[12], sv[13], fmaxf(sv[14], sv[15])));
-            xA = fmaxf(xA, __shfl_xor_sync(0xffffffffu, xA, 1));
-            xB = fmaxf(xB, __shfl_xor_sync(0xffffffffu, xB, 1));
-            xA = fmaxf(xA, __shfl_xor_sync(0xffffffffu, xA, 2)) * c2;
-            xB = fmaxf(xB, __shfl_xor_sync(0xffffffffu, xB, 2)) * c2;
-            // raise a running max only when it grows by more than the threshold
-            const bool raiseA = xA > mA + kRescaleThreshold, raiseB = xB > mB + kRescaleThreshold;
-            const bool scaleA = raiseA && mA != -INFINITY, scaleB = raiseB && mB != -INFINITY;
-            // O's scale factors when a running max is raised (applied below, once P is computed)
-            const float alA = scaleA ? ex2_approx(mA - xA) : 1.f, alB = scaleB ? ex2_approx(mB - xB) : 1.f;
-            if (raiseA)
-                mA = xA;
-            if (raiseB)
-                mB = xB;
-            // P = 2^(s * c2 - m) in bf16 pairs (masked entries give 0): pw[2k] row
-            // ra, pw[2k + 1] row ra + 8, P column 4k + q4 (keys 8k + 2 q4, + 1)
-            const float nA = mA == -INFINITY ? 0.f : -mA, nB = mB == -INFINITY ? 0.f : -mB;
+            // exponents y = s * c2 - m relative to the running maxima (masked
+            // entries: -infinity), in place
+            float nA = mA == -INFINITY ? 0.f : -mA, nB = mB == -INFINITY ? 0.f : -mB;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                ffma2(sa[2 * k], sa[2 * k + 1], sa[2 * k], sa[2 * k + 1], c2, c2, nA, nA);
+                ffma2(sv[2 * k], sv[2 * k + 1], sv[2 * k], sv[2 * k + 1], c2, c2, nB, nB);
+            }
+            // One vote per tile decides whether any row's maximum grows by more
+            // than the threshold (or is not set yet): the maximum of both rows'
+            // columns of this thread is enough for that, and the row maxima,
+            // their shuffles and the scale factors are left to the rare case.
+            float top = max3(sa[0], sa[1], sa[2]);
+#pragma unroll
+            for (int e = 3; e < 15; e += 2)
+                top = max3(top, sa[e], sa[e + 1]);
+            top = max3(top, sa[15], sv[0]);
+#pragma unroll
+            for (int e = 1; e < 15; e += 2)
+                top = max3(top, sv[e], sv[e + 1]);
+            top = fmaxf(top, sv[15]);
+            bool scaleA = false, scaleB = false;
+            float alA = 1.f, alB = 1.f;  // O's scale factors when a running max is raised
+            if (__builtin_expect(__any_sync(0xffffffffu, top > kRescaleThreshold) || fresh, 0)) {
+                auto row_max = [&](const float (&x)[16]) {
+                    float r = x[0];
+#pragma unroll
+                    for (int e = 1; e < 15; e += 2)
+                        r = max3(r, x[e], x[e + 1]);
+                    r = fmaxf(r, x[15]);
+                    r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, 1));
+                    return fmaxf(r, __shfl_xor_sync(0xffffffffu, r, 2));
+                };
+                auto raise = [&](float (&x)[16], float &m, float &n, float &al) {
+                    const float r = row_max(x);  // relative to the old maximum (to 0 while there is none)
+                    const bool none = m == -INFINITY;
+                    if (!(none ? r > -INFINITY : r > kRescaleThreshold))
+                        return false;
+                    al = none ? 1.f : ex2_approx(-r);
+                    m = none ? r : m + r;
+                    const float d = -m - n;  // (-r but for m's rounding)
+                    n = -m;
+#pragma unroll
+                    for (int e = 0; e < 16; ++e)
+                        x[e] += d;
+                    return !none;
+                };
+                scaleA = raise(sa, mA, nA, alA);
+                scaleB = raise(sv, mB, nB, alB);
+                fresh = __any_sync(0xffffffffu, (iA < N && mA == -INFINITY) || (iB < N && mB == -INFINITY));
+            }
+            // P = 2^y in bf16 pairs: pw[2k] row ra, pw[2k + 1] row ra + 8, P column
+            // 4k + q4 (keys 8k + 2 q4, + 1)
             uint32_t pw[16];
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                float x0, x1, y0, y1;
-                ffma2(x0, x1, sa[2 * k], sa[2 * k + 1], c2, c2, nA, nA);
-                ffma2(y0, y1, sv[2 * k], sv[2 * k + 1], c2, c2, nB, nB);
-                pw[2 * k] = ex2_bf16x2(cvt_bf16x2(x0, x1));
-                pw[2 * k + 1] = ex2_bf16x2(cvt_bf16x2(y0, y1));
+                pw[2 * k] = ex2_bf16x2(cvt_bf16x2(sa[2 * k], sa[2 * k + 1]));
+                pw[2 * k + 1] = ex2_bf16x2(cvt_bf16x2(sv[2 * k], sv[2 * k + 1]));
             }
             if (__builtin_expect(__any_sync(0xffffffffu, scaleA || scaleB), 0)) {
                 // every earlier PV must have landed before O is rescaled (PV(t),
