@@ -65,30 +65,35 @@ struct AppendArgs {
     int B, Hkv, n, D, DL, w, maxp, num_pages;
 };
 
+// What an append does with sequence b: its length and count, or the status to report.
+__device__ __forceinline__ int append_counts(const AppendArgs &a, int b, int &L, int &nb)
+{
+    nb = a.n_per_seq ? __ldg(a.n_per_seq + b) : a.n;
+    L = a.seq_lens[b];
+    if (nb < 0 || nb > a.n || L < 0)
+        return DAR_ERR_INVALID_ARG;
+    return (long long)L + nb > (long long)a.maxp * kTok && nb > 0 ? DAR_ERR_CAPACITY : DAR_OK;
+}
+
 constexpr int kAppTok = 4;  // tokens per block
 
-// Block (token group, b): c = round_bf16(chain_e h[e] Wdown[e][a]) for the
+// Block (token group, b): c = round_bf16(chain_k h[k] Wdown[k][c]) for the
 // group's tokens, written to their pages; ring rows of the tokens that stay in
 // the window.  The lengths are read here and advanced by latent_lens_kernel.
 __global__ void __launch_bounds__(256) latent_append_kernel(AppendArgs a)
 {
     extern __shared__ float hs[];  // [kAppTok][D]
     const int b = blockIdx.y, r0 = blockIdx.x * kAppTok;
-    const int nb = a.n_per_seq ? __ldg(a.n_per_seq + b) : a.n;
-    if (nb < 0 || nb > a.n) {
+    int L, nb;
+    const int e = append_counts(a, b, L, nb);
+    if (e != DAR_OK) {
         if (threadIdx.x == 0 && blockIdx.x == 0)
-            report(a.status, DAR_ERR_INVALID_ARG);
+            report(a.status, e);
         return;
     }
     if (r0 >= nb)
         return;
-    const int L = __ldg(a.seq_lens + b);
     const int Lnew = L + nb;
-    if (Lnew > a.maxp * kTok) {
-        if (threadIdx.x == 0)
-            report(a.status, DAR_ERR_CAPACITY);
-        return;
-    }
     const int nt = min(kAppTok, nb - r0);
     const bf16 *h = static_cast<const bf16 *>(a.h) + ((size_t)b * a.n + r0) * a.D;
     for (int i = threadIdx.x; i < nt * a.D; i += blockDim.x)
@@ -114,22 +119,184 @@ __global__ void __launch_bounds__(256) latent_append_kernel(AppendArgs a)
             continue;
         }
         float acc = 0.f;  // Eq. 1: one fp32 chain over e = 0..D-1 from +0
-        for (int e = 0; e < a.D; ++e)
-            acc = fmaf(hs[t * a.D + e], __ldg(a.Wdown + (size_t)e * a.DL + c), acc);
+        for (int k = 0; k < a.D; ++k)
+            acc = fmaf(hs[t * a.D + k], __ldg(a.Wdown + (size_t)k * a.DL + c), acc);
         static_cast<bf16 *>(a.pool_c)[((size_t)pid * kTok + p % kTok) * a.DL + c] = __float2bfloat16_rn(acc);
+    }
+}
+
+// The same append as a matrix product, for D a multiple of 8 (rows of h that
+// start on 16 bytes): rows are the B n tokens in memory order, whatever their
+// sequence; a CTA takes ROWS rows and COLS columns and walks D in pieces of K
+// through a ring of cp.async stages.  A thread holds the fp32 chains of TPT
+// rows and CPT columns, two per instruction, in the order of the kernel above.
+// The chains bound it (a chain cannot be split over threads, and no tensor core
+// rounds like one): 8 prompts of 500 to 1000 tokens, D 2048, DL 256, are 3.1 G
+// FMA, 85 us at the chip's fp32 rate: 844 us with the kernel above, 169 with
+// this one (FMA pipe 63 % busy; 2.5 CTAs per SM on average, 3 on the fullest).
+// WIDE tiles (8 rows x 4 columns per thread) read 6 operands per 32 products;
+// narrow ones, for few tokens, take one column per thread, so that a warp's read
+// of W is one wavefront and the chip's SMs share the columns.
+constexpr int kTileThreads = 128, kTileStages = 3;
+
+template <int TPT, int CPT>
+struct Tile {
+    static constexpr bool WIDE = CPT > 1;
+    static constexpr int LC = WIDE ? 8 : 32;            // lanes side by side over the columns
+    static constexpr int CW = WIDE ? 2 : 1;             // warps side by side over the columns
+    static constexpr int GROUPS = 4 / CW * (32 / LC);   // threads that share a column
+    static constexpr int ROWS = GROUPS * TPT, COLS = CW * LC * CPT;
+    static constexpr int K = WIDE ? 64 : 128;
+    static constexpr int W_BYTES = K * COLS * 4;
+    static constexpr int STAGE = W_BYTES + ROWS * K * 2;
+    static constexpr int TOTAL = kTileStages * STAGE;
+};
+
+template <int TPT, int CPT>
+__global__ void __launch_bounds__(kTileThreads) latent_append_tiled_kernel(AppendArgs a)
+{
+    using T = Tile<TPT, CPT>;
+    constexpr int NT = kTileThreads, ROWS = T::ROWS, COLS = T::COLS, K = T::K;
+    extern __shared__ __align__(128) unsigned char tile[];
+    __shared__ long long s_dst[ROWS];   // element offset of the row's bottleneck in the pool (-1: none)
+    __shared__ int s_b[ROWS], s_slot[ROWS], s_j[ROWS];  // sequence, ring slot (-1: not kept), index in the call
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int ncol = a.DL / COLS, c0 = (int)(blockIdx.x % ncol) * COLS;
+    const long long rows = (long long)a.B * a.n, r0 = (long long)(blockIdx.x / ncol) * ROWS;
+    bool live = false;
+    for (int r = tid; r < ROWS; r += NT) {
+        s_dst[r] = -1;
+        s_slot[r] = -1;
+        if (r0 + r >= rows)
+            continue;
+        const int b = (int)((r0 + r) / a.n), j = (int)((r0 + r) % a.n);
+        int L, nb;
+        const int e = append_counts(a, b, L, nb);
+        if (e != DAR_OK) {
+            if (j == 0 && c0 == 0)
+                report(a.status, e);
+            continue;
+        }
+        if (j >= nb)
+            continue;
+        live = true;
+        const int p = L + j;
+        s_b[r] = b;
+        s_j[r] = j;
+        s_slot[r] = j >= nb - a.w ? p % a.w : -1;
+        const int pid = __ldg(a.block_table + (size_t)b * a.maxp + p / kTok);
+        if (pid < 0 || pid >= a.num_pages)
+            report(a.status, DAR_ERR_CAPACITY);
+        else
+            s_dst[r] = ((long long)pid * kTok + p % kTok) * a.DL + c0;
+    }
+    if (!__syncthreads_or(live))
+        return;
+
+    const bf16 *h = static_cast<const bf16 *>(a.h) + r0 * a.D;
+    const int nr = (int)min((long long)ROWS, rows - r0), steps = (a.D + K - 1) / K;
+    const uint32_t base = smem_u32(tile);
+    auto load = [&](int st) {
+        if (st < steps) {
+            const int k0 = st * K, nk = min(K, a.D - k0);
+            const uint32_t wb = base + st % kTileStages * T::STAGE, hb = wb + T::W_BYTES;
+            for (int i = tid; i < nk * (COLS / 4); i += NT) {
+                const int k = i / (COLS / 4), c = i % (COLS / 4);
+                cp_async16(wb + i * 16, a.Wdown + (size_t)(k0 + k) * a.DL + c0 + c * 4);
+            }
+            for (int i = tid; i < nr * (K / 8); i += NT) {
+                const int r = i / (K / 8), c = i % (K / 8);
+                if (c * 8 < nk)
+                    cp_async16(hb + r * (K * 2) + ((c ^ (r & 7)) << 4), h + (size_t)r * a.D + k0 + c * 8);
+            }
+        }
+        cp_async_commit();
+    };
+#pragma unroll
+    for (int st = 0; st < kTileStages - 1; ++st)
+        load(st);
+
+    // ring rows of the tokens that stay in the window, shared out over the column tiles
+    for (int i = (int)(blockIdx.x % ncol) * NT + tid; i < nr * a.Hkv * 8; i += ncol * NT) {
+        const int r = i / (a.Hkv * 8), g = i / 8 % a.Hkv, ch = i % 8;
+        if (s_slot[r] < 0)
+            continue;
+        const size_t bg = (size_t)s_b[r] * a.Hkv + g;
+        const size_t src = (bg * a.n + s_j[r]) * 8 + ch, dst = (bg * a.w + s_slot[r]) * 8 + ch;
+        reinterpret_cast<uint4 *>(a.win_k)[dst] = reinterpret_cast<const uint4 *>(a.k_new)[src];
+        reinterpret_cast<uint4 *>(a.win_v)[dst] = reinterpret_cast<const uint4 *>(a.v_new)[src];
+    }
+
+    // this thread's rows tg + GROUPS i and columns cg CPT ..
+    const int cg = warp % T::CW * T::LC + lane % T::LC, tg = warp / T::CW * (32 / T::LC) + lane / T::LC;
+    float acc[TPT][CPT];
+#pragma unroll
+    for (int i = 0; i < TPT; ++i)
+#pragma unroll
+        for (int c = 0; c < CPT; ++c)
+            acc[i][c] = 0.f;
+#pragma unroll 1
+    for (int st = 0; st < steps; ++st) {
+        cp_async_wait<kTileStages - 2>();
+        __syncthreads();  // stage st has landed, and everyone is done with the one that load() overwrites
+        load(st + kTileStages - 1);
+        const unsigned char *ws = tile + st % kTileStages * T::STAGE, *hs = ws + T::W_BYTES;
+        const int nq = min(K, a.D - st * K) / 8;
+#pragma unroll 2
+        for (int q = 0; q < nq; ++q) {
+            uint4 x4[TPT];
+#pragma unroll
+            for (int i = 0; i < TPT; ++i) {
+                const int r = tg + T::GROUPS * i;
+                x4[i] = *reinterpret_cast<const uint4 *>(hs + r * (K * 2) + ((q ^ (r & 7)) << 4));
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                float x[TPT];
+#pragma unroll
+                for (int i = 0; i < TPT; ++i) {
+                    const uint32_t u = e < 2 ? x4[i].x : e < 4 ? x4[i].y : e < 6 ? x4[i].z : x4[i].w;
+                    x[i] = e & 1 ? bf16hi(u) : bf16lo(u);
+                }
+                const float *wr = reinterpret_cast<const float *>(ws) + (q * 8 + e) * COLS + cg * CPT;
+                if constexpr (T::WIDE) {
+                    const float4 w4 = *reinterpret_cast<const float4 *>(wr);
+#pragma unroll
+                    for (int i = 0; i < TPT; ++i) {
+                        ffma2(acc[i][0], acc[i][1], x[i], x[i], w4.x, w4.y, acc[i][0], acc[i][1]);
+                        ffma2(acc[i][2], acc[i][3], x[i], x[i], w4.z, w4.w, acc[i][2], acc[i][3]);
+                    }
+                } else if constexpr (TPT > 1) {
+#pragma unroll
+                    for (int i = 0; i < TPT; i += 2)
+                        ffma2(acc[i][0], acc[i + 1][0], x[i], x[i + 1], *wr, *wr, acc[i][0], acc[i + 1][0]);
+                } else {
+                    acc[0][0] = fmaf(x[0], *wr, acc[0][0]);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < TPT; ++i) {
+        const long long dst = s_dst[tg + T::GROUPS * i];
+        if (dst < 0)
+            continue;
+        bf16 *o = static_cast<bf16 *>(a.pool_c) + dst + cg * CPT;
+        if constexpr (T::WIDE)
+            *reinterpret_cast<uint2 *>(o) =
+                make_uint2(cvt_bf16x2(acc[i][0], acc[i][1]), cvt_bf16x2(acc[i][2], acc[i][3]));
+        else
+            *o = __float2bfloat16_rn(acc[i][0]);
     }
 }
 
 __global__ void latent_lens_kernel(AppendArgs a)
 {
+    grid_dep_wait();  // every CTA of the append has read the lengths
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= a.B)
-        return;
-    const int nb = a.n_per_seq ? a.n_per_seq[b] : a.n;
-    if (nb < 0 || nb > a.n)
-        return;
-    if (a.seq_lens[b] + nb <= a.maxp * kTok)
-        a.seq_lens[b] += nb;
+    int L, nb;
+    if (b < a.B && append_counts(a, b, L, nb) == DAR_OK)
+        a.seq_lens[b] = L + nb;
 }
 
 // A[g][c][t] = chain_e Wup[c][e] W[g][e][t] (fp32), for A_K (stored as
@@ -860,6 +1027,64 @@ static cudaError_t decode_dl(const Args &a, const void *pool_c, const void *win_
     return a.Hq <= 16 ? decode_t<DL, 1>(a, pool_c, win_k, win_v, s) : decode_t<DL, 2>(a, pool_c, win_k, win_v, s);
 }
 
+// The tiled append's launch.
+template <int TPT, int CPT>
+static cudaError_t append_tiled(const AppendArgs &a, cudaStream_t s)
+{
+    using T = Tile<TPT, CPT>;
+    static PerDeviceOnce once;
+    const cudaError_t e = per_device_once(once, [](int) {
+        return cudaFuncSetAttribute(latent_append_tiled_kernel<TPT, CPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    T::TOTAL);
+    });
+    if (e != cudaSuccess)
+        return e;
+    const long long tiles = ((long long)a.B * a.n + T::ROWS - 1) / T::ROWS;
+    latent_append_tiled_kernel<TPT, CPT><<<(unsigned)(tiles * (a.DL / T::COLS)), kTileThreads, T::TOTAL, s>>>(a);
+    return cudaGetLastError();
+}
+
+// The tile by the number of CTAs it makes: the smallest that does not fill the
+// chip several times over (small ones have the shorter chain loop, big ones read
+// less shared memory per product).  Measured, us, rows x D x DL, tiles of
+// 4 / 8 / 16 rows x 32 columns and 32 / 64 rows x 64 columns:
+//     8 x 2048 x 256   22.6   25.4   30.0   48.0   72.1
+//    64 x 2048 x 256   23.0   25.4   30.8   51.3   77.8
+//   600 x  768 x 192   25.2   17.7   18.8   25.1   36.9
+//   520 x 2048 x 256   55.5   44.5   38.1   51.3   78.0
+//  2000 x 1024 x 256   84.5   59.7   51.6   40.6   43.9
+//  8000 x 2048 x 256    571    386    312    187    169
+static cudaError_t append_tiled_any(const AppendArgs &a, cudaStream_t s)
+{
+    const auto ctas = [&](int rows, int cols) {
+        return ((long long)a.B * a.n + rows - 1) / rows * (a.DL / cols);
+    };
+    if (ctas(4, 32) <= 152)
+        return append_tiled<1, 1>(a, s);
+    if (ctas(8, 32) <= 152 * 3)
+        return append_tiled<2, 1>(a, s);
+    if (ctas(16, 32) <= 152 * 3)
+        return append_tiled<4, 1>(a, s);
+    if (ctas(32, 64) <= 152 * 4)
+        return append_tiled<4, 4>(a, s);
+    return append_tiled<8, 4>(a, s);
+}
+
+// Advances the lengths once the append has finished.
+static cudaError_t append_lens(const AppendArgs &a, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((a.B + 255) / 256);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, latent_lens_kernel, a);
+}
+
 }  // namespace lat
 
 size_t latent_decode_workspace_bytes(int B, int Hq, int DL, int maxp)
@@ -932,17 +1157,23 @@ cudaError_t launch_latent_append(const LatentAppendArgs &x, cudaStream_t s)
     a.w = x.w;
     a.maxp = x.maxp;
     a.num_pages = x.num_pages;
+    cudaError_t e;
+    if (x.D % 8 == 0 && ((long long)x.B * x.n + 3) / 4 * (x.DL / 32) <= 0x7fffffffLL) {
+        e = lat::append_tiled_any(a, s);
+        return e != cudaSuccess ? e : lat::append_lens(a, s);
+    }
     const size_t smem = (size_t)lat::kAppTok * x.D * sizeof(float);
     static PerDeviceOnce once;
-    cudaError_t e = per_device_once(once, [&](int) {
+    e = per_device_once(once, [&](int) {
         return cudaFuncSetAttribute(lat::latent_append_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)(lat::kAppTok * 8192 * sizeof(float)));
     });
     if (e != cudaSuccess)
         return e;
     lat::latent_append_kernel<<<dim3((x.n + lat::kAppTok - 1) / lat::kAppTok, x.B), 256, smem, s>>>(a);
-    lat::latent_lens_kernel<<<(x.B + 255) / 256, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    if ((e = cudaGetLastError()) != cudaSuccess)
+        return e;
+    return lat::append_lens(a, s);
 }
 
 cudaError_t launch_latent_absorb(const float *Wup, const float *WK, const float *WV, float *Ak, float *Av, int Hkv,

@@ -1,8 +1,8 @@
 """The tiled matrix-product form of the latent append: bottlenecks bit-exact
-against the oracle's chain at hidden widths with and without a 64-wide
-remainder, widths that take the token-group kernel (not a multiple of 8), token
-counts around a tile and across sequences of one tile, each number of tokens
-per thread, and sequences the call refuses."""
+against the oracle's chain at hidden widths with and without a remainder of a
+stage, widths that take the token-group kernel (not a multiple of 8), token
+counts around a tile and across sequences of one tile, each tile shape, and
+sequences the call refuses."""
 import numpy as np
 import pytest
 
@@ -30,13 +30,14 @@ def make(B, Hkv, D, dl, w, n, before, seed):
 
 
 @pytest.mark.parametrize("B,Hkv,D,dl,w,n,before", [
-    (3, 2, 64, 64, 5, 1, 0),         # one token per sequence, three sequences in a tile
-    (2, 1, 72, 64, 100, 17, 60),     # a remainder of 8 past the first chunk of D; a page boundary
+    (3, 2, 64, 64, 5, 1, 0),         # 4 x 32 tiles: one token per sequence, three sequences in a tile
+    (2, 1, 72, 64, 100, 17, 60),     # less than a stage; a page boundary
     (2, 2, 100, 128, 7, 33, 3),      # D not a multiple of 8: token groups
-    (5, 2, 200, 192, 64, 130, 10),   # a remainder of 8 past three chunks
-    (2, 3, 8, 256, 16, 40, 0),       # one 8-wide piece
-    (4, 1, 128, 256, 50, 400, 63),   # two tokens per thread
-    (8, 2, 136, 256, 300, 450, 1),   # four tokens per thread, ragged tiles
+    (5, 2, 200, 192, 64, 130, 10),   # 16 x 32 tiles, a remainder of 72 past the first stage
+    (2, 3, 8, 256, 16, 40, 0),       # 8 x 32 tiles, one 8-wide piece
+    (4, 1, 128, 256, 50, 400, 63),   # 32 x 64 tiles, two whole stages
+    (8, 2, 136, 256, 300, 450, 1),   # 32 x 64 tiles, a remainder of 8, ragged tiles
+    (11, 1, 72, 256, 10, 450, 7),    # 64 x 64 tiles, a remainder of 8, a last tile of 22 rows
 ])
 def test_bottlenecks_and_ring_are_exact(B, Hkv, D, dl, w, n, before):
     c, table, h, k, Wd = make(B, Hkv, D, dl, w, n, before, 700 + D + n)
