@@ -490,7 +490,7 @@ dar_status prefill_common(dar_dtype dtype, int32_t B, int32_t Hq, int32_t Hkv, i
     a.qd_ratio = qd ? default_scale(scale_down, d_down) / default_scale(scale, d) : 1.f;
     if (dtype == DAR_BF16)
         return from_cuda(dar::launch_prefill_tc(d_down, a, st), "dar_attn_prefill (tcgen05) launch");
-    return from_cuda(dar::launch_prefill_simt(dtype, d_down, a, st), "dar_attn_prefill launch");
+    return from_cuda(dar::launch_prefill_simt(d_down, a, st), "dar_attn_prefill launch");
 }
 
 }  // namespace

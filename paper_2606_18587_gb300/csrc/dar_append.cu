@@ -16,13 +16,8 @@ namespace dar {
 // A block takes a tile of contiguous token rows (dar_project.cuh); two chains
 // advance per instruction (fma.rn.f32x2: outputs c and c + 1 share x_t) and
 // each element is still the exact fp32 chain acc = fma(x_t, W[t][c], acc).
+// Threads take RPT rows each, NR apart.
 // blockIdx.z selects the tensor: 0 = (x0, W0, out0), 1 = (x1, W1, out1).
-template <typename T, int DD>
-__host__ __device__ constexpr int threads_bulk()
-{
-    return rows_bulk<T>() / rows_per_thread<DD>() * slices<DD>();
-}
-
 struct BulkArgs {
     const void *x[2];
     const float *W[2];
@@ -32,12 +27,12 @@ struct BulkArgs {
     int ones_col[2];  // first of 16 padding columns set to 1 (-1: all padding is 0)
 };
 
-template <typename T, int DD>
-__global__ void __launch_bounds__(threads_bulk<T, DD>()) down_project_kernel(BulkArgs a)
+template <typename T, int DD, int RPT, int NR>
+__global__ void __launch_bounds__(NR *slices<DD>()) down_project_kernel(BulkArgs a)
 {
-    constexpr int R = rows_bulk<T>(), RPT = rows_per_thread<DD>(), NT = threads_bulk<T, DD>(), NR = R / RPT;
+    constexpr int R = RPT * NR, NT = NR * slices<DD>();
     constexpr int CW = cols_per_thread<DD>();
-    __shared__ __align__(16) unsigned char rows[kStageBytesBulk];
+    __shared__ __align__(16) unsigned char rows[R * kHeadDim * sizeof(T)];
     __shared__ __align__(16) float Ws[kHeadDim * DD];
     const bool z = blockIdx.z != 0;  // (selects, not indexes: the arguments stay in parameter space)
     const T *x = static_cast<const T *>(z ? a.x[1] : a.x[0]);
@@ -53,12 +48,12 @@ __global__ void __launch_bounds__(threads_bulk<T, DD>()) down_project_kernel(Bul
     // this thread's rows: r0 + k * NR, columns c0 .. c0 + CW - 1 (rows past nr
     // compute on stale staging bytes and are not stored)
     const int r0 = threadIdx.x % NR, c0 = slices<DD>() > 1 ? (int)threadIdx.x / NR * CW : 0;
-    float acc[rows_per_thread<DD>()][CW];
-    project_rows<T, DD, CW, rows_per_thread<DD>()>(rows, Ws + c0, r0, NR, acc);
+    float acc[RPT][CW];
+    project_rows<T, DD, CW, RPT>(rows, Ws + c0, r0, NR, acc);
     const int ostride = z ? a.ostride[1] : a.ostride[0];
     const int ones_col = z ? a.ones_col[1] : a.ones_col[0];
 #pragma unroll
-    for (int k = 0; k < rows_per_thread<DD>(); ++k) {
+    for (int k = 0; k < RPT; ++k) {
         const int r = r0 + k * NR;
         if (r >= nr)
             continue;
@@ -343,19 +338,35 @@ __global__ void append_lens_kernel(AppendArgs a)
 
 // ----------------------------------------------------------------- launchers
 
+// Big tiles (several rows per thread, so that one read of W feeds them all)
+// once they give every SM two; otherwise one row per thread.  Measured on the
+// prefill, big / small, us: 8 tiles (fp32, 4 heads x N 256) 20.2 / 17.3; 128
+// tiles (16 heads x N 1000) 22.3 / 20.8; 512 tiles (32 heads x N 2000, d_down
+// 64) 92 / 101; 1024 tiles (64 heads x N 2047) 82.6 / 85.3.
+constexpr int kBulkSmallRows = 64;
+constexpr long long kProjectBigCtas = 152 * 2;
+
+template <typename T, int DD>
+static cudaError_t down_project_dd(const BulkArgs &a, int B, int nz, cudaStream_t s)
+{
+    constexpr int R = rows_bulk<T>(), RPT = rows_per_thread<DD>(), NR = R / RPT, SR = kBulkSmallRows;
+    if ((long long)(a.n + R - 1) / R * B * a.Hkv * nz >= kProjectBigCtas)
+        down_project_kernel<T, DD, RPT, NR><<<dim3((a.n + R - 1) / R, B * a.Hkv, nz), NR * slices<DD>(), 0, s>>>(a);
+    else
+        down_project_kernel<T, DD, 1, SR><<<dim3((a.n + SR - 1) / SR, B * a.Hkv, nz), SR * slices<DD>(), 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 template <typename T>
 static cudaError_t down_project_t(int dd, const BulkArgs &a, int B, int nz, cudaStream_t s)
 {
-    constexpr int R = rows_bulk<T>();
-    dim3 grid((a.n + R - 1) / R, B * a.Hkv, nz);
     switch (dd) {
-    case 8: down_project_kernel<T, 8><<<grid, threads_bulk<T, 8>(), 0, s>>>(a); break;
-    case 16: down_project_kernel<T, 16><<<grid, threads_bulk<T, 16>(), 0, s>>>(a); break;
-    case 32: down_project_kernel<T, 32><<<grid, threads_bulk<T, 32>(), 0, s>>>(a); break;
-    case 64: down_project_kernel<T, 64><<<grid, threads_bulk<T, 64>(), 0, s>>>(a); break;
+    case 8: return down_project_dd<T, 8>(a, B, nz, s);
+    case 16: return down_project_dd<T, 16>(a, B, nz, s);
+    case 32: return down_project_dd<T, 32>(a, B, nz, s);
+    case 64: return down_project_dd<T, 64>(a, B, nz, s);
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 static cudaError_t down_project_any(dar_dtype dt, int dd, const BulkArgs &a, int B, int nz, cudaStream_t s)
@@ -427,9 +438,7 @@ static cudaError_t append_bulk_launch(const AppendArgs &a, cudaStream_t s)
     return cudaLaunchKernelEx(&cfg, append_lens_kernel, a);
 }
 
-// Big tiles (several rows per thread, so that one read of W feeds them all)
-// once they fill the chip a few times over; otherwise one row per thread.
-constexpr int kBulkSmallRows = 64;
+// Here big tiles pay once they fill the chip a few times over.
 constexpr long long kBulkBigCtas = 152 * 6 * 2;
 
 template <typename T, int DD>

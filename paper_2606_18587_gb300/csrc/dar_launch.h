@@ -107,7 +107,7 @@ cudaError_t launch_down_project_kv(dar_dtype dt, int dd, const void *k, const vo
                                    int vstride, int v_ones_col, cudaStream_t s);
 cudaError_t launch_cache_append(dar_dtype dt, int dd, const AppendArgs &a, cudaStream_t s);
 cudaError_t launch_decode(dar_dtype dt, int dd, const DecodeArgs &a, cudaStream_t s);
-cudaError_t launch_prefill_simt(dar_dtype dt, int dd, const PrefillArgs &a, cudaStream_t s);
+cudaError_t launch_prefill_simt(int dd, const PrefillArgs &a, cudaStream_t s);
 cudaError_t launch_prefill_tc(int dd, const PrefillArgs &a, cudaStream_t s);
 
 // Gradients of the causal forward (dar_backward.cu); the workspace holds the
