@@ -205,6 +205,21 @@ __device__ __forceinline__ void buf_of(int t, int &b, int &u)
     u = ALIAS ? t >> 1 : t;
 }
 
+// The sequence with the n-th longest context (n = 0: the longest; ties by index) of
+// B <= 32, computed by each warp on its own.  A chunk's CTAs take as long as their
+// context, so the longest go first: a 512-token chunk of 32 heads over four contexts of
+// 2048 to 8000 tokens 150 -> 141 us.
+__device__ __forceinline__ int nth_longest(const int32_t *len, int B, int n, int lane)
+{
+    const int mine = lane < B ? len[lane] : -1;
+    int rank = 0;
+    for (int o = 0; o < B; ++o) {
+        const int x = __shfl_sync(0xffffffffu, mine, o);
+        rank += x > mine || (x == mine && o < lane);
+    }
+    return __ffs(__ballot_sync(0xffffffffu, lane < B && rank == n)) - 1;
+}
+
 // CH = false: the causal forward over positions 0..N-1 of q, k, v.  CH = true:
 // chunked prefill over a cache (positions pos0[b] .. pos0[b] + n - 1; local
 // keys from the window buffer, global keys from whole pages (tmPK, tmPV)
@@ -245,8 +260,11 @@ __global__ void __launch_bounds__(kThreads, 2)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int w = a.w;
     const bool direct = a.qd != nullptr;  // Sec. 5 direct variant: q~ given, not absorbed
-    const int bh = blockIdx.x, b = bh / a.Hq, h = bh % a.Hq, g = h / (a.Hq / a.Hkv);
-    const int L0 = CH ? __ldg(a.pos0 + b) : 0;  // position of query row 0
+    if constexpr (CH)
+        grid_dep_wait();  // the gather kernel, which writes pos0 and the buffers
+    const int bx = blockIdx.x / a.Hq, b = CH && a.B <= 32 ? nth_longest(a.pos0, a.B, bx, lane) : bx;
+    const int h = blockIdx.x % a.Hq, g = h / (a.Hq / a.Hkv);
+    const int L0 = CH ? a.pos0[b] : 0;           // position of query row 0
     const int nrows = CH ? a.n : a.N;            // query rows per (b, h)
     const int N = L0 + nrows;                    // end of the query positions
     const int nqt = (nrows + BM - 1) / BM;
@@ -301,6 +319,8 @@ __global__ void __launch_bounds__(kThreads, 2)
             }
             mbar_expect_tx(q_full, BM * 64 * 2);
             tma_load_2d(sm + Ly::Q, &tmQ, 0, (b * a.Hq + h) * nrows + qt * BM, q_full);
+            if constexpr (!CH)
+                grid_dep_wait();  // k^D and v^D come from the kernel before (nothing else here does)
             for (int t = 0; t < VT; ++t) {
                 const VTile vt = tiles.at(t);
                 const int s = t % NS;
@@ -889,8 +909,18 @@ static cudaError_t launch_kernel(const CUtensorMap (&m)[7], const PrefillArgs &a
     if (e != cudaSuccess)
         return e;
     dim3 grid(a.B * a.Hq, (nrows + BM - 1) / BM);
-    kern<<<grid, kThreads, smem, s>>>(m[0], m[1], m[2], m[3], m[4], m[5], m[6], a);
-    return cudaGetLastError();
+    // starts while the last blocks of the Eq. 1 (gather) kernel run; see grid_dep_wait
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, m[0], m[1], m[2], m[3], m[4], m[5], m[6], a);
 }
 
 template <int DP>
@@ -924,8 +954,9 @@ static cudaError_t launch_dp(const PrefillArgs &a, cudaStream_t s)
 //    the same fp32 chain as the cache append; zero otherwise.
 // grid (B, Hkv, slices), 256 threads: the rows of a (sequence, KV head) are
 // dealt out over the slices (one block per pair left 120 of the 152 SMs idle
-// on a 4-sequence, 8-head chunk of 512 tokens).  Block (b, 0, 0) records L0 in
-// pos0[b].
+// on a 4-sequence, 8-head chunk of 512 tokens; there, one element per thread
+// with two-byte loads took 23 us, four columns with 16-byte loads 12).  Block
+// (b, 0, 0) records L0 in pos0[b].
 template <int DD>
 __global__ void __launch_bounds__(256) chunk_gather_kernel(ChunkArgs c)
 {
@@ -970,36 +1001,39 @@ __global__ void __launch_bounds__(256) chunk_gather_kernel(ChunkArgs c)
         kw[i] = k4;
         vw[i] = v4;
     }
-    // ---- tail rows, one element per thread and tensor
-    bf16 *kdt = static_cast<bf16 *>(c.kdt) + bg * NT * DD;
-    bf16 *vdt = static_cast<bf16 *>(c.vdt) + bg * NT * DD;
-    const bf16 *pk = static_cast<const bf16 *>(ap.pool_kd);
-    const bf16 *pv = static_cast<const bf16 *>(ap.pool_vd);
-    for (int i = tid; i < NT * DD; i += step) {
-        const int r = i / DD, col = i % DD, p = kt0 + r;
-        bf16 kx = __float2bfloat16_rn(0.f), vx = kx;
+    // ---- tail rows, four columns of one tensor per thread
+    constexpr int QD = DD / 4;
+    for (int i = tid; i < NT * 2 * QD; i += step) {
+        const int c4 = i % QD * 4, r = i / QD % NT, p = kt0 + r;
+        const bool v = i >= NT * QD;
+        uint2 x = make_uint2(0u, 0u);
         if (p < L0 - w) {  // migrated before this call: its page
-            int pid = ap.block_table[(size_t)b * ap.maxp + p / kPage];
-            if (pid >= 0 && pid < ap.num_pages) {
-                const size_t off = (((size_t)pid * Hkv + g) * kPage + p % kPage) * DD + col;
-                kx = pk[off];
-                vx = pv[off];
-            } else {
+            const int pid = ap.block_table[(size_t)b * ap.maxp + p / kPage];
+            if (pid >= 0 && pid < ap.num_pages)
+                x = *reinterpret_cast<const uint2 *>(static_cast<const bf16 *>(v ? ap.pool_vd : ap.pool_kd) +
+                                                     (((size_t)pid * Hkv + g) * kPage + p % kPage) * DD + c4);
+            else
                 report(ap.status, DAR_ERR_CAPACITY);
-            }
         } else if (p < L0 + n - w) {  // leaves the window in this chunk: Eq. 1
-            const bf16 *xk = row_of(p, false), *xv = row_of(p, true);
-            const float *Wk = ap.Dk + (size_t)g * 64 * DD + col, *Wv = ap.Dv + (size_t)g * 64 * DD + col;
-            float ak = 0.0f, av = 0.0f;  // the fp32 chain over t = 0..63 of the cache append
-            for (int t = 0; t < 64; ++t) {
-                ak = __fmaf_rn(__bfloat162float(xk[t]), __ldg(Wk + (size_t)t * DD), ak);
-                av = __fmaf_rn(__bfloat162float(xv[t]), __ldg(Wv + (size_t)t * DD), av);
+            const uint4 *row = reinterpret_cast<const uint4 *>(row_of(p, v));
+            const float *W = (v ? ap.Dv : ap.Dk) + (size_t)g * 64 * DD + c4;
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};  // the fp32 chains over t = 0..63 of the cache append
+#pragma unroll 2
+            for (int q = 0; q < 8; ++q) {
+                float xf[8];
+                unpack(row[q], xf, bf16());
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const float4 w4 = __ldg(reinterpret_cast<const float4 *>(W + (size_t)(q * 8 + e) * DD));
+                    acc[0] = __fmaf_rn(xf[e], w4.x, acc[0]);
+                    acc[1] = __fmaf_rn(xf[e], w4.y, acc[1]);
+                    acc[2] = __fmaf_rn(xf[e], w4.z, acc[2]);
+                    acc[3] = __fmaf_rn(xf[e], w4.w, acc[3]);
+                }
             }
-            kx = __float2bfloat16_rn(ak);
-            vx = __float2bfloat16_rn(av);
+            x = make_uint2(cvt_bf16x2(acc[0], acc[1]), cvt_bf16x2(acc[2], acc[3]));
         }
-        kdt[i] = kx;
-        vdt[i] = vx;
+        *reinterpret_cast<uint2 *>(static_cast<bf16 *>(v ? c.vdt : c.kdt) + (bg * NT + r) * DD + c4) = x;
     }
 }
 
@@ -1007,7 +1041,7 @@ template <int DP>
 static cudaError_t launch_chunk_dp(const ChunkArgs &c, cudaStream_t s)
 {
     const PrefillArgs &a = c.pf;
-    const int slices = min(64, (max(a.NT * DP, a.NW * 8) + 255) / 256);
+    const int slices = min(64, (max(a.NT * DP / 2, a.NW * 8) + 255) / 256);
     chunk_gather_kernel<DP><<<dim3(a.B, a.Hkv, slices), 256, 0, s>>>(c);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
