@@ -16,10 +16,10 @@
 //    token; new keys/values into the ring; then the lengths.
 //  - latent_absorb: A_K, A_V (fp32 chains over D).
 //  - decode: prep (q~ = q A_K^T, bf16), main (a persistent kernel: work
-//    items are latent splits of four pages and windows of one KV head; a
-//    producer warp streams their 64-token tiles through a TMA ring, four
-//    consumer warps compute S = A B^T and O += P V on mma.sync tensor cores
-//    with one online softmax per head and write one partial record per item),
+//    items are latent units of four pages and windows of one KV head; their
+//    64-token tiles come through a TMA ring, four warps compute S = A B^T and
+//    O += P V on mma.sync tensor cores with one online softmax per head and
+//    write one partial record per segment),
 //    merge (exact log-sum-exp combination of the partial records, then
 //    o = (O_loc + O_lat A_V) / l).
 #include <cuda.h>
@@ -319,10 +319,11 @@ __global__ void latent_absorb_kernel(const float *Wup, const float *WK, const fl
 // ---------------------------------------------------------------- decode: prep
 
 // q~[b][h][c] = sum_t q[b][h][t] A_K[g][t][c] (fp32, stored as bf16).  Block
-// (g, 4 rows of KV head g): A_K^g staged in shared memory by one bulk copy,
+// (g, a few rows of KV head g): A_K^g staged in shared memory by one bulk copy,
 // then one warp per row, lanes over c.  It starts the main kernel's launch at once: that
 // kernel stages its first pages before it waits for q~.
-constexpr int kRowsPerBlock = 4;  // rows (one per warp) of one KV head per block
+constexpr int kRowsPerBlock = 8;  // at most: rows (one per warp) of one KV head per block
+constexpr int kRowThreads = 32 * kRowsPerBlock;
 
 // One bulk asynchronous copy of `bytes` (a multiple of 16) from global to
 // shared memory, waited for by the whole block (bounded; on a timeout the
@@ -348,7 +349,7 @@ __device__ __forceinline__ bool stage_matrix(void *dst, const void *src, unsigne
 }
 
 template <int DL>
-__global__ void __launch_bounds__(128) latent_prep_kernel(Args a)
+__global__ void __launch_bounds__(kRowThreads) latent_prep_kernel(Args a)
 {
     extern __shared__ __align__(16) float aks[];  // [64][DL], then the barrier
     grid_dep_launch();
@@ -357,7 +358,7 @@ __global__ void __launch_bounds__(128) latent_prep_kernel(Args a)
                       a.status))
         return;
     const int nrows = a.B * a.G;
-    for (int r = blockIdx.y * kRowsPerBlock + warp; r < min(nrows, (int)(blockIdx.y + 1) * kRowsPerBlock); r += 4) {
+    if (const int r = blockIdx.y * (blockDim.x >> 5) + warp; r < nrows) {
         const int row = (r / a.G) * a.Hq + g * a.G + r % a.G;
         const bf16 *qr = static_cast<const bf16 *>(a.q) + (size_t)row * 64;
         const float q0 = __bfloat162float(qr[lane]), q1 = __bfloat162float(qr[lane + 32]);
@@ -388,154 +389,248 @@ __device__ __forceinline__ uint32_t swz(uint32_t base, int row, int chunk)
     return base + (uint32_t)(row * 128 + ((chunk ^ (row & 7)) << 4));
 }
 
-constexpr int kConsumerThreads = 128;                   // warps 0-3: tensor-core work
-constexpr int kMainThreads2 = kConsumerThreads + 32;    // warp 4: TMA producer
+constexpr int kConsumerThreads = 128;  // warps 0-3: tensor-core work
 
 // Persistent main kernel.  Work items, enumerated the same way by every
-// thread: first the latent splits (sequence b, up to four 64-token pages of
-// its distant part), then the windows (sequence b, KV head g: the last
-// min(L_b, w) tokens' full keys and values, in 64-token tiles).  CTA c takes
-// items c, c + gridDim.x, ...  Warp 4 streams the items' pages and tiles
-// through a ring of NST stages with TMA; warps 0-3 run each stage on the
-// tensor cores and release it.
+// thread: first the latent units (sequence b, up to four 64-token pages of its
+// distant part), then the windows (sequence b, KV head g: the last min(L_b, w)
+// tokens' full keys and values, in 64-token tiles).  A CTA takes a run of
+// consecutive items of about equal estimated time; the units of one sequence in
+// its run form one segment with one partial record (kept in the slot of its
+// first unit; the other slots are marked empty).  The items' pages and tiles come
+// through a ring of NST stages by TMA, and warps 0-3 run each stage on the tensor
+// cores.
+//
+// Latency bounds it: two CTAs of four consumer warps share an SM (an SM holds
+// six 32 KB stages), and the steps of a stage form a chain.  So the rows' A
+// fragments stay in registers over a segment, a CTA writes one record for many
+// pages, and a stage takes two barriers (row maxima, weights).  Warp 4 issues the
+// copies, except at d_lat 256 with two row tiles, where a tenth warp on the SM
+// would leave the others 168 registers: there thread 0 refills a stage at the
+// next one's first barrier, when every warp is done with it (62 us for 64
+// sequences of 1024 to 8192 tokens, 32 heads, d_lat 256; 72 with the warp; at 8
+// heads, d_lat 128, 26 with the warp, 29 without).  Measured, prep to merge,
+// against round-robin items with a record per unit and the rows read from shared
+// memory: those 64 sequences 88 -> 62 us; 32 sequences of 4096, 12 heads, d_lat
+// 192 28 -> 25; one sequence of 8192, 32 heads, d_lat 256 22 -> 18.
 template <int DL, int MT>
 struct MainLayout {
+    static constexpr bool kProducer = !(DL == 256 && MT == 2);
+    static constexpr int THREADS = kConsumerThreads + (kProducer ? 32 : 0);
     static constexpr uint32_t CST = DL >= 128 ? DL / 64 * 8192 : 16384;  // a latent page, or a window K + V tile
-    static constexpr int NST = DL <= 128 ? 6 : DL == 192 ? 4 : 2;
-    static constexpr uint32_t QA = 0;                                     // [DL/64][MT*16][128 B] A operand
-    static constexpr uint32_t STG = (DL / 64 * MT * 16 * 128 + 1023) / 1024 * 1024;
+    static constexpr int NST = DL <= 128 ? 6 : DL == 192 ? 4 : 3;
+    static constexpr uint32_t STG = 0;
     static constexpr uint32_t P = STG + NST * CST;                        // [MT*16][128 B]
-    static constexpr uint32_t RED = P + MT * 16 * 128;                    // [4][MT*16] floats
-    static constexpr uint32_t PREF = RED + 4 * MT * 16 * 4;               // [B + 1] ints (B <= 1024)
+    static constexpr uint32_t RED = P + MT * 16 * 128;                    // [4 warps][16] floats
+    static constexpr uint32_t PREF = RED + 4 * 16 * 4;                    // [B + 1] ints (B <= 1024)
     static constexpr uint32_t BAR = PREF + (DAR_DECODE_MAX_BATCH + 1) * 4 + 4;
     static constexpr uint32_t TOTAL = (BAR + 16 * NST + 16 + 15) / 16 * 16;
 };
 
-struct Item {
+// A latent segment (units of one sequence) or a window.
+struct Segment {
     bool latent;
-    int b, part;  // latent: split index; window: KV head
+    int b, part;  // latent: first unit of the sequence; window: KV head
+    int units;    // items it covers
     int npg;      // pages / tiles
 };
 
-template <int MT>
 __device__ __forceinline__ void consumer_sync()
 {
     asm volatile("bar.sync 1, %0;" ::"n"(kConsumerThreads) : "memory");
 }
 
-// One stage on the tensor cores: S = A B^T over W-wide rows (A: the item's
-// q~ / q rows, MTT m-tiles; B: the stage's key-side tile), masks past ntok,
-// one online-softmax step per row (maxima exchanged through `red`), P into
-// shared memory, O += P V (V: the stage's value-side tile, W-wide rows).
-template <int W, int MTT, int MTR>
-__device__ __forceinline__ void run_stage(uint32_t qa, uint32_t ktile, uint32_t vtile, unsigned char *sm_p,
-                                          uint32_t pbase, float *red, int ntok, float c2, float (&o)[MTT][W / 32][4],
-                                          float (&mrun)[MTT][2], float (&lpart)[MTT][2], int warp, int lane)
-{
-    constexpr int NT = W / 32;
-    const int grp = lane >> 2, tig = lane & 3;
-    float sc[MTT][2][4];
-#pragma unroll
-    for (int mt = 0; mt < MTT; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-            sc[mt][nt][0] = sc[mt][nt][1] = sc[mt][nt][2] = sc[mt][nt][3] = 0.f;
+// What the warps hold of MT m-tiles (16 rows each) of W-wide rows.  Scores:
+// warp `warp` takes m-tile warp % MT and 16 MT of a stage's 64 tokens, with the
+// rows' A fragments in registers; values: W / 4 columns of every m-tile.
+template <int W, int MT>
+struct Rows {
+    uint32_t a[W / 16][4];
+    float o[MT][W / 32][4];
+    float m[MT][2];  // running maxima (log2 units) of rows grp, grp + 8 of each m-tile
+    float l[2];      // sums of this warp's weights, rows of its own m-tile
+
+    // x: `n` rows of stride W (rows past n: zero)
+    __device__ __forceinline__ void start(const bf16 *x, int n, int warp, int lane)
     {
-        const int tok = 16 * warp + (lane & 7) + ((lane >> 4) << 3);
-        const int khalf = (lane >> 3) & 1;
+        const int r0 = warp % MT * 16 + (lane >> 2), k0 = 2 * (lane & 3);
 #pragma unroll
-        for (int kk = 0; kk < W / 16; ++kk) {
-            const int ch = 2 * kk + khalf;
-            uint32_t bfr[4];
-            ldsm_x4(swz(ktile + (ch / 8) * 8192, tok, ch % 8), bfr);
+        for (int kk = 0; kk < W / 16; ++kk)
 #pragma unroll
-            for (int mt = 0; mt < MTT; ++mt) {
-                const int row = mt * 16 + (lane & 15), ach = 2 * kk + (lane >> 4);
-                uint32_t afr[4];
-                ldsm_x4(swz(qa + (ach / 8) * (MTR * 16 * 128), row, ach % 8), afr);
-                mma_bf16_16816(sc[mt][0], afr, bfr[0], bfr[1]);
-                mma_bf16_16816(sc[mt][1], afr, bfr[2], bfr[3]);
+            for (int e = 0; e < 4; ++e) {
+                const int r = r0 + 8 * (e & 1);
+                a[kk][e] = r < n ? *reinterpret_cast<const uint32_t *>(x + (size_t)r * W + kk * 16 + 8 * (e >> 1) + k0)
+                                 : 0u;
+            }
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+#pragma unroll
+            for (int nt = 0; nt < W / 32; ++nt)
+                o[mt][nt][0] = o[mt][nt][1] = o[mt][nt][2] = o[mt][nt][3] = 0.f;
+            m[mt][0] = m[mt][1] = -INFINITY;
+        }
+        l[0] = l[1] = 0.f;
+    }
+
+    // One stage: S = A B^T (B: the key-side tile), masks past ntok, one
+    // online-softmax step per row (maxima exchanged through `red`), P into shared
+    // memory, O += P V (V: the value-side tile).  refill() runs once every warp is
+    // done with the stage before.
+    template <typename F>
+    __device__ __forceinline__ void stage(uint32_t ktile, uint32_t vtile, unsigned char *sm_p, float *red, int ntok,
+                                          float c2, int warp, int lane, F &&refill)
+    {
+        constexpr int NTS = 2 * MT, NT = W / 32;
+        const int grp = lane >> 2, tig = lane & 3, own = warp % MT, tok0 = 16 * MT * (warp / MT);
+        float sc[NTS][4];
+#pragma unroll
+        for (int nt = 0; nt < NTS; ++nt)
+            sc[nt][0] = sc[nt][1] = sc[nt][2] = sc[nt][3] = 0.f;
+        {
+            const int tok = tok0 + (lane & 7) + ((lane >> 4) << 3), khalf = (lane >> 3) & 1;
+#pragma unroll
+            for (int kk = 0; kk < W / 16; ++kk) {
+                const int ch = 2 * kk + khalf;
+#pragma unroll
+                for (int np = 0; np < MT; ++np) {
+                    uint32_t bfr[4];
+                    ldsm_x4(swz(ktile + (ch / 8) * 8192, tok + 16 * np, ch % 8), bfr);
+                    mma_bf16_16816(sc[2 * np], a[kk], bfr[0], bfr[1]);
+                    mma_bf16_16816(sc[2 * np + 1], a[kk], bfr[2], bfr[3]);
+                }
             }
         }
-    }
+        if (ntok < kTok)
 #pragma unroll
-    for (int mt = 0; mt < MTT; ++mt) {
-        float mx0 = -INFINITY, mx1 = -INFINITY;
+            for (int nt = 0; nt < NTS; ++nt)
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int col = 16 * warp + 8 * nt + 2 * tig + e;
-                if (col >= ntok)
-                    sc[mt][nt][e] = sc[mt][nt][2 + e] = -INFINITY;
-                mx0 = fmaxf(mx0, sc[mt][nt][e]);
-                mx1 = fmaxf(mx1, sc[mt][nt][2 + e]);
-            }
-        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
-        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
-        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
-        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
-        if (tig == 0) {
-            red[warp * MTT * 16 + mt * 16 + grp] = mx0;
-            red[warp * MTT * 16 + mt * 16 + grp + 8] = mx1;
-        }
-    }
-    consumer_sync<MTT>();
-#pragma unroll
-    for (int mt = 0; mt < MTT; ++mt)
+                for (int e = 0; e < 4; ++e)
+                    if (tok0 + 8 * nt + 2 * tig + (e & 1) >= ntok)
+                        sc[nt][e] = -INFINITY;
 #pragma unroll
         for (int hr = 0; hr < 2; ++hr) {
-            const int row = mt * 16 + grp + 8 * hr;
-            float tmax = red[row];
+            float mx = -INFINITY;
 #pragma unroll
-            for (int w2 = 1; w2 < 4; ++w2)
-                tmax = fmaxf(tmax, red[w2 * MTT * 16 + row]);
-            const float mnew = fmaxf(mrun[mt][hr], tmax * c2);
-            const float alpha = mrun[mt][hr] == -INFINITY ? 0.f : ex2_approx(mrun[mt][hr] - mnew);
-            mrun[mt][hr] = mnew;
-            lpart[mt][hr] *= alpha;
+            for (int nt = 0; nt < NTS; ++nt)
+                mx = max3(mx, sc[nt][2 * hr], sc[nt][2 * hr + 1]);
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+            if (tig == 0)
+                red[warp * 16 + grp + 8 * hr] = mx;
+        }
+        consumer_sync();
+        refill();
+        float alpha[MT][2], mo[2];
+        bool grown = false;
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-                o[mt][nt][2 * hr] *= alpha;
-                o[mt][nt][2 * hr + 1] *= alpha;
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int hr = 0; hr < 2; ++hr) {
+                float mx = -INFINITY;
+#pragma unroll
+                for (int w2 = mt; w2 < 4; w2 += MT)
+                    mx = fmaxf(mx, red[w2 * 16 + grp + 8 * hr]);
+                const float mnew = fmaxf(m[mt][hr], mx * c2);
+                grown |= mnew != m[mt][hr];
+                alpha[mt][hr] = m[mt][hr] == -INFINITY ? 0.f : ex2_approx(m[mt][hr] - mnew);
+                m[mt][hr] = mnew;
+                if (mt == own) {
+                    l[hr] *= alpha[mt][hr];
+                    mo[hr] = mnew;
+                }
             }
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt) {
-                const float x0 = sc[mt][nt][2 * hr], x1 = sc[mt][nt][2 * hr + 1];
-                const float p0 = x0 == -INFINITY ? 0.f : ex2_approx(fmaf(x0, c2, -mnew));
-                const float p1 = x1 == -INFINITY ? 0.f : ex2_approx(fmaf(x1, c2, -mnew));
+        for (int hr = 0; hr < 2; ++hr) {
+            const int row = own * 16 + grp + 8 * hr;
+#pragma unroll
+            for (int nt = 0; nt < NTS; ++nt) {
+                const float x0 = sc[nt][2 * hr], x1 = sc[nt][2 * hr + 1];
+                const float p0 = x0 == -INFINITY ? 0.f : ex2_approx(fmaf(x0, c2, -mo[hr]));
+                const float p1 = x1 == -INFINITY ? 0.f : ex2_approx(fmaf(x1, c2, -mo[hr]));
                 const uint32_t pk = cvt_bf16x2(p0, p1);
-                lpart[mt][hr] += bf16lo(pk) + bf16hi(pk);  // the weights the PV product uses
-                const int col = 16 * warp + 8 * nt + 2 * tig;
-                *reinterpret_cast<uint32_t *>(sm_p + row * 128 + (((col >> 3) ^ (row & 7)) << 4) + 4 * tig) = pk;
+                l[hr] += bf16lo(pk) + bf16hi(pk);  // the weights the PV product uses
+                *reinterpret_cast<uint32_t *>(sm_p + row * 128 + ((((tok0 >> 3) + nt) ^ (row & 7)) << 4) + 4 * tig) =
+                    pk;
             }
         }
-    consumer_sync<MTT>();
+        if (__any_sync(0xffffffffu, grown)) {
 #pragma unroll
-    for (int kk = 0; kk < kTok / 16; ++kk) {
-        uint32_t afr[MTT][4];
+            for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int mt = 0; mt < MTT; ++mt)
-            ldsm_x4(swz(pbase, mt * 16 + (lane & 15), 2 * kk + (lane >> 4)), afr[mt]);
-        const int krow = 16 * kk + (lane & 7) + (((lane >> 3) & 1) << 3);
+                for (int hr = 0; hr < 2; ++hr)
 #pragma unroll
-        for (int np = 0; np < NT / 2; ++np) {
-            const int n0 = warp * (W / 4) + 16 * np + ((lane >> 4) << 3);
-            uint32_t bfr[4];
-            ldsm_x4_t(swz(vtile + (n0 / 64) * 8192, krow, (n0 % 64) / 8), bfr);
+                    for (int nt = 0; nt < NT; ++nt) {
+                        o[mt][nt][2 * hr] *= alpha[mt][hr];
+                        o[mt][nt][2 * hr + 1] *= alpha[mt][hr];
+                    }
+        }
+        consumer_sync();
+        const uint32_t pbase = smem_u32(sm_p);
 #pragma unroll
-            for (int mt = 0; mt < MTT; ++mt) {
-                mma_bf16_16816(o[mt][2 * np], afr[mt], bfr[0], bfr[1]);
-                mma_bf16_16816(o[mt][2 * np + 1], afr[mt], bfr[2], bfr[3]);
+        for (int kk = 0; kk < kTok / 16; ++kk) {
+            uint32_t afr[MT][4];
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+                ldsm_x4(swz(pbase, mt * 16 + (lane & 15), 2 * kk + (lane >> 4)), afr[mt]);
+            const int krow = 16 * kk + (lane & 7) + (((lane >> 3) & 1) << 3);
+#pragma unroll
+            for (int np = 0; np < NT / 2; ++np) {
+                const int n0 = warp * (W / 4) + 16 * np + ((lane >> 4) << 3);
+                uint32_t bfr[4];
+                ldsm_x4_t(swz(vtile + (n0 / 64) * 8192, krow, (n0 % 64) / 8), bfr);
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    mma_bf16_16816(o[mt][2 * np], afr[mt], bfr[0], bfr[1]);
+                    mma_bf16_16816(o[mt][2 * np + 1], afr[mt], bfr[2], bfr[3]);
+                }
             }
         }
     }
-}
+
+    // Records (O, m, l) of rows 0 .. n - 1: rec(row) points at W + 2 floats.
+    template <typename F>
+    __device__ __forceinline__ void finish(float *red, int n, int warp, int lane, F &&rec)
+    {
+        const int grp = lane >> 2, tig = lane & 3;
+#pragma unroll
+        for (int hr = 0; hr < 2; ++hr) {
+            l[hr] += __shfl_xor_sync(0xffffffffu, l[hr], 1);
+            l[hr] += __shfl_xor_sync(0xffffffffu, l[hr], 2);
+        }
+        consumer_sync();  // `red` is free
+        if (tig == 0) {
+            red[warp * 16 + grp] = l[0];
+            red[warp * 16 + grp + 8] = l[1];
+        }
+        consumer_sync();
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int hr = 0; hr < 2; ++hr) {
+                const int row = mt * 16 + grp + 8 * hr;
+                if (row >= n)
+                    continue;
+                float *r = rec(row);
+#pragma unroll
+                for (int nt = 0; nt < W / 32; ++nt)
+                    *reinterpret_cast<float2 *>(r + warp * (W / 4) + 8 * nt + 2 * tig) =
+                        make_float2(o[mt][nt][2 * hr], o[mt][nt][2 * hr + 1]);
+                if (warp == 0 && tig == 0) {
+                    float ls = 0.f;
+#pragma unroll
+                    for (int w2 = mt; w2 < 4; w2 += MT)
+                        ls += red[w2 * 16 + grp + 8 * hr];
+                    r[W] = m[mt][hr];
+                    r[W + 1] = ls;
+                }
+            }
+    }
+};
 
 template <int DL, int MT>
-__global__ void __launch_bounds__(kMainThreads2) latent_main_kernel(const __grid_constant__ CUtensorMap tmC,
-                                                                    const __grid_constant__ CUtensorMap tmK,
-                                                                    const __grid_constant__ CUtensorMap tmV, Args a)
+__global__ void __launch_bounds__(MainLayout<DL, MT>::THREADS, 2)
+    latent_main_kernel(const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmK,
+                       const __grid_constant__ CUtensorMap tmV, Args a)
 {
     using Ly = MainLayout<DL, MT>;
     constexpr int NST = Ly::NST;
@@ -544,14 +639,14 @@ __global__ void __launch_bounds__(kMainThreads2) latent_main_kernel(const __grid
                                                           ~uintptr_t(1023));
     const uint32_t sbase = smem_u32(sm);
     uint64_t *full = reinterpret_cast<uint64_t *>(sm + Ly::BAR);
-    uint64_t *empty = full + NST;
+    uint64_t *empty = full + NST;  // (with a producer warp)
     volatile int *abort_flag = reinterpret_cast<volatile int *>(empty + NST);
     float *red = reinterpret_cast<float *>(sm + Ly::RED);
     int *pref = reinterpret_cast<int *>(sm + Ly::PREF);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     grid_dep_launch();  // the merge kernel may launch; it waits for this grid to finish
 
-    // lengths -> latent splits per sequence, prefix sums (every CTA, the same)
+    // lengths -> latent units per sequence, prefix sums (every CTA, the same)
     const int B = a.B, cap = a.maxp * kTok;
     auto len_of = [&](int b) {
         const int L = __ldg(a.seq_lens + b);
@@ -591,9 +686,24 @@ __global__ void __launch_bounds__(kMainThreads2) latent_main_kernel(const __grid
         mbar_init_fence();
     }
     __syncthreads();
-    const int n_lat = pref[B], n_items = n_lat + B * a.Hkv;
-    auto item_of = [&](int k) {
-        Item it;
+    // This CTA's run [k0, k1) of the items: those whose estimated start falls in
+    // its share of the total (a page costs its width plus a stage's fixed part)
+    const int n_lat = pref[B];
+    int k0, k1;
+    {
+        const long long cu = kPagesPerSplit * (DL / 64 + 2), cw = 3 * ((a.w + kTok - 1) / kTok + 1);
+        const long long lat = n_lat * cu, total = lat + (long long)B * a.Hkv * cw;
+        auto first = [&](long long c) {  // the first item that starts at c or later
+            return (int)(c <= lat ? (c + cu - 1) / cu : n_lat + (c - lat + cw - 1) / cw);
+        };
+        // (few items: one CTA per SM, the first half of the grid)
+        const int ctas = n_lat + B * a.Hkv <= (int)gridDim.x / 2 ? gridDim.x / 2 : gridDim.x;
+        const long long share = (total + ctas - 1) / ctas;
+        k0 = first(min(total, share * blockIdx.x));
+        k1 = first(min(total, share * (blockIdx.x + 1)));
+    }
+    auto segment_of = [&](int k) {
+        Segment it;
         if (k < n_lat) {
             int lo = 0, hi = B - 1;  // the last b with pref[b] <= k
             while (lo < hi) {
@@ -606,251 +716,183 @@ __global__ void __launch_bounds__(kMainThreads2) latent_main_kernel(const __grid
             it.latent = true;
             it.b = lo;
             it.part = k - pref[lo];
+            it.units = min(k1, pref[lo + 1]) - k;
             const int L = len_of(lo), Lg = L > a.w ? L - a.w : 0;
-            const int t0 = it.part * kSplitTok, t1 = min(Lg, t0 + kSplitTok);
+            const int t0 = it.part * kSplitTok, t1 = min(Lg, t0 + it.units * kSplitTok);
             it.npg = (t1 - t0 + kTok - 1) / kTok;
         } else {
             const int r = k - n_lat;
             it.latent = false;
             it.b = r / a.Hkv;
             it.part = r % a.Hkv;
+            it.units = 1;
             const int nwin = min(len_of(it.b), a.w);
             it.npg = (nwin + kTok - 1) / kTok;
         }
         return it;
     };
 
-    if (warp == 4) {
-        // ------------------------------------------------ producer
-        if (lane == 0) {
-            prefetch_tensormap(&tmC);
-            prefetch_tensormap(&tmK);
-            prefetch_tensormap(&tmV);
-            int gp = 0;
-            for (int k = blockIdx.x; k < n_items; k += gridDim.x) {
-                const Item it = item_of(k);
-                for (int p = 0; p < it.npg; ++p, ++gp) {
-                    const int st = gp % NST;
-                    if (gp >= NST && !mbar_wait(&empty[st], ((gp / NST) - 1) & 1, abort_flag))
-                        goto done;
-                    unsigned char *dst = sm + Ly::STG + st * Ly::CST;
-                    if (it.latent) {
-                        int pid = __ldg(a.block_table + (size_t)it.b * a.maxp + it.part * kPagesPerSplit + p);
-                        if (pid < 0 || pid >= a.num_pages) {
-                            report(a.status, DAR_ERR_CAPACITY);
-                            pid = 0;
-                        }
-                        mbar_expect_tx(&full[st], kTok * DL * 2);
-#pragma unroll
-                        for (int cb = 0; cb < DL / 64; ++cb)
-                            tma_load_2d(dst + cb * 8192, &tmC, cb * 64, pid * kTok, &full[st]);
-                    } else {
-                        const int row = (it.b * a.Hkv + it.part) * a.w + p * kTok;
-                        mbar_expect_tx(&full[st], 2 * 8192);
-                        tma_load_2d(dst, &tmK, 0, row, &full[st]);
-                        tma_load_2d(dst + 8192, &tmV, 0, row, &full[st]);
-                    }
-                }
+    // One thread: the next page or tile of the run into its stage of the ring.  The
+    // page's index is loaded a call ahead.
+    int pk = k0, pp = 0, pi = 0, pid = 0;
+    Segment pit{};
+    auto look_ahead = [&] {  // (pit, pp) is the page to fetch next; moves on past finished segments
+        while (pp == pit.npg) {
+            if (pk >= k1) {
+                pit.npg = -1;
+                return;
             }
-        done:;
+            pit = segment_of(pk);
+            pk += pit.units;
+            pp = 0;
         }
-        return;
+        if (pit.latent)
+            pid = __ldg(a.block_table + (size_t)pit.b * a.maxp + pit.part * kPagesPerSplit + pp);
+    };
+    auto fetch = [&] {
+        const int st = pi++ % NST;
+        unsigned char *dst = sm + Ly::STG + st * Ly::CST;
+        if (pit.latent) {
+            if (pid < 0 || pid >= a.num_pages) {
+                report(a.status, DAR_ERR_CAPACITY);
+                pid = 0;
+            }
+            mbar_expect_tx(&full[st], kTok * DL * 2);
+#pragma unroll
+            for (int cb = 0; cb < DL / 64; ++cb)
+                tma_load_2d(dst + cb * 8192, &tmC, cb * 64, pid * kTok, &full[st]);
+        } else {
+            const int row = (pit.b * a.Hkv + pit.part) * a.w + pp * kTok;
+            mbar_expect_tx(&full[st], 2 * 8192);
+            tma_load_2d(dst, &tmK, 0, row, &full[st]);
+            tma_load_2d(dst + 8192, &tmV, 0, row, &full[st]);
+        }
+        ++pp;
+        look_ahead();
+    };
+    const int producer = Ly::kProducer ? kConsumerThreads : 0;  // the thread that issues the copies
+    if (tid == producer) {
+        prefetch_tensormap(&tmC);
+        prefetch_tensormap(&tmK);
+        prefetch_tensormap(&tmV);
+        look_ahead();
+        while (pit.npg >= 0 && pi < NST)
+            fetch();
+        if constexpr (Ly::kProducer)
+            while (pit.npg >= 0 && mbar_wait(&empty[pi % NST], (pi / NST - 1) & 1, abort_flag))
+                fetch();
     }
+    if (warp == 4)
+        return;
 
-    // ---------------------------------------------------- consumers (warps 0-3)
     grid_dep_wait();  // q~ comes from the prep kernel
-    const int grp = lane >> 2, tig = lane & 3;
     int gp = 0;
+    // A wait that gives up sets the abort flag, after which every later one gives
+    // up soon: the loops run on (the barriers keep their counts) and the CTA
+    // reports the error at its end.
     bool ok = true;
-    for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
-        const Item it = item_of(k);
+    // wait for a stage and zero its rows past the segment's last token (their P
+    // is 0; 0 * NaN must not arise; the barriers in stage() order the writes)
+    auto stage_wait = [&](int st, int ntok, int width) {
+        ok = mbar_wait(&full[st], (gp / NST) & 1, abort_flag) && ok;
+        if (ntok < kTok) {
+            unsigned char *t = sm + Ly::STG + st * Ly::CST;
+            for (int i = tid; i < (kTok - ntok) * (width / 8); i += kConsumerThreads) {
+                const int r = ntok + i / (width / 8), ch = i % (width / 8);
+                *reinterpret_cast<uint4 *>(t + (ch / 8) * 8192 + r * 128 + (((ch % 8) ^ (r & 7)) << 4)) =
+                    make_uint4(0u, 0u, 0u, 0u);
+            }
+            fence_proxy_async_smem();  // these writes precede the stage's next TMA fill
+        }
+    };
+    auto run = [&](auto &rows, const Segment &it, int tokens, int width, uint32_t voff) {
+        for (int p = 0; p < it.npg; ++p, ++gp) {
+            const int st = gp % NST, ntok = min(kTok, tokens - p * kTok);
+            stage_wait(st, ntok, width);
+            const uint32_t t = sbase + Ly::STG + st * Ly::CST;
+            rows.stage(t, t + voff, sm + Ly::P, red, ntok, a.c2, warp, lane, [&] {
+                if (!Ly::kProducer && tid == 0 && gp > 0 && pit.npg >= 0)
+                    fetch();  // into the stage of gp - 1
+            });
+            if constexpr (Ly::kProducer) {
+                __syncwarp();
+                if (lane == 0)
+                    mbar_arrive(&empty[st]);
+            }
+        }
+    };
+    for (int k = k0; k < k1;) {
+        const Segment it = segment_of(k);
+        k += it.units;
         if (it.npg == 0)
             continue;
-        if (it.latent) {
-            // q~ rows of every head (zero past Hq) into the A-operand tile
-            for (int i = tid; i < MT * 16 * (DL / 8); i += kConsumerThreads) {
-                const int r = i / (DL / 8), ch = i % (DL / 8);
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (r < a.Hq)
-                    v = *reinterpret_cast<const uint4 *>(a.qt + ((size_t)it.b * a.Hq + r) * DL + ch * 8);
-                *reinterpret_cast<uint4 *>(sm + Ly::QA + (ch / 8) * (MT * 16 * 128) + r * 128 +
-                                           (((ch % 8) ^ (r & 7)) << 4)) = v;
-            }
-        } else {
-            // q rows of KV head g's query heads (zero past G) into a 64-wide A tile
-            for (int i = tid; i < 16 * 8; i += kConsumerThreads) {
-                const int r = i / 8, ch = i % 8;
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (r < a.G)
-                    v = *reinterpret_cast<const uint4 *>(static_cast<const bf16 *>(a.q) +
-                                                         ((size_t)it.b * a.Hq + it.part * a.G + r) * 64 + ch * 8);
-                *reinterpret_cast<uint4 *>(sm + Ly::QA + r * 128 + ((ch ^ (r & 7)) << 4)) = v;
-            }
-        }
-        consumer_sync<MT>();
         const int L = len_of(it.b), Lg = L > a.w ? L - a.w : 0, nwin = min(L, a.w);
-        // Wait for a stage, zero its rows past the item's last token (their P is
-        // 0; 0 * NaN must not arise), then one barrier so every consumer thread
-        // takes the same decision if any wait gave up (the flag is set first).
-        auto stage_wait = [&](int st, int ntok, int rows_w) -> bool {
-            const bool got = mbar_wait(&full[st], (gp / NST) & 1, abort_flag);
-            if (got && ntok < kTok) {
-                unsigned char *t = sm + Ly::STG + st * Ly::CST;
-                for (int i = tid; i < (kTok - ntok) * (rows_w / 8); i += kConsumerThreads) {
-                    const int r = ntok + i / (rows_w / 8), ch = i % (rows_w / 8);
-                    *reinterpret_cast<uint4 *>(t + (ch / 8) * 8192 + r * 128 + (((ch % 8) ^ (r & 7)) << 4)) =
-                        make_uint4(0u, 0u, 0u, 0u);
-                }
-                fence_proxy_async_smem();  // these writes precede the stage's next TMA fill
-            }
-            consumer_sync<MT>();
-            return *abort_flag == 0;
-        };
-        auto release = [&](int st) {
-            __syncwarp();
-            if (lane == 0)
-                mbar_arrive(&empty[st]);
-        };
         if (it.latent) {
-            float o[MT][DL / 32][4];
-            float mrun[MT][2], lpart[MT][2];
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt) {
-#pragma unroll
-                for (int nt = 0; nt < DL / 32; ++nt)
-                    o[mt][nt][0] = o[mt][nt][1] = o[mt][nt][2] = o[mt][nt][3] = 0.f;
-                mrun[mt][0] = mrun[mt][1] = -INFINITY;
-                lpart[mt][0] = lpart[mt][1] = 0.f;
-            }
-            const int t0 = it.part * kSplitTok, t1 = min(Lg, t0 + kSplitTok);
-            for (int p = 0; p < it.npg; ++p, ++gp) {
-                const int st = gp % NST, ntok = min(kTok, t1 - (t0 + p * kTok));
-                if (!stage_wait(st, ntok, DL)) {
-                    ok = false;
-                    break;
-                }
-                const uint32_t t = sbase + Ly::STG + st * Ly::CST;
-                run_stage<DL, MT, MT>(sbase + Ly::QA, t, t, sm + Ly::P, sbase + Ly::P, red, ntok, a.c2, o, mrun,
-                                      lpart, warp, lane);
-                release(st);
-            }
-            if (!ok)
-                break;
-            // record (O_lat, m, l) of every head: row sums across the quad, then the warps
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-                for (int hr = 0; hr < 2; ++hr) {
-                    float ls = lpart[mt][hr];
-                    ls += __shfl_xor_sync(0xffffffffu, ls, 1);
-                    ls += __shfl_xor_sync(0xffffffffu, ls, 2);
-                    lpart[mt][hr] = ls;
-                }
-            consumer_sync<MT>();
-            if (tig == 0)
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt) {
-                    red[warp * MT * 16 + mt * 16 + grp] = lpart[mt][0];
-                    red[warp * MT * 16 + mt * 16 + grp + 8] = lpart[mt][1];
-                }
-            consumer_sync<MT>();
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-                for (int hr = 0; hr < 2; ++hr) {
-                    const int row = mt * 16 + grp + 8 * hr;
-                    if (row >= a.Hq)
-                        continue;
-                    // records of one (b, h) are consecutive over the splits
-                    float *rec = a.rec_lat + (((size_t)it.b * a.Hq + row) * a.nspl + it.part) * (DL + 2);
-#pragma unroll
-                    for (int nt = 0; nt < DL / 32; ++nt) {
-                        const int col = warp * (DL / 4) + 8 * nt + 2 * tig;
-                        *reinterpret_cast<float2 *>(rec + col) =
-                            make_float2(o[mt][nt][2 * hr], o[mt][nt][2 * hr + 1]);
-                    }
-                    if (warp == 0 && tig == 0) {
-                        rec[DL] = mrun[mt][hr];
-                        rec[DL + 1] =
-                            red[row] + red[MT * 16 + row] + red[2 * MT * 16 + row] + red[3 * MT * 16 + row];
-                    }
-                }
+            Rows<DL, MT> rows;
+            rows.start(a.qt + (size_t)it.b * a.Hq * DL, a.Hq, warp, lane);
+            run(rows, it, Lg - it.part * kSplitTok, DL, 0);
+            // records of one (b, h) are consecutive over the units
+            auto rec = [&](int row) {
+                return a.rec_lat + (((size_t)it.b * a.Hq + row) * a.nspl + it.part) * (DL + 2);
+            };
+            rows.finish(red, a.Hq, warp, lane, rec);
+            for (int i = tid; i < (it.units - 1) * a.Hq; i += kConsumerThreads)  // the other units' slots: empty
+                *reinterpret_cast<float2 *>(rec(i % a.Hq) + (i / a.Hq + 1) * (DL + 2) + DL) =
+                    make_float2(-INFINITY, 0.f);
         } else {
-            float o[1][2][4];
-            float mrun[1][2] = {{-INFINITY, -INFINITY}}, lpart[1][2] = {{0.f, 0.f}};
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-                o[0][nt][0] = o[0][nt][1] = o[0][nt][2] = o[0][nt][3] = 0.f;
-            for (int p = 0; p < it.npg; ++p, ++gp) {
-                const int st = gp % NST, ntok = min(kTok, nwin - p * kTok);
-                // zero both tiles' rows past the window (K block at +0, V block at +8192)
-                if (!stage_wait(st, ntok, 128)) {
-                    ok = false;
-                    break;
-                }
-                const uint32_t t = sbase + Ly::STG + st * Ly::CST;
-                run_stage<64, 1, 1>(sbase + Ly::QA, t, t + 8192, sm + Ly::P, sbase + Ly::P, red, ntok, a.c2, o, mrun,
-                                    lpart, warp, lane);
-                release(st);
-            }
-            if (!ok)
-                break;
-#pragma unroll
-            for (int hr = 0; hr < 2; ++hr) {
-                float ls = lpart[0][hr];
-                ls += __shfl_xor_sync(0xffffffffu, ls, 1);
-                ls += __shfl_xor_sync(0xffffffffu, ls, 2);
-                lpart[0][hr] = ls;
-            }
-            consumer_sync<MT>();
-            if (tig == 0) {
-                red[warp * 16 + grp] = lpart[0][0];
-                red[warp * 16 + grp + 8] = lpart[0][1];
-            }
-            consumer_sync<MT>();
-#pragma unroll
-            for (int hr = 0; hr < 2; ++hr) {
-                const int row = grp + 8 * hr;
-                if (row >= a.G)
+            // K block of a stage at +0, V block at +8192
+            auto window = [&](auto &rows) {
+                rows.start(static_cast<const bf16 *>(a.q) + ((size_t)it.b * a.Hq + it.part * a.G) * 64, a.G, warp,
+                           lane);
+                run(rows, it, nwin, 128, 8192);
+                rows.finish(red, a.G, warp, lane, [&](int row) {
+                    return a.rec_win + ((size_t)it.b * a.Hq + it.part * a.G + row) * 66;
+                });
+            };
+            if constexpr (MT > 1) {
+                if (a.G > 16) {
+                    Rows<64, MT> rows;
+                    window(rows);
                     continue;
-                float *rec = a.rec_win + ((size_t)it.b * a.Hq + it.part * a.G + row) * 66;
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt) {
-                    const int col = warp * 16 + 8 * nt + 2 * tig;
-                    *reinterpret_cast<float2 *>(rec + col) = make_float2(o[0][nt][2 * hr], o[0][nt][2 * hr + 1]);
-                }
-                if (warp == 0 && tig == 0) {
-                    rec[64] = mrun[0][hr];
-                    rec[65] = red[row] + red[16 + row] + red[32 + row] + red[48 + row];
                 }
             }
+            Rows<64, 1> rows;
+            window(rows);
         }
-        consumer_sync<MT>();  // the A tile and `red` are reused by the next item
     }
-    if (!ok && tid == 0)
+    if (!ok && lane == 0)
         report(a.status, DAR_ERR_DEVICE);
 }
 
 // ---------------------------------------------------------------- decode: merge
 
-// Block (g, 4 rows of KV head g): A_V^g staged in shared memory by one bulk
+// A load the compiler keeps in place (a batch of them is issued before the first
+// use; with the registers for it, see the launch bounds, the merge of 31 records of
+// 32 heads took 10 us, 25 without).
+__device__ __forceinline__ float2 ld_early_f2(const float *p)
+{
+    float2 r;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "l"(p));
+    return r;
+}
+
+// Block (g, a few rows of KV head g): A_V^g staged in shared memory by one bulk
 // copy (before the dependency wait: it does not come from the main kernel),
 // then one warp per row: combine the window record and the sequence's latent splits
 // (log-sum-exp, one split per lane), lift the latent sum with A_V, divide.
 template <int DL>
-__global__ void __launch_bounds__(128) latent_merge_kernel(Args a)
+__global__ void __launch_bounds__(kRowThreads, 2) latent_merge_kernel(Args a)
 {
     extern __shared__ __align__(16) float msm[];
     float *avs = msm;                  // [DL][64]
-    float *olat = avs + DL * 64;       // [4 warps][DL]
-    float *fs = olat + 4 * DL;         // [4 warps][32]
-    uint64_t *bar = reinterpret_cast<uint64_t *>(fs + 4 * 32);
+    float *olat = avs + DL * 64;       // [warps][DL]
+    uint64_t *bar = reinterpret_cast<uint64_t *>(olat + kRowsPerBlock * DL);
     const int g = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (!stage_matrix(avs, a.Av + (size_t)g * DL * 64, DL * 64 * 4, bar, a.status))
         return;
     grid_dep_wait();  // the main kernel's records
     const int nrows = a.B * a.G;
-    for (int r = blockIdx.y * kRowsPerBlock + warp; r < min(nrows, (int)(blockIdx.y + 1) * kRowsPerBlock); r += 4) {
+    if (const int r = blockIdx.y * (blockDim.x >> 5) + warp; r < nrows) {
         const int b = r / a.G, h = g * a.G + r % a.G, row = b * a.Hq + h;
         int L = __ldg(a.seq_lens + b);
         if (L < 0 || L > a.maxp * kTok)
@@ -860,9 +902,8 @@ __global__ void __launch_bounds__(128) latent_merge_kernel(Args a)
         const float *rw = a.rec_win + (size_t)row * 66;
         const float *rl0 = a.rec_lat + (size_t)row * a.nspl * (DL + 2);  // this row's splits, consecutive
         const float mw = L > 0 ? rw[64] : -INFINITY;
-        // the splits' maxima and sums, one split per lane (32 at a time); the
-        // weighted sum of their O in batches of 8 splits with every load issued
-        // before it is used
+        // the splits' maxima and sums, one slot per lane (32 at a time); the
+        // weighted sum of their O with every load of a batch issued before it is used
         float M = mw;
         for (int s2 = lane; s2 < ns; s2 += 32)
             M = fmaxf(M, rl0[s2 * (DL + 2) + DL]);
@@ -881,25 +922,33 @@ __global__ void __launch_bounds__(128) latent_merge_kernel(Args a)
                 f = ex2_approx(rl[DL] - M);
                 l += f * rl[DL + 1];
             }
-            fs[warp * 32 + lane] = f;
-            __syncwarp();
-            const int n = min(32, ns - s0);
-            for (int j0 = 0; j0 < n; j0 += 8) {
-                float x[8][DL / 32];
+            // slots with a weight (empty ones hold no O), in batches of 8
+            for (unsigned left = __ballot_sync(0xffffffffu, f != 0.f); left;) {
+                const float *src[8];
+                float fj[8];
+                float2 x[8][DL / 64];
+                const int at0 = __ffs(left) - 1;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {  // past the last slot: the first one again, with weight 0
+                    const int at = left ? __ffs(left) - 1 : at0;
+                    const float fa = __shfl_sync(0xffffffffu, f, at);
+                    fj[j] = left ? fa : 0.f;
+                    src[j] = rl0 + (s0 + at) * (DL + 2) + 2 * lane;
+                    left &= left - 1;
+                }
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
 #pragma unroll
-                    for (int e = 0; e < DL / 32; ++e)
-                        x[j][e] = j0 + j < n ? rl0[(s0 + j0 + j) * (DL + 2) + lane + 32 * e] : 0.f;
+                    for (int e = 0; e < DL / 64; ++e)
+                        x[j][e] = ld_early_f2(src[j] + 64 * e);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float fj = j0 + j < n ? fs[warp * 32 + j0 + j] : 0.f;
+                for (int j = 0; j < 8; ++j)
 #pragma unroll
-                    for (int e = 0; e < DL / 32; ++e)
-                        acc[e] = fmaf(fj, x[j][e], acc[e]);
-                }
+                    for (int e = 0; e < DL / 64; ++e) {
+                        acc[2 * e] = fmaf(fj[j], x[j][e].x, acc[2 * e]);
+                        acc[2 * e + 1] = fmaf(fj[j], x[j][e].y, acc[2 * e + 1]);
+                    }
             }
-            __syncwarp();
         }
 #pragma unroll
         for (int o = 16; o; o >>= 1)
@@ -908,8 +957,8 @@ __global__ void __launch_bounds__(128) latent_merge_kernel(Args a)
         if (L > 0)
             l += fw * rw[65];
 #pragma unroll
-        for (int e = 0; e < DL / 32; ++e)
-            olat[warp * DL + lane + 32 * e] = acc[e];
+        for (int e = 0; e < DL / 64; ++e)  // columns 2 lane + 64 e, + 1
+            *reinterpret_cast<float2 *>(olat + warp * DL + 2 * lane + 64 * e) = make_float2(acc[2 * e], acc[2 * e + 1]);
         __syncwarp();
         float o0 = L > 0 ? fw * rw[lane] : 0.f, o1 = L > 0 ? fw * rw[lane + 32] : 0.f;
 #pragma unroll 16
@@ -967,7 +1016,7 @@ static cudaError_t decode_t(const Args &a, const void *pool_c, const void *win_k
     using Ly = MainLayout<DL, MT>;
     const size_t smem = 1024 + Ly::TOTAL;
     constexpr size_t prep_smem = (size_t)64 * DL * sizeof(float) + 16;
-    constexpr size_t merge_smem = ((size_t)DL * 64 + 4 * DL + 4 * 32) * sizeof(float) + 16;
+    constexpr size_t merge_smem = ((size_t)DL * 64 + kRowsPerBlock * DL) * sizeof(float) + 16;
     static PerDeviceOnce once;  // records the SM count
     int sms = 0;
     cudaError_t e = per_device_once(
@@ -997,8 +1046,14 @@ static cudaError_t decode_t(const Args &a, const void *pool_c, const void *win_k
         return cudaErrorInvalidValue;
     // prep starts after all earlier work on the stream; main and merge are
     // launched programmatically (each waits in-kernel for what it reads)
-    const dim3 rgrid(a.Hkv, (a.B * a.G + kRowsPerBlock - 1) / kRowsPerBlock);
-    latent_prep_kernel<DL><<<rgrid, 128, prep_smem, s>>>(a);
+    // prep and merge: few rows are spread over the chip, many share a staged
+    // matrix (4 sequences, 4 KV heads, G 4: 16.5 us with 2 rows a block, 17.7 with
+    // 8; 64 sequences, 8 KV heads, G 4: 4 rows a block cost 3 us more than 8)
+    int rows = 2;
+    while (rows < kRowsPerBlock && a.Hkv * ((a.B * a.G + rows - 1) / rows) > sms)
+        rows *= 2;
+    const dim3 rgrid(a.Hkv, (a.B * a.G + rows - 1) / rows);
+    latent_prep_kernel<DL><<<rgrid, 32 * rows, prep_smem, s>>>(a);
     cudaLaunchAttribute pdl[1];
     pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
@@ -1007,13 +1062,13 @@ static cudaError_t decode_t(const Args &a, const void *pool_c, const void *win_k
     cfg.attrs = pdl;
     cfg.numAttrs = 1;
     cfg.gridDim = dim3(2 * (sms > 0 ? sms : 1));  // persistent: two CTAs per SM
-    cfg.blockDim = dim3(kMainThreads2);
+    cfg.blockDim = dim3(Ly::THREADS);
     cfg.dynamicSmemBytes = smem;
     e = cudaLaunchKernelEx(&cfg, latent_main_kernel<DL, MT>, tm[0], tm[1], tm[2], a);
     if (e != cudaSuccess)
         return e;
     cfg.gridDim = rgrid;
-    cfg.blockDim = dim3(128);
+    cfg.blockDim = dim3(32 * rows);
     cfg.dynamicSmemBytes = merge_smem;
     e = cudaLaunchKernelEx(&cfg, latent_merge_kernel<DL>, a);
     if (e != cudaSuccess)
