@@ -10,11 +10,13 @@ namespace dar {
 
 // A CTA stages kStageBytesBulk of rows in shared memory, 16-byte chunk c of row
 // r at chunk c ^ (r & 7), so that a warp reading one chunk of 32 different rows
-// touches every bank group once.  A thread holds 64 sums (4 rows of 16 columns,
-// 2 of 32), so that one 16-byte read of W[t][c..c+3] (the same address in the
-// whole warp) feeds 8 to 16 products; 64 columns are shared out over four
-// threads per row (all of a row in one thread fed 4: a prompt append at
-// d_down 64 took 418 us, 375 so; at 32, 165 us over two threads, 156 in one).
+// touches every bank group once.  A thread holds 16 to 64 sums: one 16-byte read of
+// W[t][c..c+3] (the same address in the whole warp) feeds a product for each of its
+// rows, and fewer sums per thread put more warps on an SM while tiles arrive.
+// Measured, columns x rows per thread, 32 prompts of 1000 to 4096 tokens, 12 heads,
+// appended, us: d_down 8 8x4 97, 8x2 81, 8x1 86; 16 16x4 141, 16x2 117, 8x4 118,
+// 8x2 127; 32 32x2 201, 16x4 215, 16x2 208; 64 16x4 494, 16x2 488 (but 230 instead
+// of 195 for the bulk projection of 1 M rows), 32x2 503.
 constexpr int kStageBytesBulk = 32 << 10;
 
 template <typename T>
@@ -30,7 +32,7 @@ __host__ __device__ constexpr int cols_per_thread()
 template <int DD>
 __host__ __device__ constexpr int rows_per_thread()
 {
-    return DD == 32 ? 2 : 4;
+    return DD == 64 ? 4 : 2;
 }
 // Threads that share out the columns of a row.
 template <int DD>
@@ -95,6 +97,7 @@ template <typename T, int CW>
 __device__ __forceinline__ void store_row(T *o, const float (&x)[CW])
 {
     constexpr int OE = 16 / sizeof(T);
+    static_assert(CW % OE == 0, "whole 16-byte words");
 #pragma unroll
     for (int c = 0; c < CW; c += OE) {
         uint32_t u[4];
