@@ -818,8 +818,13 @@ __global__ void __launch_bounds__(kDecThreads, 1)
     // kept if the counts hold.
 #pragma unroll 1
     for (int pass = 0;; ++pass) {
-        sp = make_split(s_pre[a.B] * per_chunk, gridDim.x * kDecWarps);
-        rid = blockIdx.x * kDecWarps + warp;
+        const int stages = s_pre[a.B] * per_chunk, warps = gridDim.x * kDecWarps;
+        // With fewer stages than warps each is a range of its own, spread over
+        // the SMs, and the other warps stay idle: cut into as many ranges as
+        // warps, a group's few parts would lie among dozens of empty ranges, which
+        // its merge had to step over (one sequence of 101 tokens, 8 heads: 19.7 us, now 9.3).
+        sp = make_split(stages, max(1, min(stages, warps)));
+        rid = stages < warps ? warp * gridDim.x + blockIdx.x : blockIdx.x * kDecWarps + warp;
         lo = sp.lo(rid);
         hi = sp.lo(rid + 1);
         iss_s = lo;
