@@ -199,7 +199,7 @@ dar_status prepare_decode(const dar_cache *cache, int32_t Hq, const void *q, con
     a->maxp = cache->max_pages_per_seq;
     a->num_pages = cache->num_pages;
     a->qscale = default_scale(scale, cache->d) * kLog2e;
-    a->prep_overlaps_prev = 0;
+    a->prep = dar::kPrepAfterAll;
     return ok();
 }
 
@@ -286,7 +286,7 @@ dar_status dar_attn_decode(const dar_cache *cache, int32_t Hq, const void *q, co
     dar_status s = prepare_decode(cache, Hq, q, Uk, Uv, scale, out, workspace, workspace_bytes, &a, &empty);
     if (s != DAR_OK || empty)
         return s;
-    a.prep_overlaps_prev = 0;  // the kernel before this call is the caller's: wait for it
+    a.prep = dar::kPrepAfterAll;  // the kernel before this call is the caller's: wait for it
     return from_cuda(dar::launch_decode(cache->dtype, cache->d_down, a,
                                         static_cast<cudaStream_t>(stream)),
                      "dar_attn_decode launch");
@@ -308,7 +308,7 @@ dar_status dar_attn_decode_direct(const dar_cache *cache, int32_t Hq, const void
         return fail(DAR_ERR_INVALID_ARG, "qd must be 16-byte aligned");
     a.qd = qd;
     a.qd_ratio = default_scale(scale_down, cache->d_down) / default_scale(scale, cache->d);
-    a.prep_overlaps_prev = 0;
+    a.prep = dar::kPrepAfterAll;
     return from_cuda(dar::launch_decode(cache->dtype, cache->d_down, a, static_cast<cudaStream_t>(stream)),
                      "dar_attn_decode_direct launch");
 }
@@ -329,16 +329,16 @@ dar_status dar_decode_step(const dar_cache *cache, const void *k_new, const void
     if (s != DAR_OK)
         return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (dec_empty)
+        return ok();  // B = 0: nothing to append either
     if (!app_empty) {
-        s = from_cuda(dar::launch_cache_append(cache->dtype, cache->d_down, ap, st), "dar_decode_step append launch");
+        bool prepared = false;
+        s = from_cuda(dar::launch_step_front(cache->dtype, cache->d_down, ap, dc, st, &prepared),
+                      "dar_decode_step append launch");
         if (s != DAR_OK)
             return s;
+        dc.prep = prepared ? dar::kPrepDone : dar::kPrepOverlaps;
     }
-    if (dec_empty)
-        return ok();
-    // the kernel just before the decode is the append above, which writes
-    // neither q nor Uk: the decode's query-side set-up may overlap it
-    dc.prep_overlaps_prev = app_empty ? 0 : 1;
     return from_cuda(dar::launch_decode(cache->dtype, cache->d_down, dc, st), "dar_decode_step decode launch");
 }
 

@@ -5,9 +5,9 @@
 //
 //  prep     q~ = q Uk^T for every query row (W_up absorbed into the query,
 //           exact by linearity of Eq. 2) and zeroed group counters.  Neither
-//           needs the cache, so when the kernel before it is this library's
-//           cache append (dar_decode_step) prep is launched with programmatic
-//           stream serialisation and overlaps it; it waits for that kernel
+//           needs the cache, so dar_decode_step runs it as further blocks of
+//           the append of a few tokens; behind an append of many it is launched
+//           with programmatic stream serialisation and waits for that kernel
 //           before exiting.  Otherwise it starts after all earlier work.
 //           The stream kernel is always launched programmatically after prep.
 //  stream   split-K over the sequence, balanced per warp (stream-K).  The
@@ -58,6 +58,7 @@
 
 #include "dar_common.cuh"
 #include "dar_launch.h"
+#include "dar_prep.cuh"
 #include "dar_sm100.cuh"
 
 namespace dar {
@@ -157,57 +158,16 @@ constexpr size_t decode_smem_bytes(int B)
 
 // --------------------------------------------------------------------- prep
 
-// q~ = q Uk^T for every (b, h) row, one row per warp (fp32, four partial sums
-// over t mod 4), and zeroed group counters.  In the direct variant of Sec. 5
-// (a.qd set) q~ is the row's own d_down query times scale_down / scale, so the
-// stream kernel's global scores scale * q~ . k^D are scale_down * q^D . k^D.  Neither depends on the cache, so
-// when launched programmatically after the cache append (which writes neither
+// The query-side set-up (dar_prep.cuh).  It does not need the cache, so when
+// launched programmatically after the cache append (which writes neither
 // q nor Uk) this kernel runs while the append finishes; it waits for the
 // kernel before it before exiting, so the stream kernel, which waits for this
 // one, sees the finished cache.
 template <typename T, int DD>
 __global__ void __launch_bounds__(kPrepThreads) decode_prep_kernel(DecodeArgs a)
 {
-    constexpr int QR = DD > 32 ? 2 : 1;  // q~ entries per lane
-    constexpr int kWarps = kPrepThreads / 32;
     sm100::grid_dep_launch();  // the stream kernel may start its set-up now
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rows = a.B * a.Hq;
-    for (int row = blockIdx.x * kWarps + warp; row < rows; row += gridDim.x * kWarps) {
-        if (a.qd) {  // direct variant: the row's own d_down query, rescaled to the local scale
-            for (int c = lane; c < DD; c += 32)
-                a.qt[(size_t)row * DD + c] = to_f32(static_cast<const T *>(a.qd)[(size_t)row * DD + c]) * a.qd_ratio;
-            continue;
-        }
-        const T *qrow = static_cast<const T *>(a.q) + (size_t)row * kHeadDim;
-        const float q0 = to_f32(qrow[lane]), q1 = to_f32(qrow[lane + 32]);
-        const int g = (row % a.Hq) / a.G;
-#pragma unroll
-        for (int rr = 0; rr < QR; ++rr) {
-            const int c = lane + 32 * rr;
-            const float4 *u4 = reinterpret_cast<const float4 *>(a.Uk + ((size_t)g * DD + (c < DD ? c : 0)) * kHeadDim);
-            float4 uk[kHeadDim / 4];
-#pragma unroll
-            for (int t4 = 0; t4 < kHeadDim / 4; ++t4)
-                uk[t4] = c < DD ? __ldg(u4 + t4) : make_float4(0.f, 0.f, 0.f, 0.f);
-            float p[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int t4 = 0; t4 < kHeadDim / 4; ++t4) {
-                const float uu[4] = {uk[t4].x, uk[t4].y, uk[t4].z, uk[t4].w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int t = 4 * t4 + e;
-                    const float qv = __shfl_sync(0xffffffffu, t < 32 ? q0 : q1, t & 31);
-                    p[e] = fmaf(qv, uu[e], p[e]);
-                }
-            }
-            if (c < DD)
-                a.qt[(size_t)row * DD + c] = (p[0] + p[1]) + (p[2] + p[3]);
-        }
-    }
-    const int ngroups = a.B * a.Hkv * a.HS;  // group counters, then the pool's claim counter
-    for (int i = blockIdx.x * kPrepThreads + threadIdx.x; i <= ngroups; i += gridDim.x * kPrepThreads)
-        a.counters[i] = 0;
+    prep_rows<T, DD>(a, blockIdx.x, gridDim.x);
     sm100::grid_dep_wait();
 }
 
@@ -1405,27 +1365,28 @@ static cudaError_t decode_t(const DecodeArgs &a, cudaStream_t s)
         &ctas);
     if (e != cudaSuccess)
         return e;
-    const int rows = a.B * a.Hq;
-    const int prep_blocks = min(2 * ctas, max(1, (rows + kPrepThreads / 32 - 1) / (kPrepThreads / 32)));
     // The stream kernel always uses programmatic launch: it sets up while prep
     // drains (prep is this library's own kernel and writes nothing the set-up
     // reads).  prep itself reads q and Uk before its dependency wait, so it may
     // overlap the kernel before it only when the caller vouches that this
-    // kernel writes neither (a.prep_overlaps_prev: this library's own cache
-    // append, launched by dar_decode_step); otherwise it starts after all
-    // earlier work on the stream has finished.
+    // kernel writes neither (kPrepOverlaps: this library's own cache append,
+    // launched by dar_decode_step); otherwise it starts after all earlier work
+    // on the stream has finished.
     cudaLaunchAttribute pdl[1];
     pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.stream = s;
     cfg.attrs = pdl;
-    cfg.numAttrs = a.prep_overlaps_prev ? 1 : 0;
-    cfg.gridDim = dim3(prep_blocks);
-    cfg.blockDim = dim3(kPrepThreads);
-    e = cudaLaunchKernelEx(&cfg, decode_prep_kernel<T, DD>, a);
-    if (e != cudaSuccess)
-        return e;
+    if (a.prep != kPrepDone) {
+        const int rows = a.B * a.Hq;
+        cfg.numAttrs = a.prep == kPrepOverlaps ? 1 : 0;
+        cfg.gridDim = dim3(min(2 * ctas, max(1, (rows + kPrepThreads / 32 - 1) / (kPrepThreads / 32))));
+        cfg.blockDim = dim3(kPrepThreads);
+        e = cudaLaunchKernelEx(&cfg, decode_prep_kernel<T, DD>, a);
+        if (e != cudaSuccess)
+            return e;
+    }
     // one CTA per SM (the records of the workspace are sized for kMaxDecodeCtas)
     cfg.numAttrs = 1;
     cfg.gridDim = dim3(ctas);

@@ -24,6 +24,11 @@ struct AppendArgs {
     int B, Hkv, n, w, maxp, num_pages;
 };
 
+// What comes before a decode on its stream: anything; this library's cache append
+// (which writes neither q nor Uk: the query-side set-up may overlap it); or the
+// step's first kernel, which did the set-up.
+enum { kPrepAfterAll = 0, kPrepOverlaps = 1, kPrepDone = 2 };
+
 struct DecodeArgs {
     const void *q;  // [B][Hq][64]
     void *out;      // [B][Hq][64]
@@ -43,10 +48,7 @@ struct DecodeArgs {
     // scale_down / scale (nullptr: q~ = q Uk^T)
     const void *qd = nullptr;
     float qd_ratio = 1.f;
-    // the kernel before the decode on the stream is this library's cache
-    // append (which writes neither q nor Uk): the decode's query-side set-up
-    // may overlap it
-    int prep_overlaps_prev;
+    int prep;  // one of kPrep...
 };
 
 struct PrefillArgs {
@@ -105,6 +107,10 @@ cudaError_t launch_down_project(dar_dtype dt, int dd, const void *x, const float
 cudaError_t launch_down_project_kv(dar_dtype dt, int dd, const void *k, const void *v, const float *Dk,
                                    const float *Dv, void *kd, void *vd, int B, int Hkv, int n, int kstride,
                                    int vstride, int v_ones_col, cudaStream_t s);
+// The append and the decode's query-side set-up in one kernel; false in *done when
+// the append is one of many tokens (only the append is launched then).
+cudaError_t launch_step_front(dar_dtype dt, int dd, const AppendArgs &a, const DecodeArgs &d, cudaStream_t s,
+                              bool *done);
 cudaError_t launch_cache_append(dar_dtype dt, int dd, const AppendArgs &a, cudaStream_t s);
 cudaError_t launch_decode(dar_dtype dt, int dd, const DecodeArgs &a, cudaStream_t s);
 cudaError_t launch_prefill_simt(int dd, const PrefillArgs &a, cudaStream_t s);
