@@ -1,6 +1,6 @@
 // dar_project.cuh -- rows of 64 values times a 64 x DD fp32 matrix on the CUDA
 // cores, each output ONE fp32 fused-multiply-add chain over t = 0..63 starting
-// from +0.0f (Eq. 1 and the backward's q~ and dO~).
+// from +0.0f (Eq. 1).
 #pragma once
 
 #include "dar_common.cuh"
