@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(kAppThreads) step_front_kernel(AppendArgs a, D
 // chains bound it: the same prompts take 146 us (2.0 G FMA, 50 us at the
 // chip's fp32 rate; 329 MB, 49 us at the copy rate).
 template <typename T, int DD, int RPT, int NR>
-__global__ void __launch_bounds__(NR *slices<DD>()) append_bulk_kernel(AppendArgs a, int tiles)
+__device__ __forceinline__ void append_tile(const AppendArgs &a, int tiles)
 {
     constexpr int R = RPT * NR, NT = NR * slices<DD>();
     constexpr int CW = cols_per_thread<DD>();
@@ -360,6 +360,13 @@ __global__ void __launch_bounds__(NR *slices<DD>()) append_bulk_kernel(AppendArg
         *reinterpret_cast<uint4 *>(ring + (size_t)((L + j) % w) * kHeadDim + c * E) =
             *reinterpret_cast<const uint4 *>(xnew + (size_t)last * kHeadDim + c * E);
     }
+}
+
+template <typename T, int DD, int RPT, int NR>
+__global__ void __launch_bounds__(NR *slices<DD>()) append_bulk_kernel(AppendArgs a, int tiles)
+{
+    append_tile<T, DD, RPT, NR>(a, tiles);
+    sm100::grid_dep_wait();  // launched beside the kernel before it: end after that one
 }
 
 // Advances the lengths (and reports refused sequences) after append_bulk_kernel.
@@ -488,22 +495,23 @@ static cudaError_t cache_append_t(int dd, const AppendArgs &a, const DecodeArgs 
 }
 
 template <typename T, int DD, int RPT, int NR>
-static cudaError_t append_bulk_launch(const AppendArgs &a, cudaStream_t s)
+static cudaError_t append_bulk_launch(const AppendArgs &a, bool beside_prev, cudaStream_t s)
 {
     const int tiles = (a.n + RPT * NR - 1) / (RPT * NR);
-    append_bulk_kernel<T, DD, RPT, NR>
-        <<<dim3((unsigned)(a.B * a.Hkv * tiles), 2), NR * slices<DD>(), 0, s>>>(a, tiles);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess)
-        return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((a.B + 127) / 128);
-    cfg.blockDim = dim3(128);
+    cfg.gridDim = dim3((unsigned)(a.B * a.Hkv * tiles), 2);
+    cfg.blockDim = dim3(NR * slices<DD>());
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
+    cfg.numAttrs = beside_prev ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, append_bulk_kernel<T, DD, RPT, NR>, a, tiles);
+    if (e != cudaSuccess)
+        return e;
+    cfg.gridDim = dim3((a.B + 127) / 128);
+    cfg.blockDim = dim3(128);
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, append_lens_kernel, a);
 }
@@ -512,23 +520,23 @@ static cudaError_t append_bulk_launch(const AppendArgs &a, cudaStream_t s)
 constexpr long long kBulkBigCtas = 152 * 6 * 2;
 
 template <typename T, int DD>
-static cudaError_t append_bulk(const AppendArgs &a, cudaStream_t s)
+static cudaError_t append_bulk(const AppendArgs &a, bool beside_prev, cudaStream_t s)
 {
     constexpr int R = rows_bulk<T>();
     const long long big = ((long long)a.n + R - 1) / R * a.B * a.Hkv * 2;
     if (big >= kBulkBigCtas)
-        return append_bulk_launch<T, DD, rows_per_thread<DD>(), R / rows_per_thread<DD>()>(a, s);
-    return append_bulk_launch<T, DD, 1, kBulkSmallRows>(a, s);
+        return append_bulk_launch<T, DD, rows_per_thread<DD>(), R / rows_per_thread<DD>()>(a, beside_prev, s);
+    return append_bulk_launch<T, DD, 1, kBulkSmallRows>(a, beside_prev, s);
 }
 
 template <typename T>
-static cudaError_t append_bulk_t(int dd, const AppendArgs &a, cudaStream_t s)
+static cudaError_t append_bulk_t(int dd, const AppendArgs &a, bool beside_prev, cudaStream_t s)
 {
     switch (dd) {
-    case 8: return append_bulk<T, 8>(a, s);
-    case 16: return append_bulk<T, 16>(a, s);
-    case 32: return append_bulk<T, 32>(a, s);
-    case 64: return append_bulk<T, 64>(a, s);
+    case 8: return append_bulk<T, 8>(a, beside_prev, s);
+    case 16: return append_bulk<T, 16>(a, beside_prev, s);
+    case 32: return append_bulk<T, 32>(a, beside_prev, s);
+    case 64: return append_bulk<T, 64>(a, beside_prev, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -550,12 +558,12 @@ static bool use_bulk(dar_dtype dt, const AppendArgs &a)
     return a.n >= kBulkMinTokens && row <= kAppStageBytes && tiles * a.B * a.Hkv <= 0x7fffffffLL;
 }
 
-cudaError_t launch_cache_append(dar_dtype dt, int dd, const AppendArgs &a, cudaStream_t s)
+cudaError_t launch_cache_append(dar_dtype dt, int dd, const AppendArgs &a, cudaStream_t s, bool beside_prev)
 {
     if (a.B == 0)
         return cudaSuccess;
     if (use_bulk(dt, a))
-        return dt == DAR_F32 ? append_bulk_t<float>(dd, a, s) : append_bulk_t<bf16>(dd, a, s);
+        return dt == DAR_F32 ? append_bulk_t<float>(dd, a, beside_prev, s) : append_bulk_t<bf16>(dd, a, beside_prev, s);
     return dt == DAR_F32 ? cache_append_t<float>(dd, a, nullptr, s) : cache_append_t<bf16>(dd, a, nullptr, s);
 }
 

@@ -111,7 +111,9 @@ cudaError_t launch_down_project_kv(dar_dtype dt, int dd, const void *k, const vo
 // the append is one of many tokens (only the append is launched then).
 cudaError_t launch_step_front(dar_dtype dt, int dd, const AppendArgs &a, const DecodeArgs &d, cudaStream_t s,
                               bool *done);
-cudaError_t launch_cache_append(dar_dtype dt, int dd, const AppendArgs &a, cudaStream_t s);
+// (beside_prev: it may run beside the kernel before it on the stream once that one
+// lets it, and ends after it)
+cudaError_t launch_cache_append(dar_dtype dt, int dd, const AppendArgs &a, cudaStream_t s, bool beside_prev = false);
 cudaError_t launch_decode(dar_dtype dt, int dd, const DecodeArgs &a, cudaStream_t s);
 cudaError_t launch_prefill_simt(int dd, const PrefillArgs &a, cudaStream_t s);
 cudaError_t launch_prefill_tc(int dd, const PrefillArgs &a, cudaStream_t s);

@@ -260,8 +260,10 @@ __global__ void __launch_bounds__(kThreads, 2)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int w = a.w;
     const bool direct = a.qd != nullptr;  // Sec. 5 direct variant: q~ given, not absorbed
-    if constexpr (CH)
-        grid_dep_wait();  // the gather kernel, which writes pos0 and the buffers
+    if constexpr (CH) {
+        grid_dep_wait();    // the gather kernel, which writes pos0 and the buffers
+        grid_dep_launch();  // the append may start: it writes nothing that is read here (see launch_chunk_dp)
+    }
     const int bx = blockIdx.x / a.Hq, b = CH && a.B <= 32 ? nth_longest(a.pos0, a.B, bx, lane) : bx;
     const int h = blockIdx.x % a.Hq, g = h / (a.Hq / a.Hkv);
     const int L0 = CH ? a.pos0[b] : 0;           // position of query row 0
@@ -1061,8 +1063,11 @@ static cudaError_t launch_chunk_dp(const ChunkArgs &c, cudaStream_t s)
     e = launch_kernel<DP, true>(m, a, a.n, s);
     if (e != cudaSuccess)
         return e;
-    // the chunk joins the cache last: its ring slots and migrated pages
-    return launch_cache_append(DAR_BF16, DP, c.app, s);
+    // The chunk joins the cache last: its ring slots and migrated pages.  Every
+    // attention CTA has seen the gather finish, so the ring may be overwritten, and
+    // the pages it still reads lie below those that the append writes; the append
+    // runs beside the attention's last CTAs and ends after them.
+    return launch_cache_append(DAR_BF16, DP, c.app, s, true);
 }
 
 }  // namespace tcp
