@@ -39,8 +39,8 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "decode GB/s & prefill TFLOP/s of DAR attention, % of GB300 roofline (1 GPU)"
-# kernels of one timed step: the cache append, then the decode's prep and stream kernels
-LAUNCHES_PER_STEP = 3
+# kernels of one timed step: the cache append with the decode's set-up, then the decode's stream kernel
+LAUNCHES_PER_STEP = 2
 # DRAM bytes (read + write) of one decode_kernel<bf16,16,1> launch on the
 # decode-160M workload, from an ncu capture of `python bench.py --only decode`
 # (dram__bytes_read.sum + dram__bytes_write.sum); None whenever that kernel

@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(kAppThreads) step_front_kernel(AppendArgs a, D
     if ((int)blockIdx.x < a.B)
         append_sequence<T, DD>(a);
     else
-        prep_rows<T, DD>(d, blockIdx.x - a.B, gridDim.x - a.B);
+        prep_rows<T, DD, kAppThreads>(d, blockIdx.x - a.B, gridDim.x - a.B);
 }
 
 // ------------------------------------------------------- cache append, bulk

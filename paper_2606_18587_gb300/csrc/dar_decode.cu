@@ -167,7 +167,7 @@ template <typename T, int DD>
 __global__ void __launch_bounds__(kPrepThreads) decode_prep_kernel(DecodeArgs a)
 {
     sm100::grid_dep_launch();  // the stream kernel may start its set-up now
-    prep_rows<T, DD>(a, blockIdx.x, gridDim.x);
+    prep_rows<T, DD, kPrepThreads>(a, blockIdx.x, gridDim.x);
     sm100::grid_dep_wait();
 }
 
@@ -778,13 +778,18 @@ __global__ void __launch_bounds__(kDecThreads, 1)
     // kept if the counts hold.
 #pragma unroll 1
     for (int pass = 0;; ++pass) {
+        // With fewer stages than warps each is a range of its own and the other warps
+        // stay idle: cut into as many ranges as warps, a group's few parts would lie
+        // among dozens of empty ranges, which its merge had to step over (one sequence
+        // of 101 tokens, 8 heads: 19.7 us, now 9.1).  Very few are spread over the SMs
+        // (32 stages 9.0 us, side by side 9.5), more stay side by side (8 sequences of
+        // 700 to 2000 tokens 11.5, spread 12.4).  The number of ranges goes through warp
+        // votes, so that it is uniform to the compiler (64 sequences, 32 heads 118.8 us
+        // without, 118.2 with).
         const int stages = s_pre[a.B] * per_chunk, warps = gridDim.x * kDecWarps;
-        // With fewer stages than warps each is a range of its own, spread over
-        // the SMs, and the other warps stay idle: cut into as many ranges as
-        // warps, a group's few parts would lie among dozens of empty ranges, which
-        // its merge had to step over (one sequence of 101 tokens, 8 heads: 19.7 us, now 9.3).
-        sp = make_split(stages, max(1, min(stages, warps)));
-        rid = stages < warps ? warp * gridDim.x + blockIdx.x : blockIdx.x * kDecWarps + warp;
+        const bool few = __any_sync(0xffffffffu, stages < warps);
+        sp = make_split(stages, few ? max(1, (int)__reduce_max_sync(0xffffffffu, (unsigned)stages)) : warps);
+        rid = few && 2 * stages <= (int)gridDim.x ? warp * gridDim.x + blockIdx.x : blockIdx.x * kDecWarps + warp;
         lo = sp.lo(rid);
         hi = sp.lo(rid + 1);
         iss_s = lo;

@@ -11,12 +11,13 @@ namespace dar {
 // over t mod 4), and zeroed group counters.  In the direct variant of Sec. 5
 // (a.qd set) q~ is the row's own d_down query times scale_down / scale, so the
 // stream kernel's global scores scale * q~ . k^D are scale_down * q^D . k^D.
-// Reads q and Uk only.  `block` of `blocks` blocks.
-template <typename T, int DD>
+// Reads q and Uk only.  `block` of `blocks` blocks of THREADS threads.
+template <typename T, int DD, int THREADS>
 __device__ __forceinline__ void prep_rows(const DecodeArgs &a, int block, int blocks)
 {
     constexpr int QR = DD > 32 ? 2 : 1;  // q~ entries per lane
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    constexpr int warps = THREADS / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rows = a.B * a.Hq;
     for (int row = block * warps + warp; row < rows; row += blocks * warps) {
         if (a.qd) {  // direct variant: the row's own d_down query, rescaled to the local scale
@@ -51,7 +52,7 @@ __device__ __forceinline__ void prep_rows(const DecodeArgs &a, int block, int bl
         }
     }
     const int ngroups = a.B * a.Hkv * a.HS;  // group counters, then the pool's claim counter
-    for (int i = block * (int)blockDim.x + (int)threadIdx.x; i <= ngroups; i += blocks * (int)blockDim.x)
+    for (int i = block * THREADS + (int)threadIdx.x; i <= ngroups; i += blocks * THREADS)
         a.counters[i] = 0;
 }
 
