@@ -8,7 +8,6 @@
 #include "dar_launch.h"
 #include "dar_prep.cuh"
 #include "dar_project.cuh"
-#include "dar_project_tc.cuh"
 #include "dar_sm100.cuh"
 
 namespace dar {
@@ -25,8 +24,8 @@ struct BulkArgs {
     const float *W[2];
     void *out[2];
     int Hkv, n;
-    int ostride[2];   // output row stride of each tensor
-    int ones_col[2];  // tensor-core kernel: first of 16 padding columns set to 1 (-1: all padding is 0)
+    int ostride[2];   // output row stride of each tensor (columns dd.. are padding)
+    int ones_col[2];  // first of 16 padding columns set to 1 (-1: all padding is 0)
 };
 
 template <typename T, int DD, int RPT, int NR>
@@ -53,6 +52,7 @@ __global__ void __launch_bounds__(NR *slices<DD>()) down_project_kernel(BulkArgs
     float acc[RPT][CW];
     project_rows<T, DD, CW, RPT>(rows, Ws + c0, r0, NR, acc);
     const int ostride = z ? a.ostride[1] : a.ostride[0];
+    const int ones_col = z ? a.ones_col[1] : a.ones_col[0];
 #pragma unroll
     for (int k = 0; k < RPT; ++k) {
         const int r = r0 + k * NR;
@@ -60,37 +60,15 @@ __global__ void __launch_bounds__(NR *slices<DD>()) down_project_kernel(BulkArgs
             continue;
         T *o = static_cast<T *>(z ? a.out[1] : a.out[0]) + ((size_t)bg * a.n + j0 + r) * ostride;
         store_row<T, CW>(o + c0, acc[k]);
-    }
-}
-
-// The same products for a call's own workspace (not the cache, whose vectors are
-// Eq. 1's chain bit for bit), bf16 on the tensor cores.  blockIdx.z: tensor, then
-// block of COLS columns; a CTA takes `rows` token rows.
-template <int DD>
-__global__ void __launch_bounds__(32 * kTcWarps) down_project_tc_kernel(BulkArgs a, int rows)
-{
-    constexpr int COLS = DD < 32 ? DD : 32, NT = COLS / 8;
-    const bool z = blockIdx.z >= DD / COLS;
-    const int c0 = blockIdx.z % (DD / COLS) * COLS, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int bg = blockIdx.y, g = bg % a.Hkv;
-    const int ostride = z ? a.ostride[1] : a.ostride[0];
-    const bf16 *x = static_cast<const bf16 *>(z ? a.x[1] : a.x[0]) + (size_t)bg * a.n * kHeadDim;
-    bf16 *out = static_cast<bf16 *>(z ? a.out[1] : a.out[0]) + (size_t)bg * a.n * ostride + c0;
-    const float *W = (z ? a.W[1] : a.W[0]) + (size_t)g * kHeadDim * DD + c0;
-    const auto w = [&](int t, int c) { return __ldg(W + t * DD + c); };
-    const int share = rows / kTcWarps, r0 = blockIdx.x * rows + warp * share, r1 = min(a.n, r0 + share);
-    if (r0 >= r1)
-        return;
-    ProjectTc<NT> p;
-    p.load(lane, w);
-    project_rows_tc<NT>(x, out, ostride, r0, r1, p, lane, w, [](const uint4(&)[2][2], int) {});
-    const int pad = (ostride - DD) / 8;  // padding after the values: zeros, or a block of 16 ones
-    if (pad > 0 && c0 == 0) {
-        const int ones_col = z ? a.ones_col[1] : a.ones_col[0];
-        for (int i = lane; i < (r1 - r0) * pad; i += 32) {
-            const int c = DD + i % pad * 8;
-            const uint32_t v = ones_col >= 0 && c >= ones_col && c < ones_col + 16 ? 0x3f803f80u : 0u;
-            *reinterpret_cast<uint4 *>(out + (size_t)(r0 + i / pad) * ostride + c) = make_uint4(v, v, v, v);
+        if (ostride > DD && c0 == 0) {  // padding after the values: zeros, or a block of 16 ones
+            constexpr int OE = 16 / sizeof(T);
+            for (int c = DD; c < ostride; c += OE) {
+                float v[OE];
+#pragma unroll
+                for (int e = 0; e < OE; ++e)
+                    v[e] = ones_col >= 0 && c + e >= ones_col && c + e < ones_col + 16 ? 1.f : 0.f;
+                store_row<T, OE>(o + c, v);
+            }
         }
     }
 }
@@ -431,30 +409,12 @@ cudaError_t launch_down_project(dar_dtype dt, int dd, const void *x, const float
     return down_project_any(dt, dd, a, B, 1, s);
 }
 
-template <int DD>
-static cudaError_t down_project_tc(const BulkArgs &a, int B, cudaStream_t s)
-{
-    const int blocks = 2 * (DD < 32 ? 1 : DD / 32), rows = project_tc_rows(a.n, (long long)B * a.Hkv * blocks);
-    down_project_tc_kernel<DD><<<dim3((a.n + rows - 1) / rows, B * a.Hkv, blocks), 32 * kTcWarps, 0, s>>>(a, rows);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_down_project_kv(dar_dtype dt, int dd, const void *k, const void *v, const float *Dk,
                                    const float *Dv, void *kd, void *vd, int B, int Hkv, int n, int kstride,
                                    int vstride, int v_ones_col, cudaStream_t s)
 {
     BulkArgs a = {{k, v}, {Dk, Dv}, {kd, vd}, Hkv, n, {kstride, vstride}, {-1, v_ones_col}};
-    if (dt == DAR_F32)
-        return down_project_any(dt, dd, a, B, 2, s);
-    if (n == 0 || B == 0)
-        return cudaSuccess;
-    switch (dd) {
-    case 8: return down_project_tc<8>(a, B, s);
-    case 16: return down_project_tc<16>(a, B, s);
-    case 32: return down_project_tc<32>(a, B, s);
-    case 64: return down_project_tc<64>(a, B, s);
-    default: return cudaErrorInvalidValue;
-    }
+    return down_project_any(dt, dd, a, B, 2, s);
 }
 
 // d: the decode whose query-side set-up joins the launch, or nullptr.

@@ -1,7 +1,6 @@
 // dar_project_tc.cuh -- rows of 64 bf16 values times a 64 x C fp32 matrix on the
 // tensor cores (mma.sync m16n8k16), for results that need fp32 accuracy but not
-// the one chain of Eq. 1's cached vectors: the prefill's own k^D and v^D, and the
-// backward's q~, dO~, k^D and v^D.
+// the one chain of Eq. 1's vectors: the backward's q~ and dO~.
 //
 // The matrix enters as the sum of three bf16 terms: its top 8 significant bits,
 // the next 8 and the last 8, so the split is exact and a product x w is off by no

@@ -1,7 +1,7 @@
-"""The forward's own k^D and v^D on the tensor cores: token counts around its
-16-row steps and the rows of a warp, every width and padding (w = 0: every pair is
-global, so the output is all bottleneck), against the oracle (2e-2, bf16 storage);
-and an infinity in one token's key, which must reach no earlier row."""
+"""The forward's own k^D and v^D: token counts around 16 rows and around a projection
+tile, every width and padding (w = 0: every pair is global, so the output is all
+bottleneck), against the oracle (2e-2, bf16 storage); and an infinity in one token's
+key, which must reach no earlier row."""
 import numpy as np
 import pytest
 
@@ -30,9 +30,8 @@ def test_all_global_rows(B, H, N, dd):
 
 @pytest.mark.parametrize("dd", [8, 16, 32, 64])
 def test_an_infinity_stays_in_its_row(dd):
-    """Token 270's key holds an infinity: rows before it mask that score, and use k^D of the tokens that share
-    its 16-row step (256 to 269), which take chains then and may differ by one rounding to bf16 (2^-8 of a
-    score below 8, far below 2e-2 in the output)."""
+    """Token 270's key holds an infinity: rows before it mask that score.  (The vectors of the tokens beside it,
+    256 to 269, are Eq. 1's chains with or without it; the last bound would allow one rounding of them to bf16.)"""
     from paper_2606_18587_gb300 import dar
     g = torch.Generator(device="cuda").manual_seed(dd)
     q, k, v = (torch.randn(1, 2, 300, 64, device="cuda", generator=g).bfloat16() for _ in range(3))
