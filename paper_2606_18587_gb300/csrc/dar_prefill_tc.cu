@@ -583,7 +583,6 @@ __global__ void __launch_bounds__(kThreads, 2)
 
         const float c2 = a.qscale;  // softmax scale * log2(e)
         float mA = -INFINITY, mB = -INFINITY;  // running maxima (log2 units) of rows ra, ra + 8
-        bool fresh = true;  // some row of the warp has no running maximum yet
         // last tile whose PV this thread has seen complete, per S buffer
         int pv_seen0 = -1, pv_seen1 = -1;
         // wait until PV(v) (its own products) has completed
@@ -683,64 +682,48 @@ __global__ void __launch_bounds__(kThreads, 2)
                     }
                 }
             }
-            // exponents y = s * c2 - m relative to the running maxima (masked
-            // entries: -infinity), in place
-            float nA = mA == -INFINITY ? 0.f : -mA, nB = mB == -INFINITY ? 0.f : -mB;
+            // One vote per tile decides whether any row's maximum grows by more than
+            // the threshold (or is not set yet).  This thread's 16 columns of a row
+            // are enough for that: scaling and rounding keep the order, so some
+            // thread's maximum passes the test exactly if the row's does.  The row
+            // maxima, their shuffles and the scale factors are left to the rare case.
+            auto col_max = [&](const float (&x)[16]) {
+                float r = max3(x[0], x[1], x[2]);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                ffma2(sa[2 * k], sa[2 * k + 1], sa[2 * k], sa[2 * k + 1], c2, c2, nA, nA);
-                ffma2(sv[2 * k], sv[2 * k + 1], sv[2 * k], sv[2 * k + 1], c2, c2, nB, nB);
-            }
-            // One vote per tile decides whether any row's maximum grows by more
-            // than the threshold (or is not set yet): the maximum of both rows'
-            // columns of this thread is enough for that, and the row maxima,
-            // their shuffles and the scale factors are left to the rare case.
-            float top = max3(sa[0], sa[1], sa[2]);
-#pragma unroll
-            for (int e = 3; e < 15; e += 2)
-                top = max3(top, sa[e], sa[e + 1]);
-            top = max3(top, sa[15], sv[0]);
-#pragma unroll
-            for (int e = 1; e < 15; e += 2)
-                top = max3(top, sv[e], sv[e + 1]);
-            top = fmaxf(top, sv[15]);
+                for (int e = 3; e < 15; e += 2)
+                    r = max3(r, x[e], x[e + 1]);
+                return fmaxf(r, x[15]) * c2;
+            };
+            float xA = col_max(sa), xB = col_max(sv);
             bool scaleA = false, scaleB = false;
             float alA = 1.f, alB = 1.f;  // O's scale factors when a running max is raised
-            if (__builtin_expect(__any_sync(0xffffffffu, top > kRescaleThreshold) || fresh, 0)) {
-                auto row_max = [&](const float (&x)[16]) {
-                    float r = x[0];
-#pragma unroll
-                    for (int e = 1; e < 15; e += 2)
-                        r = max3(r, x[e], x[e + 1]);
-                    r = fmaxf(r, x[15]);
-                    r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, 1));
-                    return fmaxf(r, __shfl_xor_sync(0xffffffffu, r, 2));
-                };
-                auto raise = [&](float (&x)[16], float &m, float &n, float &al) {
-                    const float r = row_max(x);  // relative to the old maximum (to 0 while there is none)
-                    const bool none = m == -INFINITY;
-                    if (!(none ? r > -INFINITY : r > kRescaleThreshold))
+            if (__builtin_expect(__any_sync(0xffffffffu, xA > mA + kRescaleThreshold || xB > mB + kRescaleThreshold),
+                                 0)) {
+                auto raise = [&](float x, float &m, float &al) {  // x: the row's maximum so far in this thread
+                    x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 1));
+                    x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 2));
+                    if (!(x > m + kRescaleThreshold))
                         return false;
-                    al = none ? 1.f : ex2_approx(-r);
-                    m = none ? r : m + r;
-                    const float d = -m - n;  // (-r but for m's rounding)
-                    n = -m;
-#pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        x[e] += d;
-                    return !none;
+                    const bool first = m == -INFINITY;
+                    al = first ? 1.f : ex2_approx(m - x);
+                    m = x;
+                    return !first;
                 };
-                scaleA = raise(sa, mA, nA, alA);
-                scaleB = raise(sv, mB, nB, alB);
-                fresh = __any_sync(0xffffffffu, (iA < N && mA == -INFINITY) || (iB < N && mB == -INFINITY));
+                scaleA = raise(xA, mA, alA);
+                scaleB = raise(xB, mB, alB);
             }
-            // P = 2^y in bf16 pairs: pw[2k] row ra, pw[2k + 1] row ra + 8, P column
-            // 4k + q4 (keys 8k + 2 q4, + 1)
+            // P = 2^(s * c2 - m) in bf16 pairs (masked entries give 0): pw[2k] row
+            // ra, pw[2k + 1] row ra + 8, P column 4k + q4 (keys 8k + 2 q4, + 1).  The
+            // exponent is rounded once, from the score, also where m has just risen.
+            const float nA = mA == -INFINITY ? 0.f : -mA, nB = mB == -INFINITY ? 0.f : -mB;
             uint32_t pw[16];
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                pw[2 * k] = ex2_bf16x2(cvt_bf16x2(sa[2 * k], sa[2 * k + 1]));
-                pw[2 * k + 1] = ex2_bf16x2(cvt_bf16x2(sv[2 * k], sv[2 * k + 1]));
+                float x0, x1, y0, y1;
+                ffma2(x0, x1, sa[2 * k], sa[2 * k + 1], c2, c2, nA, nA);
+                ffma2(y0, y1, sv[2 * k], sv[2 * k + 1], c2, c2, nB, nB);
+                pw[2 * k] = ex2_bf16x2(cvt_bf16x2(x0, x1));
+                pw[2 * k + 1] = ex2_bf16x2(cvt_bf16x2(y0, y1));
             }
             if (__builtin_expect(__any_sync(0xffffffffu, scaleA || scaleB), 0)) {
                 // every earlier PV must have landed before O is rescaled (PV(t),
