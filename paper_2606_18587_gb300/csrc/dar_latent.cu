@@ -587,7 +587,7 @@ struct Rows {
         }
     }
 
-    // Records (O, m, l) of rows 0 .. n - 1: rec(row) points at W + 2 floats.
+    // Records (O, m, l) of rows 0 .. n - 1, after a stage: rec(row) points at W + 2 floats.
     template <typename F>
     __device__ __forceinline__ void finish(float *red, int n, int warp, int lane, F &&rec)
     {
@@ -597,7 +597,7 @@ struct Rows {
             l[hr] += __shfl_xor_sync(0xffffffffu, l[hr], 1);
             l[hr] += __shfl_xor_sync(0xffffffffu, l[hr], 2);
         }
-        consumer_sync();  // `red` is free
+        // (`red` is free: its maxima were read before the last stage's second barrier)
         if (tig == 0) {
             red[warp * 16 + grp] = l[0];
             red[warp * 16 + grp + 8] = l[1];
@@ -624,6 +624,7 @@ struct Rows {
                     r[W + 1] = ls;
                 }
             }
+        consumer_sync();  // the sums are read: the next segment may write its maxima
     }
 };
 
