@@ -435,6 +435,8 @@ struct Segment {
     int npg;      // pages / tiles
 };
 
+constexpr float kMaxDrop = 64.f;  // log2 units
+
 __device__ __forceinline__ void consumer_sync()
 {
     asm volatile("bar.sync 1, %0;" ::"n"(kConsumerThreads) : "memory");
@@ -447,7 +449,8 @@ template <int W, int MT>
 struct Rows {
     uint32_t a[W / 16][4];
     float o[MT][W / 32][4];
-    float m[MT][2];  // running maxima (log2 units) of rows grp, grp + 8 of each m-tile
+    float m[MT][2];  // reference of the weights (log2 units) of rows grp, grp + 8 of each m-tile
+    float top[MT][2];  // the largest it has been
     float l[2];      // sums of this warp's weights, rows of its own m-tile
 
     // x: `n` rows of stride W (rows past n: zero)
@@ -467,7 +470,7 @@ struct Rows {
 #pragma unroll
             for (int nt = 0; nt < W / 32; ++nt)
                 o[mt][nt][0] = o[mt][nt][1] = o[mt][nt][2] = o[mt][nt][3] = 0.f;
-            m[mt][0] = m[mt][1] = -INFINITY;
+            m[mt][0] = m[mt][1] = top[mt][0] = top[mt][1] = -INFINITY;
         }
         l[0] = l[1] = 0.f;
     }
@@ -475,10 +478,16 @@ struct Rows {
     // One stage: S = A B^T (B: the key-side tile), masks past ntok, one
     // online-softmax step per row (maxima exchanged through `red`), P into shared
     // memory, O += P V (V: the value-side tile).  refill() runs once every warp is
-    // done with the stage before.
+    // done with the stage before.  fresh: the weights' reference starts anew at this
+    // tile's maximum, which may be the lower one (by kMaxDrop at most, so that the
+    // sums stay finite).  A weight is rounded to bf16 relative to its reference, and
+    // the token that sets it has a weight of exactly 1: a reference per unit keeps
+    // the error of separate records per unit (against 64 bits, 64 sequences of 1024
+    // to 8192 tokens, 32 heads: 0.002368 both; 0.002373 with one maximum over a
+    // segment, which is 2 us faster, 65 us; separate records take 79).
     template <typename F>
     __device__ __forceinline__ void stage(uint32_t ktile, uint32_t vtile, unsigned char *sm_p, float *red, int ntok,
-                                          float c2, int warp, int lane, F &&refill)
+                                          float c2, bool fresh, int warp, int lane, F &&refill)
     {
         constexpr int NTS = 2 * MT, NT = W / 32;
         const int grp = lane >> 2, tig = lane & 3, own = warp % MT, tok0 = 16 * MT * (warp / MT);
@@ -521,7 +530,7 @@ struct Rows {
         consumer_sync();
         refill();
         float alpha[MT][2], mo[2];
-        bool grown = false;
+        bool moved = false;
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
@@ -530,8 +539,9 @@ struct Rows {
 #pragma unroll
                 for (int w2 = mt; w2 < 4; w2 += MT)
                     mx = fmaxf(mx, red[w2 * 16 + grp + 8 * hr]);
-                const float mnew = fmaxf(m[mt][hr], mx * c2);
-                grown |= mnew != m[mt][hr];
+                const float mnew = fmaxf(fresh ? top[mt][hr] - kMaxDrop : m[mt][hr], mx * c2);
+                top[mt][hr] = fmaxf(top[mt][hr], mnew);
+                moved |= mnew != m[mt][hr];
                 alpha[mt][hr] = m[mt][hr] == -INFINITY ? 0.f : ex2_approx(m[mt][hr] - mnew);
                 m[mt][hr] = mnew;
                 if (mt == own) {
@@ -553,7 +563,7 @@ struct Rows {
                     pk;
             }
         }
-        if (__any_sync(0xffffffffu, grown)) {
+        if (__any_sync(0xffffffffu, moved)) {
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
@@ -811,7 +821,8 @@ __global__ void __launch_bounds__(MainLayout<DL, MT>::THREADS, 2)
             const int st = gp % NST, ntok = min(kTok, tokens - p * kTok);
             stage_wait(st, ntok, width);
             const uint32_t t = sbase + Ly::STG + st * Ly::CST;
-            rows.stage(t, t + voff, sm + Ly::P, red, ntok, a.c2, warp, lane, [&] {
+            rows.stage(t, t + voff, sm + Ly::P, red, ntok, a.c2, it.latent && p % kPagesPerSplit == 0, warp, lane,
+                       [&] {
                 if (!Ly::kProducer && tid == 0 && gp > 0 && pit.npg >= 0)
                     fetch();  // into the stage of gp - 1
             });
