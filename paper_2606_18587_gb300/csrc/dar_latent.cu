@@ -880,11 +880,18 @@ __global__ void __launch_bounds__(MainLayout<DL, MT>::THREADS, 2)
 
 // A load the compiler keeps in place (a batch of them is issued before the first
 // use; with the registers for it, see the launch bounds, the merge of 31 records of
-// 32 heads took 10 us, 25 without).
-__device__ __forceinline__ float2 ld_early_f2(const float *p)
+// 32 heads took 10 us, 25 without).  Zeros, and no load, when !on.
+__device__ __forceinline__ float2 ld_early_f2(const float *p, bool on)
 {
     float2 r;
-    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "l"(p));
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %3, 0;\n\t"
+        "mov.b32 %0, 0;\n\t"
+        "mov.b32 %1, 0;\n\t"
+        "@p ld.global.v2.f32 {%0, %1}, [%2];\n\t}"
+        : "=&f"(r.x), "=&f"(r.y)
+        : "l"(p), "r"((uint32_t)on));
     return r;
 }
 
@@ -937,14 +944,15 @@ __global__ void __launch_bounds__(kRowThreads, 2) latent_merge_kernel(Args a)
             // slots with a weight (empty ones hold no O), in batches of 8
             for (unsigned left = __ballot_sync(0xffffffffu, f != 0.f); left;) {
                 const float *src[8];
+                bool on[8];
                 float fj[8];
                 float2 x[8][DL / 64];
-                const int at0 = __ffs(left) - 1;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {  // past the last slot: the first one again, with weight 0
-                    const int at = left ? __ffs(left) - 1 : at0;
+                for (int j = 0; j < 8; ++j) {  // past the last slot: 0 times 0 (a record may hold an infinity)
+                    on[j] = left != 0u;
+                    const int at = on[j] ? __ffs(left) - 1 : 0;
                     const float fa = __shfl_sync(0xffffffffu, f, at);
-                    fj[j] = left ? fa : 0.f;
+                    fj[j] = on[j] ? fa : 0.f;
                     src[j] = rl0 + (s0 + at) * (DL + 2) + 2 * lane;
                     left &= left - 1;
                 }
@@ -952,7 +960,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) latent_merge_kernel(Args a)
                 for (int j = 0; j < 8; ++j)
 #pragma unroll
                     for (int e = 0; e < DL / 64; ++e)
-                        x[j][e] = ld_early_f2(src[j] + 64 * e);
+                        x[j][e] = ld_early_f2(src[j] + 64 * e, on[j]);
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
 #pragma unroll

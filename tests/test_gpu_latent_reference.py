@@ -63,3 +63,23 @@ def test_weights_of_one_are_exact(dl):
 def test_scores_that_fall_or_rise_far(step):
     got, want = _decode(304, np.tile(step * np.arange(6.0), (304, 1)), 64)
     assert (got.double() - want).abs().max().item() <= 2e-2
+
+
+@pytest.mark.parametrize("units", [1, 3, 8, 9])
+def test_an_infinite_record_stays_infinite(units):
+    """Two tokens whose values overflow fp32 together, in a record among others: every output is the infinity that
+    its weight in A_V gives it the sign of, and the sequence without them is finite."""
+    dl, w = 64, 16
+    cache = dar.DarLatentCache(2, 1, 64, dl, w, 4 * units + 1)
+    cache.pool_c.zero_()
+    cache.pool_c[0, 3, 5] = cache.pool_c[0, 4, 5] = 3.0e38
+    cache.seq_lens.fill_(units * UNIT + w)
+    q = torch.zeros(2, 1, 64, device="cuda", dtype=torch.bfloat16)
+    A_K = torch.zeros(1, 64, dl, device="cuda")
+    sign = torch.where(torch.arange(64, device="cuda") % 3 == 0, -1.0, 1.0)
+    A_V = sign.expand(1, dl, 64).contiguous()
+    out = dar.dar_latent_decode(cache, q, A_K, A_V, dar.latent_decode_workspace(cache, 1))
+    torch.cuda.synchronize()
+    assert cache.device_status() == 0
+    assert torch.equal(out[0, 0].float(), sign * float("inf"))
+    assert torch.equal(out[1, 0].float(), torch.zeros(64, device="cuda"))
