@@ -825,6 +825,25 @@ struct WpartTc {
     static_assert(RW * 64 * DD * 4 <= (int)TOTAL, "the warps' sums fit in the stage area");
 };
 
+// The same sums as fp32 chains on the CUDA cores, for a chunk whose tensor-core sums
+// are not all finite: an infinity times the split's rests (of either sign, or 0) is
+// NaN there also where the product itself is an infinity.  Row r of the sum is token
+// r % N of one of `heads` heads from head0 (of all_heads) of sequence r / (N heads).
+template <int DD>
+__device__ __noinline__ void wpart_chains(const bf16 *X, const float *Y, const float *fac, long r0, long r1, int N,
+                                          int heads, int head0, int all_heads, float *dst)
+{
+    for (int o = threadIdx.x; o < 64 * DD; o += 256) {
+        float s = 0.f;
+        for (long r = r0; r < r1; ++r) {
+            const long u = r / N, at = (u / heads * all_heads + head0 + u % heads) * N + r % N;
+            const float y = Y[at * DD + o % DD];
+            s = fmaf(__bfloat162float(X[at * 64 + o / DD]), fac ? y * fac[at] : y, s);
+        }
+        dst[o] = s;
+    }
+}
+
 template <int DD>
 __global__ void __launch_bounds__(256) bwd_wpart_tc_kernel(Args a)
 {
@@ -926,10 +945,9 @@ __global__ void __launch_bounds__(256) bwd_wpart_tc_kernel(Args a)
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         b[k][e] = cvt_bf16x2(y0, y1);
-                        // (an infinity has no rest: it stays one, and is not turned into inf - inf)
-                        const float h0 = bf16lo(b[k][e]), h1 = bf16hi(b[k][e]);
-                        y0 = k == 0 && fabsf(h0) == INFINITY ? 0.f : y0 - h0;
-                        y1 = k == 0 && fabsf(h1) == INFINITY ? 0.f : y1 - h1;
+                        // (an infinity gives NaN here; see wpart_chains)
+                        y0 -= bf16lo(b[k][e]);
+                        y1 -= bf16hi(b[k][e]);
                     }
                 }
 #pragma unroll
@@ -952,13 +970,17 @@ __global__ void __launch_bounds__(256) bwd_wpart_tc_kernel(Args a)
                     make_float2(acc[mt][n][2 * hr], acc[mt][n][2 * hr + 1]);
     __syncthreads();
     float *dst = a.part + (((size_t)chunk * 4 + which) * a.Hkv + g) * 64 * DD;
+    bool bad = false;
     for (int o = tid; o < 64 * DD; o += 256) {
         float s = red[o];
 #pragma unroll
         for (int k = 1; k < RW; ++k)
             s += red[k * 64 * DD + o];
+        bad |= !(fabsf(s) < INFINITY);
         dst[o] = s;
     }
+    if (__syncthreads_or(bad))
+        wpart_chains<DD>(X, Yp, per_kv ? nullptr : a.fac, r0, r1, a.N, heads, g * heads, per_kv ? a.Hkv : a.Hq, dst);
 }
 
 // ---------------------------------------------------------------- host side
