@@ -779,10 +779,10 @@ __global__ void __launch_bounds__(32 * kTcWarps) bwd_rows_tc_kernel(Args a, int 
     auto each = [&](const uint4(&v)[2][2], int r) {
         if (!z || c0 > 0)
             return;
-        float s[2] = {0.f, 0.f};
 #pragma unroll
         for (int hr = 0; hr < 2; ++hr) {
             const int row = r + (lane >> 2) + 8 * hr;
+            float s[2] = {0.f, 0.f};  // a chain per 16-byte chunk, the eight added pairwise
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 float d[8], y[8];
@@ -792,12 +792,12 @@ __global__ void __launch_bounds__(32 * kTcWarps) bwd_rows_tc_kernel(Args a, int 
                        y, bf16());
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
-                    s[hr] = fmaf(d[k], y[k], s[hr]);
+                    s[i] = fmaf(d[k], y[k], s[i]);
+                s[i] += __shfl_xor_sync(0xffffffffu, s[i], 1);
+                s[i] += __shfl_xor_sync(0xffffffffu, s[i], 2);
             }
-            s[hr] += __shfl_xor_sync(0xffffffffu, s[hr], 1);
-            s[hr] += __shfl_xor_sync(0xffffffffu, s[hr], 2);
             if (tig == 0 && row < r1)
-                a.drow[row0 + row] = -s[hr];
+                a.drow[row0 + row] = -(s[0] + s[1]);
         }
     };
     project_rows_tc<NT>(x, (z ? a.dotb : a.qtb) + row0 * DD + c0, DD, r0, r1, p, lane, w, each);
