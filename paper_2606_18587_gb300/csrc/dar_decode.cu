@@ -786,6 +786,7 @@ __global__ void __launch_bounds__(kDecThreads, 1)
         // 700 to 2000 tokens 11.5, spread 12.4).  The number of ranges goes through warp
         // votes, so that it is uniform to the compiler (64 sequences, 32 heads 118.8 us
         // without, 118.2 with).
+        static_assert(kDecodePoolPercent == 0, "range numbers past the last one must name no pool chunk");
         const int stages = s_pre[a.B] * per_chunk, warps = gridDim.x * kDecWarps;
         const bool few = __any_sync(0xffffffffu, stages < warps);
         sp = make_split(stages, few ? max(1, (int)__reduce_max_sync(0xffffffffu, (unsigned)stages)) : warps);

@@ -9,7 +9,10 @@ segments of a part write records into the range's slots (slot 0 if the
 group began before the range, else slot 1), each part adds its stage count
 to the group's counter, and the part that completes the count merges the
 group by enumerating, for every range the group meets, the records that
-range must have written.
+range must have written.  With fewer stages than warps (and no pool) each
+stage is a range of its own: NW is the number of stages, and the warps of
+the grid take range numbers side by side, or across the CTAs when there are
+at most half as many stages as CTAs; the others find an empty range.
 
 This module restates that arithmetic in plain Python and checks the
 invariants the kernel relies on, over random batches, lengths, grids and
@@ -22,6 +25,8 @@ pool shares:
   * the records a merge enumerates are exactly the records written;
   * no record slot is written twice for two groups while the first is
     still unmerged;
+  * the warps of a grid own every range once, and warps past the last range
+    own nothing;
 and checks the kernel's division by the warp count (a float reciprocal with
 a one-step correction) exhaustively against integer division.
 """
@@ -160,6 +165,47 @@ def test_split_bookkeeping(seed):
         simulate(Ls, rng.randint(1, 4), rng.choice([8, 37, 64, 152 * 8]), rng.choice([1, 16, 128, 200]),
                  rng.choice([16, 32]), rng.choice([16, 32, 64, 128, 256]), rng.choice([0, 0, 15, 50, 100]),
                  rng.choice([7, 100, 2 * 160 * 8]), rng)
+
+
+def warp_ranges(stages, ctas, warps_per_cta=8):
+    """What each warp of the grid owns: (number of ranges, [(range number, lo, hi)])."""
+    warps = ctas * warps_per_cta
+    few = stages < warps
+    NW = max(1, stages) if few else warps
+    sp = Split(stages, NW, 0, 2 * 160 * 8)
+    own = []
+    for cta in range(ctas):
+        for warp in range(warps_per_cta):
+            rid = warp * ctas + cta if few and 2 * stages <= ctas else cta * warps_per_cta + warp
+            own.append((rid, sp.lo(rid), sp.lo(rid + 1)))
+    return NW, own
+
+
+@pytest.mark.parametrize("ctas", [1, 148, 152, 160])
+def test_warps_own_every_stage_once(ctas):
+    warps = 8 * ctas
+    for stages in sorted({0, 1, 2, 7, 8, 9, ctas // 2, ctas // 2 + 1, ctas, warps // 2, warps - 1, warps, warps + 1,
+                          3 * warps + 5}):
+        NW, own = warp_ranges(stages, ctas)
+        assert len({rid for rid, _, _ in own}) == warps  # no number twice
+        busy = sorted((lo, hi) for _, lo, hi in own if lo < hi)
+        assert [t for lo, hi in busy for t in range(lo, hi)] == list(range(stages))
+        assert all(rid < NW for rid, lo, hi in own if lo < hi)
+        if stages < warps:
+            assert all(hi - lo == 1 for lo, hi in busy)
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_split_bookkeeping_with_a_range_per_stage(seed):
+    """Fewer stages than warps: the same invariants with as many ranges as stages."""
+    rng = random.Random(100 + seed)
+    for _ in range(100):
+        Ls = [rng.choice([0, 1, 31, 33, 128, 129, rng.randint(0, 900)]) for _ in range(rng.randint(1, 6))]
+        w, tps_w, tps_d, per_group = rng.choice([1, 16, 128, 200]), rng.choice([16, 32]), rng.choice([16, 64, 256]), \
+            rng.randint(1, 4)
+        stages = per_group * sum(stages_of(L, w, tps_w, tps_d)[1] for L in Ls)
+        if 0 < stages < 152 * 8:
+            simulate(Ls, per_group, stages, w, tps_w, tps_d, 0, 2 * 160 * 8, rng)
 
 
 def test_decode160m_split():
