@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(kAppThreads) step_front_kernel(AppendArgs a, D
 // with the last new token that lands there.  A ring slot therefore has one
 // reader and one writer, in one CTA, and no order between CTAs is needed.  The
 // length is advanced by a second kernel once every CTA has read it.  The FMA
-// chains bound it: the same prompts take 146 us (2.0 G FMA, 50 us at the
+// chains bound it: the same prompts take 122 us a call (2.0 G FMA, 50 us at the
 // chip's fp32 rate; 329 MB, 49 us at the copy rate).
 template <typename T, int DD, int RPT, int NR>
 __device__ __forceinline__ void append_tile(const AppendArgs &a, int tiles)

@@ -19,8 +19,8 @@
 //   dUv = sum_i O^D_i^T dO_i (O^D_i = sum_global p_ij v^D_j).
 //
 // Kernels (fp32 arithmetic on the CUDA cores; used for fp32 storage and for
-// bf16 with d_down = 8 -- other bf16 shapes run steps 2 and 3 on the tensor
-// cores, dar_backward_tc.cu, and share steps 1 and 4):
+// bf16 with d_down = 8 -- other bf16 shapes have tensor-core kernels for all
+// four steps, dar_backward_tc.cu, and share only the last sum, bwd_wsum):
 //  1. bwd_rows: per row, q~, dO~ and D (one warp per row, Uk and Uv staged
 //     in shared memory per KV head).
 //  2. bwd_dq: per 64-row query tile, the row log-sum-exp (first pass over the
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(kThreads) bwd_wpart_kernel(Args a)
             for (int e = tid; e < n * YC; e += kThreads)
                 sm100::cp_async16(d + Sm::X + e * 16, Y + row_of(e / YC) * DD + e % YC * 4);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        sm100::cp_async_commit();
     };
     const int grp = tid / TPG, c0 = tid % TPG % YC * 4, t0 = tid % TPG / YC * 4;
     float acc[4][4];
@@ -572,7 +572,7 @@ __global__ void __launch_bounds__(kThreads) bwd_wpart_kernel(Args a)
     for (int t = 0; t < NS - 1; ++t)
         stage(t);
     for (int t = 0; t < ntiles; ++t) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(NS - 2) : "memory");
+        sm100::cp_async_wait<NS - 2>();
         __syncthreads();
         stage(t + NS - 1);
         const unsigned char *st = sm + (t % NS) * Sm::STAGE;
@@ -601,7 +601,7 @@ __global__ void __launch_bounds__(kThreads) bwd_wpart_kernel(Args a)
             }
         }
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    sm100::cp_async_wait<0>();
     __syncthreads();
     float *red = reinterpret_cast<float *>(sm);  // [NG][64 * DD]
 #pragma unroll

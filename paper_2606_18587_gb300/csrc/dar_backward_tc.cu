@@ -35,6 +35,8 @@ namespace dar {
 namespace bwd {
 
 using sm100::add2;
+using sm100::cp_async_commit;
+using sm100::cp_async_wait;
 using sm100::cvt_bf16x2;
 using sm100::ex2_approx;
 using sm100::ffma2;
@@ -53,12 +55,6 @@ __device__ __forceinline__ void cp16z(uint32_t dst, const void *src, bool valid)
 {
     const int n = valid ? 16 : 0;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 // Bytes per padded row of a W-wide bf16 tile.
@@ -239,14 +235,14 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
             stage_rows<W, BK>(dst, kp + (size_t)j * W, N - j, tid);
             stage_rows<W, BK>(dst + Sm::V, vp + (size_t)j * W, N - j, tid);
         }
-        cp_commit();
+        cp_async_commit();
     };
     // this CTA's rows into the last stage, then the first tiles
     stage_rows<W, ROWS>(sb + (NS - 1) * Sm::STAGE,
                         (LOCAL ? static_cast<const bf16 *>(a.q) : a.qtb) + (headrow + i0) * W, N - i0, tid);
     stage_rows<W, ROWS>(sb + (NS - 1) * Sm::STAGE + Sm::V,
                         (LOCAL ? static_cast<const bf16 *>(a.dout) : a.dotb) + (headrow + i0) * W, N - i0, tid);
-    cp_commit();
+    cp_async_commit();
     for (int t = 0; t < NS - 1; ++t)
         stage(t);
 
@@ -261,7 +257,7 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
             const int i = r0 + 16 * mt + grp + 8 * hr;
             drow[mt][hr] = i < N ? a.drow[headrow + i] : 0.f;
         }
-    cp_wait<NS - 1>();
+    cp_async_wait<NS - 1>();
     __syncthreads();
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt) {
@@ -427,7 +423,7 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
     };
 
     for (int t = 0; t < ntiles; ++t) {
-        cp_wait<NS - 2>();
+        cp_async_wait<NS - 2>();
         __syncthreads();  // tile t is in; every warp is done with tile t - 1
         stage(t + NS - 1);
         const uint32_t ks = sb + (t % NS) * Sm::STAGE;
@@ -491,7 +487,7 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dq_tc_kernel(A
     } else {
         static_assert(!LOCAL || MT == 1, "the lift stages 64 rows");
         // merge with the global part; dq = scale dq_loc / l + (dq~ / l) Uk
-        cp_wait<0>();
+        cp_async_wait<0>();
         __syncthreads();  // the stage area is idle
         float *lift = reinterpret_cast<float *>(tsm);  // [64][DD + 1]
         float *uk = lift + 64 * (DD + 1);              // [DD][64]; 16-byte words: 64 * (DD + 1) floats come before
@@ -580,17 +576,17 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dkv_tc_kernel(
                 }
             }
         }
-        cp_commit();
+        cp_async_commit();
     };
     // this CTA's keys and values into the last stage, then the first tiles
     stage_rows<W, ROWS>(sb + (NS - 1) * Sm::STAGE, static_cast<const bf16 *>(LOCAL ? a.k : a.kd) + (kvbase + j0) * W,
                         N - j0, tid);
     stage_rows<W, ROWS>(sb + (NS - 1) * Sm::STAGE + Sm::DO,
                         static_cast<const bf16 *>(LOCAL ? a.v : a.vd) + (kvbase + j0) * W, N - j0, tid);
-    cp_commit();
+    cp_async_commit();
     for (int t = 0; t < NS - 1; ++t)
         stage(t);
-    cp_wait<NS - 1>();
+    cp_async_wait<NS - 1>();
     __syncthreads();
 
     const int r0 = j0 + 16 * MT * warp;  // this warp's keys r0 .. r0 + 16 MT - 1
@@ -668,7 +664,7 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dkv_tc_kernel(
     };
 
     for (int t = 0; t < ntiles; ++t) {
-        cp_wait<NS - 2>();
+        cp_async_wait<NS - 2>();
         __syncthreads();
         stage(t + NS - 1);
         const uint32_t qs = sb + (t % NS) * Sm::STAGE;
@@ -721,7 +717,7 @@ __global__ void __launch_bounds__(kTc, Shape<W, LOCAL>::MINB) bwd_dkv_tc_kernel(
         const int nv = min(ROWS, N - j0);
 #pragma unroll
         for (int kv = 0; kv < 2; ++kv) {
-            cp_wait<0>();
+            cp_async_wait<0>();
             __syncthreads();  // the stage area (or the other lift) is idle
             const float *Wd = (kv ? a.Dv : a.Dk) + (size_t)g * 64 * DD;
             const float *x = (kv ? a.dvd : a.dkd) + (kvbase + j0) * DD;
@@ -897,7 +893,7 @@ __global__ void __launch_bounds__(256) bwd_wpart_tc_kernel(Args a)
             else
                 reinterpret_cast<float *>(tsm + (t & 1) * L::STAGE + L::FAC)[tid] = 0.f;
         }
-        cp_commit();
+        cp_async_commit();
         for (i += kWtRows; i >= a.N; i -= a.N)
             base = base_of(++u);
     };
@@ -911,7 +907,7 @@ __global__ void __launch_bounds__(256) bwd_wpart_tc_kernel(Args a)
     if (ntiles > 0)
         stage(0);
     for (int t = 0; t < ntiles; ++t) {
-        cp_wait<0>();
+        cp_async_wait<0>();
         __syncthreads();  // tile t is in; every warp is done with tile t - 1
         if (t + 1 < ntiles)
             stage(t + 1);
