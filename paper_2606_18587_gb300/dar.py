@@ -120,7 +120,10 @@ def _stream(stream=None):
     """The raw handle of ``stream`` (default: the current stream of the current device)."""
     if stream is not None:
         return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    try:  # without making a Stream object on every call
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except AttributeError:  # a torch that does not have these two
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t):
