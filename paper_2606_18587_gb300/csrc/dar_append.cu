@@ -370,7 +370,7 @@ __global__ void append_lens_kernel(AppendArgs a)
 // tiles (16 heads x N 1000) 22.3 / 20.8; 512 tiles (32 heads x N 2000, d_down
 // 64) 92 / 101; 1024 tiles (64 heads x N 2047) 82.6 / 85.3.
 constexpr int kBulkSmallRows = 64;
-constexpr long long kProjectBigCtas = 152 * 2;
+constexpr long long kProjectBigCtas = kSms * 2;
 
 template <typename T, int DD>
 static cudaError_t down_project_dd(const BulkArgs &a, int B, int nz, cudaStream_t s)
@@ -434,7 +434,7 @@ static cudaError_t cache_append_dd(const AppendArgs &a, const DecodeArgs *d, cud
     const size_t smem = (size_t)app_rows<T>(a.Hkv) * 2 * a.Hkv * kHeadDim * sizeof(T);
     if (d) {
         constexpr int warps = kAppThreads / 32;
-        const int prep = min(2 * 152, (d->B * d->Hq + warps - 1) / warps);
+        const int prep = min(2 * kSms, (d->B * d->Hq + warps - 1) / warps);
         step_front_kernel<T, DD><<<a.B + prep, kAppThreads, smem, s>>>(a, *d);
     } else {
         cache_append_kernel<T, DD><<<a.B, kAppThreads, smem, s>>>(a);
@@ -477,7 +477,7 @@ static cudaError_t append_bulk_launch(const AppendArgs &a, bool beside_prev, cud
 }
 
 // Here big tiles pay once they fill the chip a few times over.
-constexpr long long kBulkBigCtas = 152 * 6 * 2;
+constexpr long long kBulkBigCtas = kSms * 6 * 2;
 
 template <typename T, int DD>
 static cudaError_t append_bulk(const AppendArgs &a, bool beside_prev, cudaStream_t s)

@@ -1134,13 +1134,13 @@ static cudaError_t append_tiled_any(const AppendArgs &a, cudaStream_t s)
     const auto ctas = [&](int rows, int cols) {
         return ((long long)a.B * a.n + rows - 1) / rows * (a.DL / cols);
     };
-    if (ctas(4, 32) <= 152)
+    if (ctas(4, 32) <= kSms)
         return append_tiled<1, 1>(a, s);
-    if (ctas(8, 32) <= 152 * 3)
+    if (ctas(8, 32) <= kSms * 3)
         return append_tiled<2, 1>(a, s);
-    if (ctas(16, 32) <= 152 * 3)
+    if (ctas(16, 32) <= kSms * 3)
         return append_tiled<4, 1>(a, s);
-    if (ctas(32, 64) <= 152 * 4)
+    if (ctas(32, 64) <= kSms * 4)
         return append_tiled<4, 4>(a, s);
     return append_tiled<8, 4>(a, s);
 }

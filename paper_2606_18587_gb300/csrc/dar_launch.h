@@ -12,6 +12,10 @@
 
 namespace dar {
 
+// SMs of a GB300, where the rules that choose a tile by the number of its CTAs were
+// measured.  (Persistent kernels size their grids by the device's own count.)
+constexpr int kSms = 152;
+
 struct AppendArgs {
     const void *k_new, *v_new;  // [B][Hkv][n][64]
     const float *Dk, *Dv;       // [Hkv][64][dd]

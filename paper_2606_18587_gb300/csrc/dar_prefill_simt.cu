@@ -338,9 +338,9 @@ template <int DD>
 static cudaError_t simt_dd(const PrefillArgs &a, cudaStream_t s)
 {
     const auto ctas = [&](int rows) { return ((long long)a.N + rows - 1) / rows * a.B * a.Hq; };
-    if (ctas(8) <= 152)
+    if (ctas(8) <= kSms)
         return simt_launch<DD, 2>(a, s);
-    return ctas(32) > 152 ? simt_launch<DD, 4>(a, s) : simt_launch<DD, 8>(a, s);
+    return ctas(32) > kSms ? simt_launch<DD, 4>(a, s) : simt_launch<DD, 8>(a, s);
 }
 
 cudaError_t launch_prefill_simt(int dd, const PrefillArgs &a, cudaStream_t s)

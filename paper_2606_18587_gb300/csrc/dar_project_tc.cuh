@@ -13,6 +13,7 @@
 #pragma once
 
 #include "dar_common.cuh"
+#include "dar_launch.h"
 #include "dar_project.cuh"
 #include "dar_sm100.cuh"
 
@@ -164,7 +165,7 @@ __device__ __forceinline__ void project_rows_tc(const bf16 *x, bf16 *out, int os
 __host__ inline int project_tc_rows(long long rows_per_head, long long heads)
 {
     int r = 16 * kTcWarps * 16;
-    while (r > 16 * kTcWarps && (rows_per_head + r - 1) / r * heads < 152 * 8)
+    while (r > 16 * kTcWarps && (rows_per_head + r - 1) / r * heads < kSms * 8)
         r /= 2;
     return r;
 }
