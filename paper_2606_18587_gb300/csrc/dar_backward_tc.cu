@@ -190,7 +190,9 @@ struct Shape {
     // 16-wide global kernels do best with few warps and long independent runs
     // (B8 H16 N8192 w512, us, dq / dk, dv: 1431 / 1345 at 4, 8 and two CTAs per
     // SM; 1461 / 1349 at 2, 2 and four; 1536 / 1378 at 1, 1 and four; at B8 H8
-    // N2047 w128 59 / 51, 69 / 57 and 65 / 58)
+    // N2047 w128 59 / 51, 69 / 57 and 65 / 58).  Wider ones gain little from more
+    // (forward and backward of the larger shape, ms, d_down 32 and 64: 9.12 and 16.5
+    // at 1, 1; 8.85 and 15.9 at 2, 2; 8.82 and 15.8 at 2, 8; 8.78 and 15.6 at 4, 4)
     static constexpr int KSQ = W == 16 ? 4 : 2, UNKV = W == 16 ? 8 : 2;
     // a stage also takes the CTA's own rows, whose A fragments are read before it is needed
     static_assert(ROWS <= BK, "the CTA's tile fits in a stage");

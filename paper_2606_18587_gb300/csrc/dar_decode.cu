@@ -781,7 +781,9 @@ __global__ void __launch_bounds__(kDecThreads, 1)
         // With fewer stages than warps each is a range of its own and the other warps
         // stay idle: cut into as many ranges as warps, a group's few parts would lie
         // among dozens of empty ranges, which its merge had to step over (one sequence
-        // of 101 tokens, 8 heads: 19.7 us, now 9.1).  Very few are spread over the SMs
+        // of 101 tokens, 8 heads: 19.7 us, now 9.1; one of 32768, one KV head, d_down 16,
+        // 259 stages in one group: 106 and 32, with four query heads 385 and 100; d_down
+        // 64, 1024 stages: 113 and 97).  Very few are spread over the SMs
         // (32 stages 9.0 us, side by side 9.5), more stay side by side (8 sequences of
         // 700 to 2000 tokens 11.5, spread 12.4).  The number of ranges goes through warp
         // votes, so that it is uniform to the compiler (64 sequences, 32 heads 118.8 us
