@@ -434,7 +434,12 @@ static cudaError_t cache_append_dd(const AppendArgs &a, const DecodeArgs *d, cud
     const size_t smem = (size_t)app_rows<T>(a.Hkv) * 2 * a.Hkv * kHeadDim * sizeof(T);
     if (d) {
         constexpr int warps = kAppThreads / 32;
-        const int prep = min(2 * kSms, (d->B * d->Hq + warps - 1) / warps);
+        // A row's reads of Uk (one 16-byte word of each of its d_down lines at a time)
+        // keep an SM's L1 busy for about 16 d_down cycles: wide rows go to more blocks
+        // than their warps fill, as long as there are SMs.
+        constexpr int per = DD > 16 ? 256 / DD : warps;
+        const int rows = d->B * d->Hq, full = (rows + warps - 1) / warps;
+        const int prep = min(2 * kSms, max(full, min((rows + per - 1) / per, kSms - a.B)));
         step_front_kernel<T, DD><<<a.B + prep, kAppThreads, smem, s>>>(a, *d);
     } else {
         cache_append_kernel<T, DD><<<a.B, kAppThreads, smem, s>>>(a);

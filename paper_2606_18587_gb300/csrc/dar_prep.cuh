@@ -19,7 +19,7 @@ __device__ __forceinline__ void prep_rows(const DecodeArgs &a, int block, int bl
     constexpr int warps = THREADS / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rows = a.B * a.Hq;
-    for (int row = block * warps + warp; row < rows; row += blocks * warps) {
+    for (int row = warp * blocks + block; row < rows; row += blocks * warps) {  // few rows: spread over the blocks
         if (a.qd) {  // direct variant: the row's own d_down query, rescaled to the local scale
             for (int c = lane; c < DD; c += 32)
                 a.qt[(size_t)row * DD + c] = to_f32(static_cast<const T *>(a.qd)[(size_t)row * DD + c]) * a.qd_ratio;
