@@ -321,14 +321,16 @@ __device__ __forceinline__ void append_tile(const AppendArgs &a, int tiles)
         }
         sm100::cp_async_wait_all();
         __syncthreads();  // every ring row this CTA reads is in shared memory
-        float acc[RPT][CW];
-        project_rows<T, DD, CW, RPT>(rows, Ws + c0, r0, NR, acc);
-        T *pool = static_cast<T *>(kv ? a.pool_vd : a.pool_kd);
+        if (r0 - (tid & 31) < nr) {  // (a warp past the last row has nothing to do)
+            float acc[RPT][CW];
+            project_rows<T, DD, CW, RPT>(rows, Ws + c0, r0, NR, acc);
+            T *pool = static_cast<T *>(kv ? a.pool_vd : a.pool_kd);
 #pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-            const int m = L + j0 + r0 + k * NR - w;
-            if (id[k] >= 0)
-                store_row<T, CW>(pool + (((size_t)id[k] * a.Hkv + g) * kPage + m % kPage) * DD + c0, acc[k]);
+            for (int k = 0; k < RPT; ++k) {
+                const int m = L + j0 + r0 + k * NR - w;
+                if (id[k] >= 0)
+                    store_row<T, CW>(pool + (((size_t)id[k] * a.Hkv + g) * kPage + m % kPage) * DD + c0, acc[k]);
+            }
         }
     }
     // ring slots (L + j) % w, j < min(nb, w): the last new token of each
@@ -481,15 +483,17 @@ static cudaError_t append_bulk_launch(const AppendArgs &a, bool beside_prev, cud
     return cudaLaunchKernelEx(&cfg, append_lens_kernel, a);
 }
 
-// Here big tiles pay once they fill the chip a few times over.
+// Here big tiles pay once they fill the chip a few times over, if their last rows
+// are not mostly past the call's end (64 sequences, 32 heads, d_down 64, n = 9: 199 us
+// with big tiles, 45 with small ones; 512 sequences, 4 heads, d_down 16: 47 and 19).
 constexpr long long kBulkBigCtas = kSms * 6 * 2;
 
 template <typename T, int DD>
 static cudaError_t append_bulk(const AppendArgs &a, bool beside_prev, cudaStream_t s)
 {
     constexpr int R = rows_bulk<T>();
-    const long long big = ((long long)a.n + R - 1) / R * a.B * a.Hkv * 2;
-    if (big >= kBulkBigCtas)
+    const long long tiles = (a.n + R - 1) / R, small = (a.n + kBulkSmallRows - 1) / kBulkSmallRows;
+    if (tiles * a.B * a.Hkv * 2 >= kBulkBigCtas && 4 * tiles * R <= 5 * small * kBulkSmallRows)
         return append_bulk_launch<T, DD, rows_per_thread<DD>(), R / rows_per_thread<DD>()>(a, beside_prev, s);
     return append_bulk_launch<T, DD, 1, kBulkSmallRows>(a, beside_prev, s);
 }
@@ -509,25 +513,36 @@ static cudaError_t append_bulk_t(int dd, const AppendArgs &a, bool beside_prev, 
 // More tokens than one round of the one-CTA-per-sequence kernel: the bulk
 // kernel.  Measured (d_down 16, w 128, context 500), one CTA per sequence / bulk:
 //   n = 8:  B 1, 8 heads 7.8 / 6.2 us; B 32, 12 heads 9.6 / 8.0; B 64, 8 heads 8.2 / 9.3
-//   n = 9:               9.2 / 6.6;                  11.3 / 8.4;                 9.4 / 9.7
-//   n = 64:             37.5 / 8.4;                  48.5 / 10.7;               37.7 / 11.9
-// and at n = 1 the bulk kernel's second launch costs 2 to 4 us.  (A cache with so many heads that not one row of them fits the
-// staging area stays with the kernel that refuses it; so does a call whose CTAs
-// a grid cannot count.)
-constexpr int kBulkMinTokens = kAppRows + 1;
+//   n = 9:               9.0 / 6.6;                                             9.5 / 8.7
+//   n = 64:             38.0 / 8.5;                                            38.3 / 11.9
+// and at n = 1 the bulk kernel's second launch costs 2 to 4 us.  It takes a CTA per
+// (sequence, head, tensor) however few the tokens, so with many of those the other
+// kernel keeps the calls of up to 32 tokens that it does faster: it costs about
+// 0.6 us per token, 512 chains and wave of sequences, the bulk kernel 1.2 + 0.15
+// d_down ns per CTA.  Measured, one CTA per sequence / bulk at n = 9, 16 and 24:
+//   B 128, 16 heads, d_down 32:  19 / 32, 27 / 32, 37 / 33;   B 256, 8, 16:  18 / 19, 24 / 19, 32 / 20
+//   B 256, 16 heads, d_down 64:  55 / 82, 83 / 83, 122 / 84;  B 152, 8, 32:  12 / 20, 16 / 20, 21 / 21
+//   B 512, 16 heads, d_down 16:  47 / 62, 74 / 62, 113 / 65;  B 512, 4, 16:  26 / 19, 32 / 19, 45 / 20
+//   B 64, 32 heads, d_down 64:   50 / 45, 77 / 46, 110 / 46;  B 512, 8, 8:   30 / 23, 40 / 23, 52 / 24
+// (A cache with so many heads that not one row of them fits the staging area stays
+// with the kernel that refuses it; so does a call whose CTAs a grid cannot count.)
+constexpr int kBulkMinTokens = kAppRows + 1, kBulkAlwaysTokens = 33;
 
-static bool use_bulk(dar_dtype dt, const AppendArgs &a)
+static bool use_bulk(dar_dtype dt, int dd, const AppendArgs &a)
 {
     const long long row = 2ll * a.Hkv * kHeadDim * (dt == DAR_F32 ? 4 : 2);
     const long long tiles = ((long long)a.n + kBulkSmallRows - 1) / kBulkSmallRows;
-    return a.n >= kBulkMinTokens && row <= kAppStageBytes && tiles * a.B * a.Hkv <= 0x7fffffffLL;
+    if (a.n < kBulkMinTokens || row > kAppStageBytes || tiles * a.B * a.Hkv > 0x7fffffffLL)
+        return false;
+    const long long groups = (2ll * a.Hkv * dd + kAppThreads - 1) / kAppThreads, waves = (a.B + kSms - 1) / kSms;
+    return a.n >= kBulkAlwaysTokens || 2ll * a.B * a.Hkv * (8 + dd) < 4000ll * a.n * groups * waves;
 }
 
 cudaError_t launch_cache_append(dar_dtype dt, int dd, const AppendArgs &a, cudaStream_t s, bool beside_prev)
 {
     if (a.B == 0)
         return cudaSuccess;
-    if (use_bulk(dt, a))
+    if (use_bulk(dt, dd, a))
         return dt == DAR_F32 ? append_bulk_t<float>(dd, a, beside_prev, s) : append_bulk_t<bf16>(dd, a, beside_prev, s);
     return dt == DAR_F32 ? cache_append_t<float>(dd, a, nullptr, s) : cache_append_t<bf16>(dd, a, nullptr, s);
 }
@@ -535,7 +550,7 @@ cudaError_t launch_cache_append(dar_dtype dt, int dd, const AppendArgs &a, cudaS
 cudaError_t launch_step_front(dar_dtype dt, int dd, const AppendArgs &a, const DecodeArgs &d, cudaStream_t s,
                               bool *done)
 {
-    *done = !use_bulk(dt, a);
+    *done = !use_bulk(dt, dd, a);
     if (!*done)
         return launch_cache_append(dt, dd, a, s);
     return dt == DAR_F32 ? cache_append_t<float>(dd, a, &d, s) : cache_append_t<bf16>(dd, a, &d, s);

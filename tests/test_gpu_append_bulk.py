@@ -1,7 +1,7 @@
 """The bulk cache append (many tokens per sequence in one call) leaves the same
 bytes as appends of a few tokens each, which the one-CTA-per-sequence kernel
 takes: tile edges, calls shorter and longer than the window, a context that
-ends inside the window or past it, both tile sizes, and refused sequences."""
+ends inside the window or past it, many tiles, and refused sequences."""
 import numpy as np
 import pytest
 
@@ -37,7 +37,7 @@ def same(a, b):
     (3, 2, 32, 100, 65, [0, 35, 36]),       # one row past a tile; the window fills inside the call
     (2, 2, 64, 1, 129, [0, 200]),           # window of one token
     (2, 1, 16, 300, 130, [10, 500]),        # call shorter than the window
-    (40, 12, 16, 33, 300, [0, 1, 40, 500]),  # enough tiles for several rows per thread
+    (40, 12, 16, 33, 300, [0, 1, 40, 500]),  # many tiles, the last ones mostly empty
     (40, 12, 64, 400, 300, [7, 399]),
 ])
 def test_bulk_equals_few_at_a_time(dtype, B, Hkv, dd, w, n, before):
