@@ -712,11 +712,17 @@ __global__ void __launch_bounds__(MainLayout<DL, MT>::THREADS, 2)
         auto first = [&](long long c) {  // the first item that starts at c or later
             return (int)(c <= lat ? (c + cu - 1) / cu : n_lat + (c - lat + cw - 1) / cw);
         };
-        // (few items: one CTA per SM, the first half of the grid)
-        const int ctas = n_lat + B * a.Hkv <= (int)gridDim.x / 2 ? gridDim.x / 2 : gridDim.x;
-        const long long share = (total + ctas - 1) / ctas;
-        k0 = first(min(total, share * blockIdx.x));
-        k1 = first(min(total, share * (blockIdx.x + 1)));
+        // No more items than CTAs: one each (us, shares of the cost / one each: 3 sequences
+        // of 2128 to 5765 tokens, 16 KV heads, d_lat 256, w 950 22.1 / 18.8; 20 of 100 to
+        // 800, 8, 192, 64 20.7 / 17.7; 30 of 100 to 500, 8, 128, 40 16.8 / 15.8).
+        if (const int items = n_lat + B * a.Hkv; items <= (int)gridDim.x) {
+            k0 = min(items, (int)blockIdx.x);
+            k1 = min(items, k0 + 1);
+        } else {
+            const long long share = (total + gridDim.x - 1) / gridDim.x;
+            k0 = first(min(total, share * blockIdx.x));
+            k1 = first(min(total, share * (blockIdx.x + 1)));
+        }
     }
     auto segment_of = [&](int k) {
         Segment it;
