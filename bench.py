@@ -43,9 +43,9 @@ METRIC = "decode GB/s & prefill TFLOP/s of DAR attention, % of GB300 roofline (1
 LAUNCHES_PER_STEP = 2
 # DRAM bytes (read + write) of one decode_kernel<bf16,16,1> launch on the
 # decode-160M workload, from an ncu capture of `python bench.py --only decode`
-# (dram__bytes_read.sum + dram__bytes_write.sum); None whenever that kernel
-# has changed since the capture.
-DECODE_TRAFFIC_BYTES = 112_347_648 + 2_752_512
+# (dram__bytes_read.sum + dram__bytes_write.sum, profiles/decode_kernel_decode160m.md);
+# None whenever that kernel has changed since the capture.
+DECODE_TRAFFIC_BYTES = 112_350_976 + 3_337_984
 # ex2 results per clock per SM on the multi-function unit, measured on GB300
 # with a throughput probe (f32 and packed bf16x2 alike), and the maximum SM
 # clock: the prefill's exponential roofline

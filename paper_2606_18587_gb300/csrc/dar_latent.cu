@@ -411,8 +411,8 @@ constexpr int kConsumerThreads = 128;  // warps 0-3: tensor-core work
 // sequences of 1024 to 8192 tokens, 32 heads, d_lat 256; 72 with the warp; at 8
 // heads, d_lat 128, 26 with the warp, 29 without).  Measured, prep to merge,
 // against round-robin items with a record per unit and the rows read from shared
-// memory: those 64 sequences 88 -> 62 us; 32 sequences of 4096, 12 heads, d_lat
-// 192 28 -> 25; one sequence of 8192, 32 heads, d_lat 256 22 -> 18.
+// memory: those 64 sequences 88 -> 64 us; 32 sequences of 4096, 12 heads, d_lat
+// 192 28 -> 22; one sequence of 8192, 32 heads, d_lat 256 22 -> 18.
 template <int DL, int MT>
 struct MainLayout {
     static constexpr bool kProducer = !(DL == 256 && MT == 2);
