@@ -435,7 +435,7 @@ struct Segment {
     int npg;      // pages / tiles
 };
 
-constexpr float kMaxDrop = 64.f;  // log2 units
+constexpr float kMaxDrop = 16.f;  // log2 units: a unit further below weighs less than the rounding of the others
 
 __device__ __forceinline__ void consumer_sync()
 {
