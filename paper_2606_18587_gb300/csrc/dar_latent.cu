@@ -1080,11 +1080,12 @@ static cudaError_t decode_t(const Args &a, const void *pool_c, const void *win_k
     // prep and merge: few rows are spread over the chip, many share a staged
     // matrix (4 sequences, 4 KV heads, G 4: 16.5 us with 2 rows a block, 17.7 with
     // 8; 64 sequences, 8 KV heads, G 4: 4 rows a block cost 3 us more than 8).  The
-    // merge takes two blocks per SM before rows share one, the prep, beside which the
+    // merge takes two blocks per SM before rows share one, except at d_lat 64, where
+    // its small blocks find room beside the main kernel's; the prep, beside which the
     // main kernel has to start, one (calls, us, merge at one / two blocks per SM, then
     // both at two: 32 sequences of 4096 tokens, 12 heads, d_lat 192 24.5 / 21.9 / 21.9;
     // 61 of 340 to 484, 12, 256 23.6 / 22.4 / 22.7; 10 of 4000 to 8000, 32, 256 40.4 /
-    // 38.2 / 40.5; 64 of 300 to 900, 8, 64 11.7 / 12.8 / 12.4).
+    // 38.2 / 40.5; 64 of 300 to 900, 8, 64 11.7 / 12.8 / 12.4; 64 of 16384, 8, 64 47 / 51).
     const auto rows_for = [&](int blocks) {
         int rows = 2;
         while (rows < kRowsPerBlock && a.Hkv * ((a.B * a.G + rows - 1) / rows) > blocks)
@@ -1106,7 +1107,7 @@ static cudaError_t decode_t(const Args &a, const void *pool_c, const void *win_k
     e = cudaLaunchKernelEx(&cfg, latent_main_kernel<DL, MT>, tm[0], tm[1], tm[2], a);
     if (e != cudaSuccess)
         return e;
-    rows = rows_for(2 * sms);
+    rows = rows_for(DL > 64 ? 2 * sms : sms);
     cfg.gridDim = dim3(a.Hkv, (a.B * a.G + rows - 1) / rows);
     cfg.blockDim = dim3(32 * rows);
     cfg.dynamicSmemBytes = merge_smem;
